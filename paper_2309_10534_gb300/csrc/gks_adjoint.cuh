@@ -99,6 +99,107 @@ GKS_HD void teno_gauss_T(const TenoSel<T>& S, T g, T gv, T gd, T* gq)
 }
 
 // ------------------------------------------------------------------ kinetic layer (2-D)
+// Moment matrix H^(k,m)_ab = <u^k v^m psi_a psi_b>, psi = (1, u, v, (u^2+v^2+xi^2)/2),
+// of a unit-mass Maxwellian from its moment tables; 10 unique entries
+// (H00 H01 H02 H03 H11 H12 H13 H22 H23 H33).  <u^k v^m (a.psi) psi> = H a.
+// 1-D: v == 0, so only m = 0 occurs and the v entries vanish.
+template <int k, int m, typename T, int DIM>
+GKS_HD void hmat(const T* u, const T* v, T xi2, T xi4, T* H)
+{
+    if constexpr (DIM == 2) {
+        H[0] = u[k] * v[m];
+        H[1] = u[k + 1] * v[m];
+        H[2] = u[k] * v[m + 1];
+        H[4] = u[k + 2] * v[m];
+        H[5] = u[k + 1] * v[m + 1];
+        H[7] = u[k] * v[m + 2];
+        H[3] = T(0.5) * (H[4] + H[7] + H[0] * xi2);
+        H[6] = T(0.5) * (u[k + 3] * v[m] + u[k + 1] * v[m + 2] + H[1] * xi2);
+        H[8] = T(0.5) * (u[k + 2] * v[m + 1] + u[k] * v[m + 3] + H[2] * xi2);
+        H[9] = T(0.25) * (u[k + 4] * v[m] + u[k] * v[m + 4] + H[0] * xi4
+                          + T(2) * (u[k + 2] * v[m + 2] + (H[4] + H[7]) * xi2));
+    } else {
+        static_assert(m == 0, "1-D has no v moments");
+        H[0] = u[k];
+        H[1] = u[k + 1];
+        H[4] = u[k + 2];
+        H[3] = T(0.5) * (H[4] + H[0] * xi2);
+        H[6] = T(0.5) * (u[k + 3] + H[1] * xi2);
+        H[9] = T(0.25) * (u[k + 4] + H[0] * xi4 + T(2) * H[4] * xi2);
+        H[2] = H[5] = H[7] = H[8] = T(0);
+    }
+}
+
+// o = H a for the symmetric moment matrix of hmat
+template <typename T, int DIM>
+GKS_HD void hmv(const T* H, const T* a, T* o)
+{
+    if constexpr (DIM == 2) {
+        o[0] = H[0] * a[0] + H[1] * a[1] + H[2] * a[2] + H[3] * a[3];
+        o[1] = H[1] * a[0] + H[4] * a[1] + H[5] * a[2] + H[6] * a[3];
+        o[2] = H[2] * a[0] + H[5] * a[1] + H[7] * a[2] + H[8] * a[3];
+        o[3] = H[3] * a[0] + H[6] * a[1] + H[8] * a[2] + H[9] * a[3];
+    } else {
+        o[0] = H[0] * a[0] + H[1] * a[1] + H[3] * a[3];
+        o[1] = H[1] * a[0] + H[4] * a[1] + H[6] * a[3];
+        o[2] = T(0);
+        o[3] = H[3] * a[0] + H[6] * a[1] + H[9] * a[3];
+    }
+}
+
+// Jacobian-vector products of the Euler fluxes.  For the micro slope a of a
+// state derivative dW (<a psi> rho = dW), chain rule through the Maxwellian
+// gives rho <u (a.psi) psi> = (dF/dW) dW and rho <v (a.psi) psi> = (dG/dW) dW,
+// with F, G the normal and tangential Euler fluxes of an ideal gas whose
+// gamma matches K.  h = (E + p)/rho.
+template <typename T, int DIM>
+GKS_HD void euler_jvp(const T* dW, T U, T V, T h, T gm1, T* dF, T* dG)
+{
+    const T q = T(0.5) * (U * U + V * V);
+    if constexpr (DIM == 2) {
+        const T dp = gm1 * (dW[3] - U * dW[1] - V * dW[2] + q * dW[0]);
+        const T cross = V * dW[1] + U * dW[2] - U * V * dW[0];
+        if (dF) {
+            dF[0] = dW[1];
+            dF[1] = T(2) * U * dW[1] - U * U * dW[0] + dp;
+            dF[2] = cross;
+            dF[3] = U * (dW[3] + dp) + h * (dW[1] - U * dW[0]);
+        }
+        if (dG) {
+            dG[0] = dW[2];
+            dG[1] = cross;
+            dG[2] = T(2) * V * dW[2] - V * V * dW[0] + dp;
+            dG[3] = V * (dW[3] + dp) + h * (dW[2] - V * dW[0]);
+        }
+    } else {
+        const T dp = gm1 * (dW[3] - U * dW[1] + q * dW[0]);
+        if (dF) {
+            dF[0] = dW[1];
+            dF[1] = T(2) * U * dW[1] - U * U * dW[0] + dp;
+            dF[2] = T(0);
+            dF[3] = U * (dW[3] + dp) + h * (dW[1] - U * dW[0]);
+        }
+        if (dG) dG[0] = dG[1] = dG[2] = dG[3] = T(0);
+    }
+}
+
+// Micro slope: <a psi> = b with the full-space moments of a Maxwellian
+// (Eq. 2.7), solved in closed form.  ntot = K + DIM degrees of freedom
+// besides... (all translational + internal); inv2l = 1/(2 lambda).
+template <typename T, int DIM>
+GKS_HD void micro_slope(const T* b, T U, T V, T lam, T inv2l, T ntot, T inv_ntot, T* a)
+{
+    const T E = T(0.5) * (U * U + V * V + ntot * inv2l);
+    const T R2 = b[1] - U * b[0];
+    const T R3 = (DIM == 2) ? b[2] - V * b[0] : T(0);
+    const T R4 = T(2) * (b[3] - E * b[0]);
+    const T tl = T(2) * lam;
+    a[3] = tl * tl * inv_ntot * (R4 - T(2) * U * R2 - T(2) * V * R3);
+    a[2] = (DIM == 2) ? tl * R3 - V * a[3] : T(0);
+    a[1] = tl * R2 - U * a[3];
+    a[0] = b[0] - U * a[1] - V * a[2] - E * a[3];
+}
+
 // euler_jvp's dF = (dF/dW)(U, V, h) d: adds (dF/dW)^T y to gd and the
 // derivatives with respect to U, V, h to gU, gV, gh
 template <typename T>
@@ -441,8 +542,8 @@ GKS_HD void point_flux_vjp(const Side<T>& L, const Side<T>& R, const FluxParams<
 {
     T W0[4] = {T(0), T(0), T(0), T(0)}, W0n[4] = {T(0), T(0), T(0), T(0)}, W0t[4] = {T(0), T(0), T(0), T(0)};
     T d4[4], d5[4], d6[4], d7[4], d8[4], pl, pr;
-    side_terms<T, 2, false, false>(L, true, P, W0, W0n, W0t, d4, d5, d6, d7, d8, pl);
-    side_terms<T, 2, false, false>(R, false, P, W0, W0n, W0t, d4, d5, d6, d7, d8, pr);
+    side_terms<true, T, 2, false, false>(L, P, W0, W0n, W0t, d4, d5, d6, d7, d8, pl);
+    side_terms<false, T, 2, false, false>(R, P, W0, W0n, W0t, d4, d5, d6, d7, d8, pr);
     T gW0[4] = {T(0), T(0), T(0), T(0)}, gW0n[4] = {T(0), T(0), T(0), T(0)}, gW0t[4] = {T(0), T(0), T(0), T(0)};
     equilibrium_vjp(W0, W0n, W0t, P.gm1, gF, gdF, gW0, gW0n, gW0t);
     side_vjp(L, true, P, gW0, gW0n, gW0t, gL);

@@ -11,7 +11,7 @@ template <typename T>
 int time_coeffs_t(double s, double* cF, double* cD)
 {
     T f[6], d[6];
-    gks::time_coeffs<T>((T)s, f, d);
+    gks::time_coeffs<T>((T)s, T(1) / (T)s, f, d);
     for (int k = 0; k < 6; ++k) { cF[k] = (double)f[k]; cD[k] = (double)d[k]; }
     return 0;
 }
@@ -76,6 +76,8 @@ int flux_t(int tau_mode, double gamma, double mu, double Pr, double c1, double c
     p.c2 = (T)c2;
     p.mu = (T)mu;
     p.prfac = (T)(1.0 / Pr - 1.0);
+    p.hkv = (T)(0.5 * (K + DIM - 1.0));
+    p.cp = (T)(0.5 * (K + DIM + 2.0));
     p.tau_mode = tau_mode;
     gks::Side<T> L, R;
     for (int k = 0; k < 4; ++k) {
@@ -127,6 +129,8 @@ int flux_vjp_t(double gamma, const double* Wl, const double* Wln, const double* 
     p.K = (T)K;
     p.ntot = (T)(K + 2.0);
     p.inv_ntot = (T)(1.0 / (K + 2.0));
+    p.hkv = (T)(0.5 * (K + 1.0));
+    p.cp = (T)(0.5 * (K + 4.0));
     p.tau_mode = 0;
     gks::Side<T> L, R, gL, gR;
     T f[4], d[4];

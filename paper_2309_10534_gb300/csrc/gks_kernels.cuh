@@ -333,9 +333,9 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(GridDev g, Stage1DArgs a, Fl
             for (int v = 0; v < 3; ++v)
                 w0n[slot[v]] = (T(1.25) * (sq[v][f + 3] - sq[v][f + 2]) - T(1.0 / 12.0) * (sq[v][f + 4] - sq[v][f + 1]))
                              * idx_;
-            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, w0n);
+            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, w0n);
         } else {
-            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF);
+            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1);
         }
         const T tdt = s_scal[0];
 #pragma unroll
@@ -689,27 +689,33 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
                 // a non-physical linear state (the quartic across a
                 // discontinuity) falls back to the kinetic merge at the point
                 if (physical<T, 2>(w0g, fp.gm1)) {
-                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, w0n, w0g, w0t);
+                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, w0n, w0g, w0t);
                 } else {
                     ++nfb;
-                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF);
+                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1);
                 }
             } else {
-                point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF);
+                point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1);
             }
         }
+        // the stage's combinations at both points, averaged (weights 1/2): each
+        // lane finishes half of the face's values, one shuffle per value
+        // stage 1: lane 0 the four W* combinations, lane 1 the accumulator's;
+        // stage 2: variables 2 gpi and 2 gpi + 1
+        T g0[4], g1[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            F[v] = T(0.5) * (F[v] + __shfl_xor_sync(0xffffffffu, F[v], 1));
-            dF[v] = T(0.5) * (dF[v] + __shfl_xor_sync(0xffffffffu, dF[v], 1));
-        }
-        if (gpi == 0) {
+        for (int v = 0; v < 4; ++v) stage_comb<T>(a.stage, F[v], dF[v], tdt, g0[v], g1[v]);
+        if (a.stage == 1) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                T g0, g1;
-                stage_comb<T>(a.stage, F[v], dF[v], tdt, g0, g1);
-                sF[sfi(v, r, f)] = g0;
-                if (a.stage == 1) sF[sfi(4 + v, r, f)] = g1;
+                const T got = __shfl_xor_sync(0xffffffffu, gpi ? g0[v] : g1[v], 1);
+                sF[sfi(4 * gpi + v, r, f)] = T(0.5) * ((gpi ? g1[v] : g0[v]) + got);
+            }
+        } else {
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const T got = __shfl_xor_sync(0xffffffffu, gpi ? g0[v] : g0[v + 2], 1);
+                sF[sfi(2 * gpi + v, r, f)] = T(0.5) * ((gpi ? g0[v + 2] : g0[v]) + got);
             }
         }
     }

@@ -56,6 +56,8 @@ inline FluxParams<T> make_flux_params(const HostFlux& h)
     p.c2 = (T)h.c2;
     p.mu = (T)h.mu;
     p.prfac = (T)h.prfac;
+    p.hkv = (T)(0.5 * (h.ntot - 1.0));
+    p.cp = (T)(0.5 * (h.ntot + 2.0));
     p.tau_mode = h.tau_mode;
     p.merge = h.merge;
     return p;

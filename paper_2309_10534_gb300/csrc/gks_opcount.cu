@@ -58,6 +58,7 @@ template <typename B> struct M<opc::Cnt<B>> {
     static C erfc_(C x) { opc::g_cnt.erfc += 1; return C(std::erfc((double)x.v)); }
     static C exp_(C x) { opc::g_cnt.exp += 1; return C(std::exp((double)x.v)); }
     static C sqrt_(C x) { opc::g_cnt.sqrt += 1; return C(std::sqrt((double)x.v)); }
+    static C rsqrt_(C x) { opc::g_cnt.sqrt += 1; opc::g_cnt.div += 1; return C(1.0 / std::sqrt((double)x.v)); }
     static C rcp(C x) { opc::g_cnt.div += 1; return C(1.0 / (double)x.v); }
     static constexpr double tiny = M<B>::tiny;
     static constexpr int nseries = M<B>::nseries;
@@ -106,6 +107,8 @@ void count(int tau_mode, double Pr, gks_flop_model* out)
     fp.c2 = T(1.0);
     fp.mu = T(tau_mode == 2 ? 1e-4 : 0.0);
     fp.prfac = T(1.0 / Pr - 1.0);
+    fp.hkv = T(0.5 * (K + DIM - 1.0));
+    fp.cp = T(0.5 * (K + DIM + 2.0));
     fp.tau_mode = tau_mode;
     const TenoParams tp0{1e-40, 7, 1e-7, 1e-5};
     TenoT<T> tp;
