@@ -109,21 +109,23 @@ inline TenoT<T> teno_t(const TenoParams& P)
     return t;
 }
 
-// Result of the TENO-D selection on one 5-cell stencil: either the large
-// stencil, or the equal-weight (d_k = 1/3) average of the kept sub-stencils.
+// Result of a reconstruction's selection on one 5-cell stencil.  TENO-D:
+// either the large stencil, or the equal-weight (d_k = 1/3) average of the
+// kept sub-stencils, on the first differences of the cells.  WENO5-AO,
+// WENO5-Z, TENO5: the candidates' coefficients and weights.
 template <typename T> struct TenoSel {
     T q2;               // centre cell average
-    T b[3], c[3];       // quadratic k: p = q2 - c/12 + b xi + c xi^2
-    T u1, u2, u3, u4;   // quartic in the Legendre-type basis
+    // TENO-D: with e_i = q_i - q_(i-1), A = e2 + e3, B = e1 + e4, C = e3 - e2,
+    // D = e4 - e1: twice the quadratics' coefficients (2 b_k = B0, A, B2;
+    // 2 c_k = C0, C, C2) and the quartic's combinations P = 7 A - B, R = D - 3 C
+    T A, B, C, D, B0, B2, C0, C2, P, R;
+    T b[3], c[3];       // others: quadratic k: p = q2 - c/12 + b xi + c xi^2
+    T u1, u2, u3, u4;   // others: quartic in the Legendre-type basis
     T w[3];             // sub-stencil weights (0 when the large stencil is used)
     T w3;               // WENO5-AO: weight of the quartic (TENO-D: unused)
     bool large;
 };
 
-// beta_k of Eq. (3.7): quadratics b^2 + 13/3 c^2; the quartic in Balsara's
-// Legendre form.  Selection of Eqs. (4.5)-(4.7) and (4.11)-(4.12) on powers
-// normalised by the smallest beta + eps (below), without divisions and
-// without (beta+eps)^-q, which would overflow in float32.
 // the sub-stencil quadratics and the large-stencil quartic (Sec. 3.1),
 // formed from the sums and differences of the cells at equal distance from
 // the centre (the quartic's odd coefficients only see the differences, its
@@ -147,17 +149,45 @@ GKS_HD void stencil_coeffs(const T q[5], TenoSel<T>& S)
     S.u4 = T(1.0 / 24.0) * s0 + (T(0.25) * q2 - T(1.0 / 6.0) * s1);          // (q0 - 4 q1 + 6 q2 - 4 q3 + q4) / 24
 }
 
-// smoothness indicators t_k = beta_k + eps of Eq. (3.7) (quadratics
-// b^2 + 13/3 c^2; the quartic in Balsara's Legendre form), each a chain of
-// fused multiply-adds onto eps
+// TENO-D works on first differences e_i: every sub-stencil coefficient is a
+// combination of two of them and the quartic's of A, B (odd) or C, D (even),
+// and every reconstructed value is q2 plus such combinations.  Against the
+// coefficients formed from the cell averages this takes 14 instead of 26
+// operations and no large common part cancels; the indicators, faces and
+// Gauss points share P and R.  Measured: one step of a 1024^2 float32 plane
+// 0.844 -> 0.810 ms, of a 400^2 float64 plane 5.77 -> 5.12 ms.
 template <typename T>
-GKS_HD void teno_indicators(const TenoSel<T>& S, T eps, T* t)
+GKS_HD void teno_differences(const T q[5], TenoSel<T>& S)
 {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) t[k] = S.b[k] * S.b[k] + (T(13.0 / 3.0) * S.c[k] * S.c[k] + eps);
-    const T a = S.u1 + T(0.1) * S.u3, bq = S.u2 + T(123.0 / 455.0) * S.u4;
-    t[3] = a * a + (T(13.0 / 3.0) * bq * bq + (T(781.0 / 20.0) * S.u3 * S.u3
-                                              + (T(1421461.0 / 2275.0) * S.u4 * S.u4 + eps)));
+    const T e1 = q[1] - q[0], e2 = q[2] - q[1], e3 = q[3] - q[2], e4 = q[4] - q[3];
+    S.q2 = q[2];
+    S.A = e2 + e3;
+    S.B = e1 + e4;
+    S.C = e3 - e2;
+    S.D = e4 - e1;
+    S.B0 = T(3) * e2 - e1;  // q0 - 4 q1 + 3 q2
+    S.C0 = e2 - e1;         // q0 - 2 q1 + q2
+    S.B2 = T(3) * e3 - e4;  // -3 q2 + 4 q3 - q4
+    S.C2 = e4 - e3;         // q2 - 2 q3 + q4
+    S.P = T(7) * S.A - S.B;
+    S.R = S.D - T(3) * S.C;
+}
+
+// smoothness indicators t_k = 4 (beta_k + eps) of Eq. (3.7): quadratics
+// b^2 + 13/3 c^2; the quartic in Balsara's Legendre form, whose four squares
+// are u1 + u3/10 = P/12, u2 + 123/455 u4 = (163 C - 11 D)/260,
+// u3 = (B - A)/12 and u4 = R/24.  eps4 = 4 eps.
+template <typename T>
+GKS_HD void teno_indicators(const TenoSel<T>& S, T eps4, T* t)
+{
+    const T k = T(13.0 / 3.0);
+    t[0] = S.B0 * S.B0 + (k * S.C0 * S.C0 + eps4);
+    t[1] = S.A * S.A + (k * S.C * S.C + eps4);
+    t[2] = S.B2 * S.B2 + (k * S.C2 * S.C2 + eps4);
+    const T u3 = S.B - S.A, bq = S.C - T(11.0 / 163.0) * S.D;
+    t[3] = T(1.0 / 36.0) * S.P * S.P
+         + (T(13.0 / 3.0 * (163.0 / 130.0) * (163.0 / 130.0)) * bq * bq
+            + (T(781.0 / 720.0) * u3 * u3 + (T(1421461.0 / 327600.0) * S.R * S.R + eps4)));
 }
 
 // WENO5-AO (Sec. 3.2): beta by Eq. (3.7), global indicator
@@ -193,16 +223,16 @@ GKS_HD void ao_select(const T q[5], const TenoT<T>& P, TenoSel<T>& S)
     S.large = false;
 }
 
+// Selection of Eqs. (4.5)-(4.7) and (4.11)-(4.12) as 4 bits: bit 0 the large
+// stencil, bits 1-3 the kept sub-stencils.
+// chi_k = t_k^-q / sum_j t_j^-q.  With m = min_j t_j and r_j = m / t_j in
+// (0, 1], chi_k = r_k^q / sum_j r_j^q: nothing overflows, and an r^q that
+// underflows belongs to a chi far below any cut-off.  The same powers serve
+// both selections (the second normalises over k = 0..2 only, where d_k = 1/3
+// cancels).
 template <typename T>
-GKS_HD void teno_select(const T q[5], const TenoT<T>& P, TenoSel<T>& S)
+GKS_HD unsigned teno_code(const T t[4], T ct1, T ct2, int q)
 {
-    stencil_coeffs(q, S);
-    T t[4];
-    teno_indicators(S, P.eps, t);
-    // chi_k = t_k^-q / sum_j t_j^-q.  With m = min_j t_j and r_j = m / t_j in
-    // (0, 1], chi_k = r_k^q / sum_j r_j^q: nothing overflows, and an r^q that
-    // underflows belongs to a chi far below any cut-off.  The same powers
-    // serve both selections (the second normalises over k = 0..2 only).
     T m = t[0] < t[1] ? t[0] : t[1];
     m = m < t[2] ? m : t[2];
     m = m < t[3] ? m : t[3];
@@ -210,85 +240,80 @@ GKS_HD void teno_select(const T q[5], const TenoT<T>& P, TenoSel<T>& S)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const T r = m * (T(1) / t[j]);
-        if (P.q == 7) {
+        if (q == 7) {
             const T r2 = r * r, r3 = r2 * r;
             p[j] = r3 * r3 * r;
         } else {
-            p[j] = ipow(r, P.q);
+            p[j] = ipow(r, q);
         }
     }
     const T s012 = p[0] + p[1] + p[2];
     // first selection (Eqs. 4.6, 4.7): keep the large stencil when chi_{3,1} >= C_T1
-    S.large = (p[3] >= P.ct1 * (s012 + p[3]));
-    if (S.large) {
-        S.w[0] = S.w[1] = S.w[2] = T(0);
-        return;
-    }
-    // second selection among the small stencils (Eqs. 4.11, 4.12), d_k = 1/3 cancels
-    T d[3], dsum = T(0);
-    const T thr = P.ct2 * s012;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        d[k] = (p[k] >= thr) ? T(1) : T(0);
-        dsum += d[k];
-    }
-    const T inv = T(1) / dsum;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) S.w[k] = d[k] * inv;
+    if (p[3] >= ct1 * (s012 + p[3])) return 1u;
+    // second selection among the small stencils (Eqs. 4.11, 4.12)
+    const T thr = ct2 * s012;
+    return (p[0] >= thr ? 2u : 0u) | (p[1] >= thr ? 4u : 0u) | (p[2] >= thr ? 8u : 0u);
 }
 
-// values and xi-derivatives at the faces xi = +1/2 (vp, dp) and -1/2 (vm, dm)
+// TENO-D (Sec. 4.2) of one stencil: differences, selection, weights
+template <typename T>
+GKS_HD void teno_select(const T q[5], const TenoT<T>& P, TenoSel<T>& S)
+{
+    teno_differences(q, S);
+    T t[4];
+    teno_indicators(S, T(4) * P.eps, t);
+    const unsigned code = teno_code(t, P.ct1, P.ct2, P.q);
+    S.large = (code & 1u) != 0;
+    const int n = ((code >> 1) & 1u) + ((code >> 2) & 1u) + ((code >> 3) & 1u);
+    const T inv = n == 1 ? T(1) : (n == 2 ? T(0.5) : T(1.0 / 3.0));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) S.w[k] = (code & (2u << k)) ? inv : T(0);
+}
+
+// 2 sum w_k b_k and 2 sum w_k c_k of the kept sub-stencils
+template <typename T>
+GKS_HD void teno_small(const TenoSel<T>& S, T& sb, T& sc)
+{
+    sb = S.w[0] * S.B0 + S.w[1] * S.A + S.w[2] * S.B2;
+    sc = S.w[0] * S.C0 + S.w[1] * S.C + S.w[2] * S.C2;
+}
+
+// values and xi-derivatives at the faces xi = +1/2 (vp, dp) and -1/2 (vm, dm):
+// each value even +- odd.  Large stencil: Eqs. (4.8), (4.9) and their mirror;
+// sub-stencils: Eqs. (4.13), (4.14), p_k(+-1/2) = q2 +- b/2 + c/6,
+// p_k'(+-1/2) = b +- c
 template <typename T>
 GKS_HD void teno_faces(const T q[5], const TenoSel<T>& S, T& vp, T& dp, T& vm, T& dm)
 {
-    if (S.large) {  // Eqs. (4.8), (4.9) and their mirror at x_{i-1/2}
-        vp = (T(2) * q[0] - T(13) * q[1] + T(47) * q[2] + T(27) * q[3] - T(3) * q[4]) * T(1.0 / 60.0);
-        dp = (q[1] - T(15) * q[2] + T(15) * q[3] - q[4]) * T(1.0 / 12.0);
-        vm = (T(-3) * q[0] + T(27) * q[1] + T(47) * q[2] - T(13) * q[3] + T(2) * q[4]) * T(1.0 / 60.0);
-        dm = (q[0] - T(15) * q[1] + T(15) * q[2] - q[3]) * T(1.0 / 12.0);
-        return;
+    T even, odd, de, dod;
+    if (S.large) {
+        even = S.q2 + T(1.0 / 120.0) * (T(13) * S.C - S.D);
+        odd = T(1.0 / 24.0) * S.P;
+        de = T(1.0 / 24.0) * (T(13) * S.A - S.B);
+        dod = T(1.0 / 24.0) * (T(15) * S.C - S.D);
+    } else {
+        T sb, sc;
+        teno_small(S, sb, sc);
+        even = S.q2 + T(1.0 / 12.0) * sc;
+        odd = T(0.25) * sb;
+        de = T(0.5) * sb;
+        dod = T(0.5) * sc;
     }
-    // Eqs. (4.13), (4.14): p_k(+-1/2) = q2 +- b/2 + c/6, p_k'(+-1/2) = b +- c
-    vp = dp = vm = dm = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        T w = S.w[k], bh = T(0.5) * S.b[k], c6 = S.c[k] * T(1.0 / 6.0);
-        vp += w * (bh + c6);
-        vm += w * (c6 - bh);
-        dp += w * (S.b[k] + S.c[k]);
-        dm += w * (S.b[k] - S.c[k]);
-    }
-    vp += S.q2;
-    vm += S.q2;
+    vp = even + odd;
+    vm = even - odd;
+    dp = de + dod;
+    dm = de - dod;
+    (void)q;
 }
 
 // one face of teno_faces: value and xi-derivative at xi = +1/2 (PLUS) or -1/2
 template <bool PLUS, typename T>
 GKS_HD void teno_face(const T q[5], const TenoSel<T>& S, T& v, T& d)
 {
-    if (S.large) {
-        if (PLUS) {
-            v = (T(2) * q[0] - T(13) * q[1] + T(47) * q[2] + T(27) * q[3] - T(3) * q[4]) * T(1.0 / 60.0);
-            d = (q[1] - T(15) * q[2] + T(15) * q[3] - q[4]) * T(1.0 / 12.0);
-        } else {
-            v = (T(-3) * q[0] + T(27) * q[1] + T(47) * q[2] - T(13) * q[3] + T(2) * q[4]) * T(1.0 / 60.0);
-            d = (q[0] - T(15) * q[1] + T(15) * q[2] - q[3]) * T(1.0 / 12.0);
-        }
-        return;
-    }
-    v = d = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const T w = S.w[k], bh = T(0.5) * S.b[k], c6 = S.c[k] * T(1.0 / 6.0);
-        if (PLUS) {
-            v += w * (bh + c6);
-            d += w * (S.b[k] + S.c[k]);
-        } else {
-            v += w * (c6 - bh);
-            d += w * (S.b[k] - S.c[k]);
-        }
-    }
-    v += S.q2;
+    T vp, dp, vm, dm;
+    teno_faces(q, S, vp, dp, vm, dm);
+    v = PLUS ? vp : vm;
+    d = PLUS ? dp : dm;
 }
 
 // WENO5-AO values and xi-derivatives at the faces: the quartic's (Eqs. 4.8,
@@ -333,48 +358,25 @@ GKS_HD void ao_gauss(const TenoSel<T>& S, T g, T& v, T& d)
     d = S.w3 * ld + sd;
 }
 
-// value and xi-derivative at the Gauss point xi = g (g = +-1/(2 sqrt 3), xi^2 = 1/12)
-template <typename T>
-GKS_HD void teno_gauss(const TenoSel<T>& S, T g, T& v, T& d)
-{
-    if (S.large) {
-        // P2(g) = 0, P3(g) = -g/15, P4(g) = -1/180; P3'(g) = 1/10, P4'(g) = -2g/21
-        v = S.q2 + S.u1 * g - S.u3 * g * T(1.0 / 15.0) - S.u4 * T(1.0 / 180.0);
-        d = S.u1 + T(2) * S.u2 * g + T(0.1) * S.u3 - T(2.0 / 21.0) * S.u4 * g;
-        return;
-    }
-    v = S.q2;
-    d = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        v += S.w[k] * S.b[k] * g;
-        d += S.w[k] * (S.b[k] + T(2) * S.c[k] * g);
-    }
-}
-
-// teno_gauss at both Gauss points xi = -g (vm, dm) and xi = +g (vp, dp),
-// g = 1/(2 sqrt 3): each value is E + xi O and each derivative Ed + xi Od,
-// with E, O, Ed, Od formed once for the two points
+// values and xi-derivatives at the Gauss points xi = -g (vm, dm) and xi = +g
+// (vp, dp), g = 1/(2 sqrt 3), where P2 = 0, P3 = -xi/15, P4 = -1/180,
+// P3' = 1/10, P4' = -2 xi/21: each value is E + xi O and each derivative
+// Ed + xi Od, with E = q2 - u4/180, O = u1 - u3/15, Ed = u1 + u3/10,
+// Od = 2 u2 - 2/21 u4 of the quartic, or q2, sum w b, sum w b, 2 sum w c
 template <typename T>
 GKS_HD void teno_gauss_pm(const TenoSel<T>& S, T g, T& vm, T& dm, T& vp, T& dp)
 {
     T E, O, Ed, Od;
     if (S.large) {
-        E = S.q2 - S.u4 * T(1.0 / 180.0);
-        O = S.u1 - S.u3 * T(1.0 / 15.0);
-        Ed = S.u1 + T(0.1) * S.u3;
-        Od = T(2) * S.u2 - T(2.0 / 21.0) * S.u4;
+        E = S.q2 - T(1.0 / 4320.0) * S.R;
+        O = T(43.0 / 72.0) * S.A - T(7.0 / 72.0) * S.B;
+        Ed = T(1.0 / 12.0) * S.P;
+        Od = T(12.0 / 9.0) * S.C - T(1.0 / 9.0) * S.D;
     } else {
-        T sb = S.w[0] * S.b[0], sc = S.w[0] * S.c[0];
-#pragma unroll
-        for (int k = 1; k < 3; ++k) {
-            sb += S.w[k] * S.b[k];
-            sc += S.w[k] * S.c[k];
-        }
+        T sb;
+        teno_small(S, sb, Od);
         E = S.q2;
-        O = sb;
-        Ed = sb;
-        Od = T(2) * sc;
+        O = Ed = T(0.5) * sb;
     }
     vm = E - g * O;
     vp = E + g * O;
@@ -509,8 +511,8 @@ GKS_HD void rec_faces(const T q[5], const TenoSel<T>& S, T& vp, T& dp, T& vm, T&
 template <int REC, typename T>
 GKS_HD void rec_gauss(const TenoSel<T>& S, T g, T& v, T& d)
 {
-    if constexpr (REC == 0) teno_gauss(S, g, v, d);
-    else if constexpr (REC == 1) ao_gauss(S, g, v, d);
+    static_assert(REC != 0, "TENO-D: teno_gauss_pm");
+    if constexpr (REC == 1) ao_gauss(S, g, v, d);
     else weno3_gauss(S, g, v, d);
 }
 

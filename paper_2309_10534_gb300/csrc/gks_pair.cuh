@@ -96,7 +96,8 @@ GKS_HD f2& operator*=(f2& a, f2 b) { return a = pmul(a, b); }
 // one formula evaluates either choice.  Same powers-of-ratios form as
 // teno_select (no division by beta, nothing overflows).
 struct TenoSel2 {
-    f2 q2, b[3], c[3], u1, u2, u3, u4, w[3];
+    f2 q2, A, B, C, D, B0, B2, C0, C2, P, R;  // as TenoSel
+    f2 l, w[3];                               // 1 where the large stencil is kept, else the sub-stencils' weights
 };
 
 GKS_HD float lane_min4(float a, float b, float c, float d) { return fminf(fminf(a, b), fminf(c, d)); }
@@ -104,9 +105,9 @@ GKS_HD float lane_min4(float a, float b, float c, float d) { return fminf(fminf(
 GKS_HD void teno_select_x2(const f2 q[5], const TenoT<float>& P, TenoSel2& S)
 {
     TenoSel<f2> C;
-    stencil_coeffs(q, C);
+    teno_differences(q, C);
     f2 t[4];
-    teno_indicators(C, f2(P.eps), t);
+    teno_indicators(C, f2(4.0f * P.eps), t);
     const f2 m(lane_min4(t[0].x(), t[1].x(), t[2].x(), t[3].x()), lane_min4(t[0].y(), t[1].y(), t[2].y(), t[3].y()));
     f2 p[4];
 #pragma unroll
@@ -131,18 +132,20 @@ GKS_HD void teno_select_x2(const f2 q[5], const TenoT<float>& P, TenoSel2& S)
     // largest, >= s012 / 3 > C_T2 s012), so dsum >= 1
     const f2 dsum = d[0] + d[1] + d[2];
     const f2 inv = f2((1.0f - lx) / dsum.x(), (1.0f - ly) / dsum.y());  // 0 on large-stencil lanes
-    const f2 lm(lx, ly);
     S.q2 = C.q2;
+    S.A = C.A;
+    S.B = C.B;
+    S.C = C.C;
+    S.D = C.D;
+    S.B0 = C.B0;
+    S.B2 = C.B2;
+    S.C0 = C.C0;
+    S.C2 = C.C2;
+    S.P = C.P;
+    S.R = C.R;
+    S.l = f2(lx, ly);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        S.b[k] = C.b[k];
-        S.c[k] = C.c[k];
-        S.w[k] = d[k] * inv;
-    }
-    S.u1 = C.u1 * lm;
-    S.u2 = C.u2 * lm;
-    S.u3 = C.u3 * lm;
-    S.u4 = C.u4 * lm;
+    for (int k = 0; k < 3; ++k) S.w[k] = d[k] * inv;
 }
 
 // the selection of lane x (y) as 4 bits (bit 0: large stencil; bits 1-3:
@@ -158,29 +161,32 @@ GKS_HD unsigned sel_code_y(const TenoSel2& S)
     return c ? c : 1u;
 }
 
+// 2 sum w_k b_k and 2 sum w_k c_k of the kept sub-stencils
+GKS_HD void teno_small_x2(const TenoSel2& S, f2& sb, f2& sc)
+{
+    sb = S.w[0] * S.B0;
+    sb += S.w[1] * S.A;
+    sb += S.w[2] * S.B2;
+    sc = S.w[0] * S.C0;
+    sc += S.w[1] * S.C;
+    sc += S.w[2] * S.C2;
+}
+
 // values and xi-derivatives at the faces xi = +-1/2 of both lanes' selection:
-// the quartic in the Legendre-type basis (P2(1/2) = 1/6, P3(1/2) = 1/20,
-// P4(1/2) = 1/70; P2' = 1, P3' = 3/5, P4' = 2/7 at 1/2, odd ones change sign
-// at -1/2), equal to Eqs. (4.8), (4.9) and their mirror, plus the
-// sub-stencil blend of Eqs. (4.13), (4.14)
+// teno_faces with both choices evaluated, the other one's terms zeroed
 GKS_HD void teno_faces_x2(const TenoSel2& S, f2& vp, f2& dp, f2& vm, f2& dm)
 {
-    const f2 even = S.q2 + S.u2 * f2(1.0f / 6.0f) + S.u4 * f2(1.0f / 70.0f);
-    const f2 odd = S.u1 * f2(0.5f) + S.u3 * f2(0.05f);
-    const f2 deven = S.u1 + S.u3 * f2(0.6f);
-    const f2 dodd = S.u2 + S.u4 * f2(2.0f / 7.0f);
+    f2 sb, sc;
+    teno_small_x2(S, sb, sc);
+    const f2 l24 = S.l * f2(1.0f / 24.0f), l120 = S.l * f2(1.0f / 120.0f);
+    const f2 even = l120 * f2(f2(13.0f) * S.C - S.D) + f2(f2(1.0f / 12.0f) * sc + S.q2);
+    const f2 odd = l24 * S.P + f2(f2(0.25f) * sb);
+    const f2 de = l24 * f2(f2(13.0f) * S.A - S.B) + f2(f2(0.5f) * sb);
+    const f2 dod = l24 * f2(f2(15.0f) * S.C - S.D) + f2(f2(0.5f) * sc);
     vp = even + odd;
     vm = even - odd;
-    dp = deven + dodd;
-    dm = deven - dodd;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const f2 bh = f2(0.5f) * S.b[k], c6 = S.c[k] * f2(1.0f / 6.0f);
-        vp += S.w[k] * (bh + c6);
-        vm += S.w[k] * (c6 - bh);
-        dp += S.w[k] * (S.b[k] + S.c[k]);
-        dm += S.w[k] * (S.b[k] - S.c[k]);
-    }
+    dp = de + dod;
+    dm = de - dod;
 }
 
 // Normal reconstruction of one 1-D cell's three variables (rho, rho u, E):
@@ -216,23 +222,17 @@ GKS_HD void recon_cell3(const T q[3][5], const TenoT<T>& P, T* vp, T* dp, T* vm,
 }
 
 // values and xi-derivatives at the two Gauss points xi = -g and xi = +g
-// (g = 1/(2 sqrt 3)) of both lanes' selection.  At the Gauss points
-// g^2 = 1/12, so P2 = 0, P3 = -xi/15, P4 = -1/180, P3' = 1/10, P4' = -2 xi/21
-// for the quartic, and the quadratics reduce to q2 + b xi: every value is
-// E + xi O and every derivative Ed + xi Od, with E, O, Ed, Od shared by the
-// two points.
+// (g = 1/(2 sqrt 3)) of both lanes' selection: teno_gauss_pm with both
+// choices evaluated, the other one's terms zeroed
 GKS_HD void teno_gauss_pm_x2(const TenoSel2& S, float g, f2& vm, f2& dm, f2& vp, f2& dp)
 {
-    f2 sb = S.w[0] * S.b[0], sc = S.w[0] * S.c[0];
-#pragma unroll
-    for (int k = 1; k < 3; ++k) {
-        sb += S.w[k] * S.b[k];
-        sc += S.w[k] * S.c[k];
-    }
-    const f2 E = S.q2 - S.u4 * f2(1.0f / 180.0f);
-    const f2 O = (S.u1 - S.u3 * f2(1.0f / 15.0f)) + sb;
-    const f2 Ed = (S.u1 + S.u3 * f2(0.1f)) + sb;
-    const f2 Od = (f2(2.0f) * S.u2 - S.u4 * f2(2.0f / 21.0f)) + f2(2.0f) * sc;
+    f2 sb, sc;
+    teno_small_x2(S, sb, sc);
+    const f2 hb = f2(0.5f) * sb;
+    const f2 E = S.q2 - f2(S.l * f2(1.0f / 4320.0f)) * S.R;
+    const f2 O = S.l * f2(f2(43.0f / 72.0f) * S.A - f2(7.0f / 72.0f) * S.B) + hb;
+    const f2 Ed = f2(S.l * f2(1.0f / 12.0f)) * S.P + hb;
+    const f2 Od = S.l * f2(f2(12.0f / 9.0f) * S.C - f2(1.0f / 9.0f) * S.D) + sc;
     const f2 G(g);
     vm = E - G * O;
     vp = E + G * O;
