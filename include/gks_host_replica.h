@@ -39,6 +39,11 @@ int gks_host_physical(int dim, int precision, double gamma, const double *W);
 int gks_host_teno(int precision, const double *q, double eps, int qpow, double ct1, double ct2,
                   double *faces, double *gauss);
 
+/* TENO-D selection of one stencil as 4 bits (bit 0: large stencil, bits 1-3:
+ * the kept sub-stencils): in float64, and as the float64 kernels decide it in
+ * float32 first (0: not decided there, the float64 selection is taken). */
+int gks_host_teno_code(const double *q, double eps, int qpow, double ct1, double ct2, int *code64, int *code32);
+
 /* F and dF/dt (per unit time, Sec. 2.2) at one interface point in the local
  * frame from the two sides' conserved variables and their normal (n) and
  * tangential (t) derivatives; 4 slots each, slot 2 unused in 1-D.

@@ -198,6 +198,20 @@ int weno_ao_packed(const double* q, double eps_ao, double d_hi, double d_lo, dou
 
 }  // namespace
 
+extern "C" int gks_host_teno_code(const double* q, double eps, int qpow, double ct1, double ct2, int* code64,
+                                  int* code32)
+{
+    if (!q || !code64 || !code32 || qpow < 1 || qpow > 32 || !(eps >= 0.0)) return -1;
+    const gks::TenoT<double> P = gks::teno_t<double>(gks::TenoParams{eps, qpow, ct1, ct2});
+    gks::TenoSel<double> S;
+    gks::teno_differences(q, S);
+    double t[4];
+    gks::teno_indicators(S, 4.0 * P.eps, t);
+    *code64 = (int)gks::teno_code(t, P.ct1, P.ct2, P.q);
+    *code32 = (int)gks::teno_code_f32(q, P);
+    return 0;
+}
+
 extern "C" int gks_host_weno_ao(int precision, const double* q, double eps_ao, double d_hi, double d_lo,
                                 double* faces, double* gauss)
 {

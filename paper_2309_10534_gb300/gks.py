@@ -425,6 +425,19 @@ def host_teno(q, precision="fp64", eps=1e-40, q_pow=7, ct1=1e-7, ct2=1e-5):
     return f, g, bool(r)
 
 
+def host_teno_code(q, eps=1e-40, q_pow=7, ct1=1e-7, ct2=1e-5):
+    """(float64 selection, the float64 kernels' float32 decision or 0) of one
+    stencil as 4-bit codes."""
+    qq, pq = _arr(q, 5)
+    a, b = C.c_int(0), C.c_int(0)
+    f = _replica().gks_host_teno_code
+    f.argtypes = [_dp, C.c_double, C.c_int, C.c_double, C.c_double, C.POINTER(C.c_int), C.POINTER(C.c_int)]
+    f.restype = C.c_int
+    if f(pq, eps, int(q_pow), ct1, ct2, C.byref(a), C.byref(b)):
+        raise ValueError("bad argument")
+    return a.value, b.value
+
+
 def host_point_flux(dim, Wl, Wln, Wlt, Wr, Wrn, Wrt, dt, precision="fp64", tau="euler", gamma=1.4,
                     mu=0.0, Pr=1.0, c1=0.01, c2=1.0):
     """(F, dF/dt) at one point from the host build of the device code; 4 slots."""
