@@ -541,9 +541,12 @@ GKS_HD void point_flux_vjp(const Side<T>& L, const Side<T>& R, const FluxParams<
                            Side<T>& gL, Side<T>& gR)
 {
     T W0[4] = {T(0), T(0), T(0), T(0)}, W0n[4] = {T(0), T(0), T(0), T(0)}, W0t[4] = {T(0), T(0), T(0), T(0)};
-    T d4[4], d5[4], d6[4], d7[4], d8[4], pl, pr;
-    side_terms<true, T, 2, false, false>(L, P, W0, W0n, W0t, d4, d5, d6, d7, d8, pl);
-    side_terms<false, T, 2, false, false>(R, P, W0, W0n, W0t, d4, d5, d6, d7, d8, pr);
+    T d4[4], d5[4], d6[4], d7[4], d8[4];
+    Prim<T> pl, pr;
+    prim_state<T, 2>(L.W, P.gm1, pl);
+    prim_state<T, 2>(R.W, P.gm1, pr);
+    side_terms<true, T, 2, false, false>(L, pl, P, W0, W0n, W0t, d4, d5, d6, d7, d8);
+    side_terms<false, T, 2, false, false>(R, pr, P, W0, W0n, W0t, d4, d5, d6, d7, d8);
     T gW0[4] = {T(0), T(0), T(0), T(0)}, gW0n[4] = {T(0), T(0), T(0), T(0)}, gW0t[4] = {T(0), T(0), T(0), T(0)};
     equilibrium_vjp(W0, W0n, W0t, P.gm1, gF, gdF, gW0, gW0n, gW0t);
     side_vjp(L, true, P, gW0, gW0n, gW0t, gL);

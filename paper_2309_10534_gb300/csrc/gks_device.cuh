@@ -55,6 +55,47 @@ template <> struct M<double> {
     static constexpr double s_noexp = 90.0;           // above: exp(-s/2) < 3e-20, below float64 resolution
 };
 
+// bits of a float64 and float32 (device: register moves)
+GKS_HD int hi_word(double x)
+{
+#ifdef __CUDA_ARCH__
+    return __double2hiint(x);
+#else
+    int64_t b;
+    memcpy(&b, &x, 8);
+    return (int)(b >> 32);
+#endif
+}
+GKS_HD unsigned lo_word(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (unsigned)__double2loint(x);
+#else
+    int64_t b;
+    memcpy(&b, &x, 8);
+    return (unsigned)b;
+#endif
+}
+GKS_HD float as_float(unsigned u)
+{
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(u);
+#else
+    float f;
+    memcpy(&f, &u, 4);
+    return f;
+#endif
+}
+GKS_HD float quick_div(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fdividef(a, b);
+#else
+    return a / b;
+#endif
+}
+GKS_HD int imax(int a, int b) { return a > b ? a : b; }
+
 // integer power by squaring (q of Eq. 4.5 is a small positive integer)
 template <typename T>
 GKS_HD T ipow(T x, int q)
@@ -266,47 +307,6 @@ GKS_HD unsigned teno_code(const T t[4], T ct1, T ct2, int q)
     const T thr = ct2 * s012;
     return (p[0] >= thr ? 2u : 0u) | (p[1] >= thr ? 4u : 0u) | (p[2] >= thr ? 8u : 0u);
 }
-
-// bits of a float64 and float32 (device: register moves)
-GKS_HD int hi_word(double x)
-{
-#ifdef __CUDA_ARCH__
-    return __double2hiint(x);
-#else
-    int64_t b;
-    memcpy(&b, &x, 8);
-    return (int)(b >> 32);
-#endif
-}
-GKS_HD unsigned lo_word(double x)
-{
-#ifdef __CUDA_ARCH__
-    return (unsigned)__double2loint(x);
-#else
-    int64_t b;
-    memcpy(&b, &x, 8);
-    return (unsigned)b;
-#endif
-}
-GKS_HD float as_float(unsigned u)
-{
-#ifdef __CUDA_ARCH__
-    return __uint_as_float(u);
-#else
-    float f;
-    memcpy(&f, &u, 4);
-    return f;
-#endif
-}
-GKS_HD float quick_div(float a, float b)
-{
-#ifdef __CUDA_ARCH__
-    return __fdividef(a, b);
-#else
-    return a / b;
-#endif
-}
-GKS_HD int imax(int a, int b) { return a > b ? a : b; }
 
 // The float64 selection decided in float32, or 0 where float32 cannot decide.
 //
@@ -807,15 +807,15 @@ template <typename T, int DIM>
 GKS_HD void prim_slope(const T* d, T U, T V, T q, T th, T gm1, Grad<T>& s)
 {
     s.r = d[0];
-    s.mU = d[1] - U * d[0];
+    s.mU = fma(-U, d[0], d[1]);
     if constexpr (DIM == 2) {
-        s.mV = d[2] - V * d[0];
-        s.p = gm1 * (d[3] - U * s.mU - V * s.mV - q * d[0]);
+        s.mV = fma(-V, d[0], d[2]);
+        s.p = gm1 * fma(-U, s.mU, fma(-V, s.mV, fma(-q, d[0], d[3])));
     } else {
         s.mV = T(0);
-        s.p = gm1 * (d[3] - U * s.mU - q * d[0]);
+        s.p = gm1 * fma(-U, s.mU, fma(-q, d[0], d[3]));
     }
-    s.mT = s.p - th * d[0];
+    s.mT = fma(-th, d[0], s.p);
 }
 
 // the time slopes that the compatibility condition <a_n u + a_t v + A> = 0
@@ -825,17 +825,17 @@ GKS_HD void time_slope(const Grad<T>& n, const Grad<T>& t, T U, T V, T th, T gm1
 {
     if constexpr (DIM == 2) {
         const T div = n.mU + t.mV;
-        g.r = -(U * n.r + V * t.r + div);
-        g.mU = -(U * n.mU + V * t.mU + n.p);
-        g.mV = -(U * n.mV + V * t.mV + t.p);
-        g.mT = -(U * n.mT + V * t.mT + gm1 * th * div);
+        g.r = fma(-U, n.r, fma(-V, t.r, -div));
+        g.mU = fma(-U, n.mU, fma(-V, t.mU, -n.p));
+        g.mV = fma(-U, n.mV, fma(-V, t.mV, -t.p));
+        g.mT = fma(-U, n.mT, fma(-V, t.mT, -(gm1 * th) * div));
     } else {
-        g.r = -(U * n.r + n.mU);
-        g.mU = -(U * n.mU + n.p);
+        g.r = fma(-U, n.r, -n.mU);
+        g.mU = fma(-U, n.mU, -n.p);
         g.mV = T(0);
-        g.mT = -(U * n.mT + gm1 * th * n.mU);
+        g.mT = fma(-U, n.mT, -(gm1 * th) * n.mU);
     }
-    g.p = g.mT + th * g.r;
+    g.p = fma(th, g.r, g.mT);
 }
 
 // a Maxwellian's u-moments (half or full space) with the multiples their
@@ -847,13 +847,13 @@ template <typename T> struct UMom {
 template <typename T>
 GKS_HD void u_moments(UMom<T>& m, T U, T th, bool fourth)
 {
-    m.u2 = U * m.u1 + th * m.u0;
+    m.u2 = fma(U, m.u1, th * m.u0);
     m.u1x2 = T(2) * m.u1;
-    m.u3 = U * m.u2 + th * m.u1x2;
+    m.u3 = fma(U, m.u2, th * m.u1x2);
     if (fourth) {
         m.u1x3 = T(3) * m.u1;
         m.u2x3 = T(3) * m.u2;
-        m.u4 = U * m.u3 + th * m.u2x3;
+        m.u4 = fma(U, m.u3, th * m.u2x3);
         m.u2x6 = T(2) * m.u2x3;
         m.u3x4 = T(4) * m.u3;
     }
@@ -864,23 +864,28 @@ template <typename T> GKS_HD T d_u2(const UMom<T>& m, const Grad<T>& g) { return
 template <typename T> GKS_HD T d_u3(const UMom<T>& m, const Grad<T>& g) { return fma(g.mT, m.u1x3, fma(g.mU, m.u2x3, g.r * m.u3)); }
 template <typename T> GKS_HD T d_u4(const UMom<T>& m, const Grad<T>& g) { return fma(g.mT, m.u2x6, fma(g.mU, m.u3x4, g.r * m.u4)); }
 
+// rho d((V^2 + (K + D - 1) th)/2)
+template <int DIM, typename T> GKS_HD T kappa(T V, const Grad<T>& g, T hkv)
+{
+    return (DIM == 2) ? fma(V, g.mV, hkv * g.mT) : hkv * g.mT;
+}
+
 // o (+)= d(rho <u^k psi>) from Dk = d(rho u_k), Dk+1, Dk+2: with
 // e = (V^2 + (K + D - 1) th)/2, <u^k psi> = (u_k, u_(k+1), V u_k,
 // u_(k+2)/2 + e u_k); kap = rho de
 template <bool ADD, typename T, int DIM>
 GKS_HD void d_mom(T* o, T Dk, T Dk1, T Dk2, T uk, T V, T e, T mV, T kap)
 {
-    const T x = e * Dk + T(0.5) * Dk2;
     if constexpr (ADD) {
         o[0] += Dk;
         o[1] += Dk1;
         if constexpr (DIM == 2) o[2] = fma(V, Dk, fma(mV, uk, o[2]));
-        o[3] += fma(kap, uk, x);
+        o[3] = fma(kap, uk, fma(e, Dk, fma(T(0.5), Dk2, o[3])));
     } else {
         o[0] = Dk;
         o[1] = Dk1;
         o[2] = (DIM == 2) ? fma(V, Dk, mV * uk) : T(0);
-        o[3] = fma(kap, uk, x);
+        o[3] = fma(kap, uk, fma(e, Dk, T(0.5) * Dk2));
     }
 }
 
@@ -900,17 +905,17 @@ GKS_HD void d_cross(T* o, T Dk, T Dk1, T Dk2, T uk, T uk1, T uk2, T V, T th, T e
 template <bool ADD, typename T, int DIM>
 GKS_HD void mom(T* o, T r, T uk, T uk1, T uk2, T V, T e)
 {
-    const T ru = r * uk;
+    const T ru = r * uk, hr = T(0.5) * r;
     if constexpr (ADD) {
         o[0] += ru;
         o[1] = fma(r, uk1, o[1]);
         if constexpr (DIM == 2) o[2] = fma(V, ru, o[2]);
-        o[3] = fma(e, ru, fma(T(0.5) * r, uk2, o[3]));
+        o[3] = fma(e, ru, fma(hr, uk2, o[3]));
     } else {
         o[0] = ru;
         o[1] = r * uk1;
         o[2] = (DIM == 2) ? V * ru : T(0);
-        o[3] = fma(e, ru, T(0.5) * r * uk2);
+        o[3] = fma(e, ru, hr * uk2);
     }
 }
 
@@ -932,7 +937,7 @@ GKS_HD void half_space_start<double>(double z, double sg, double& h0, double& g)
     g = exp(-z * z);
 #ifdef __CUDA_ARCH__
     const double h = 0.5 * (g * erfcx(fabs(z)));
-    h0 = (sg * z >= 0.0) ? 1.0 - h : h;
+    h0 = ((hi_word(z) < 0) == (sg < 0.0)) ? 1.0 - h : h;
 #else
     h0 = 0.5 * erfc(-sg * z);
 #endif
@@ -943,7 +948,7 @@ GKS_HD void half_space_start<float>(float z, float sg, float& h0, float& g)
     const float x = fabsf(z);
 #ifdef __CUDA_ARCH__
     g = __expf(-x * x);
-    const float t = __frcp_rn(1.0f + 0.3275911f * x);
+    const float t = __fdividef(1.0f, fmaf(0.3275911f, x, 1.0f));
 #else
     g = expf(-x * x);
     const float t = 1.0f / (1.0f + 0.3275911f * x);
@@ -1106,18 +1111,48 @@ template <typename T> struct Side {  // one reconstructed side (local frame, 4 s
 // colder than that need the float64 path.
 constexpr double kMinInternalFractionF32 = 1e-4;
 
-// rho > 0 and p > 0 (finite); float32 states also need an internal energy
-// of at least kMinInternalFractionF32 of E
+// Primitive variables of a conserved state: 1/rho, velocities, V^2/2,
+// |U|^2/2, pressure
+template <typename T> struct Prim {
+    T r, ir, U, V, hv2, q, p;
+};
+
+// x > 0 and finite (float64: by its bits, a comparison would run on the
+// float64 pipe)
+GKS_HD bool pos_finite(double x)
+{
+    const unsigned hi = (unsigned)hi_word(x);
+    return hi < 0x7ff00000u && (hi | lo_word(x)) != 0u;
+}
+template <typename T>
+GKS_HD bool pos_finite(T x)
+{
+    return x > T(0) && isfinite(x);
+}
+
+// Fills s and tests the state: rho > 0 and p > 0 (finite); float32 states
+// also need an internal energy of at least kMinInternalFractionF32 of E
+template <typename T, int DIM>
+GKS_HD bool prim_state(const T* W, T gm1, Prim<T>& s)
+{
+    s.r = W[0];
+    s.ir = T(1) / s.r;
+    s.U = W[1] * s.ir;
+    s.V = (DIM == 2) ? W[2] * s.ir : T(0);
+    s.hv2 = (DIM == 2) ? T(0.5) * s.V * s.V : T(0);
+    s.q = fma(T(0.5) * s.U, s.U, s.hv2);
+    const T e = fma(-s.r, s.q, W[3]);  // internal energy per volume
+    s.p = gm1 * e;
+    bool ok = s.r > T(0) && pos_finite(s.p);
+    if constexpr (std::is_same<T, double>::value) ok = pos_finite(s.r) && pos_finite(s.p);
+    if constexpr (sizeof(T) == 4) ok = ok && e >= T(kMinInternalFractionF32) * W[3];
+    return ok;
+}
 template <typename T, int DIM>
 GKS_HD bool physical(const T* W, T gm1)
 {
-    const T r = W[0];
-    const T ke = (DIM == 2) ? (W[1] * W[1] + W[2] * W[2]) : W[1] * W[1];
-    const T e = W[3] - T(0.5) * ke * (T(1) / r);  // internal energy per volume
-    const T p = gm1 * e;
-    bool ok = r > T(0) && p > T(0) && isfinite(p);
-    if constexpr (sizeof(T) == 4) ok = ok && e >= T(kMinInternalFractionF32) * W[3];
-    return ok;
+    Prim<T> s;
+    return prim_state<T, DIM>(W, gm1, s);
 }
 
 // Kinetic merge of two states (values only; Eq. 3.25 with reading R2): the
@@ -1155,17 +1190,12 @@ GKS_HD void merge_values(const T* Wl, const T* Wr, const FluxParams<T>& P, T* W0
 // Eqs. 2.6, 3.25, 3.26) and to the non-equilibrium terms of Eq. (2.5); the
 // left side (u > 0) sets the sums, the right side (u < 0) adds to them.
 template <bool UPPER, typename T, int DIM, bool NONEQ, bool PRFIX>
-GKS_HD void side_terms(const Side<T>& S, const FluxParams<T>& P, T* W0, T* W0n, T* W0t, T* S3, T* S4, T* S5, T* N4,
-                       T* N5, T& pside)
+GKS_HD void side_terms(const Side<T>& S, const Prim<T>& pr, const FluxParams<T>& P, T* W0, T* W0n, T* W0t, T* S3, T* S4, T* S5, T* N4,
+                       T* N5)
 {
     constexpr bool ADD = !UPPER;
-    const T r = S.W[0], ir = T(1) / r;
-    const T U = S.W[1] * ir;
-    const T V = (DIM == 2) ? S.W[2] * ir : T(0);
-    const T q = (DIM == 2) ? T(0.5) * (U * U + V * V) : T(0.5) * U * U;
-    const T p = P.gm1 * (S.W[3] - r * q);
-    pside = p;
-    const T th = p * ir;                     // 1/(2 lambda)
+    const T r = pr.r, U = pr.U, V = pr.V, q = pr.q, hv2 = pr.hv2;
+    const T th = pr.p * pr.ir;               // 1/(2 lambda)
     const T sl = M<T>::rsqrt_(T(2) * th);    // sqrt(lambda)
 
     // half-space u-moments: u > 0 (left state) or u < 0 (right state);
@@ -1176,26 +1206,26 @@ GKS_HD void side_terms(const Side<T>& S, const FluxParams<T>& P, T* W0, T* W0n, 
     half_space_start<T>(sl * U, sg, m.u0, gz);
     const T w = (sg * T(0.56418958354775628)) * (sl * gz);  // 1/sqrt(pi)
     const T wt = th * w;
-    m.u1 = U * m.u0 + wt;
+    m.u1 = fma(U, m.u0, wt);
     u_moments(m, U, th, NONEQ);
-    const T e = (DIM == 2) ? T(0.5) * (V * V) + P.hkv * th : P.hkv * th;
+    const T e = fma(P.hkv, th, hv2);
 
     Grad<T> n, t;
     prim_slope<T, DIM>(S.Wn, U, V, q, th, P.gm1, n);
     const T hit = sl * sl;                   // 1/(2 th)
-    const T kn = (DIM == 2) ? V * n.mV + P.hkv * n.mT : P.hkv * n.mT;
+    const T kn = kappa<DIM>(V, n, P.hkv);
     mom<ADD, T, DIM>(W0, r, m.u0, m.u1, m.u2, V, e);
     const T cn = hit * n.mT;
-    const T n0 = fma(n.r, m.u0, w * (n.mU - U * cn));
+    const T n0 = fma(n.r, m.u0, w * fma(-U, cn, n.mU));
     const T n1 = fma(n.r, m.u1, fma(n.mU, m.u0, cn * wt));
     const T n2 = d_u2(m, n);
     d_mom<ADD, T, DIM>(W0n, n0, n1, n2, m.u0, V, e, n.mV, kn);
     T t0 = T(0), t1 = T(0), t2 = T(0), kt = T(0);
     if constexpr (DIM == 2) {
         prim_slope<T, DIM>(S.Wt, U, V, q, th, P.gm1, t);
-        kt = V * t.mV + P.hkv * t.mT;
+        kt = kappa<DIM>(V, t, P.hkv);
         const T ct = hit * t.mT;
-        t0 = fma(t.r, m.u0, w * (t.mU - U * ct));
+        t0 = fma(t.r, m.u0, w * fma(-U, ct, t.mU));
         t1 = fma(t.r, m.u1, fma(t.mU, m.u0, ct * wt));
         t2 = d_u2(m, t);
         d_mom<ADD, T, DIM>(W0t, t0, t1, t2, m.u0, V, e, t.mV, kt);
@@ -1207,12 +1237,12 @@ GKS_HD void side_terms(const Side<T>& S, const FluxParams<T>& P, T* W0, T* W0n, 
     if constexpr (NONEQ) {
         Grad<T> g;  // time derivative of the side's Maxwellian
         time_slope<T, DIM>(n, t, U, V, th, P.gm1, g);
-        const T kg = (DIM == 2) ? V * g.mV + P.hkv * g.mT : P.hkv * g.mT;
+        const T kg = kappa<DIM>(V, g, P.hkv);
         const T cg = hit * g.mT;
         const T g1 = fma(g.r, m.u1, fma(g.mU, m.u0, cg * wt));
         const T g2 = d_u2(m, g);
         if constexpr (PRFIX) {  // density moments of the A and slope terms (heat flux)
-            const T g0 = fma(g.r, m.u0, w * (g.mU - U * cg));
+            const T g0 = fma(g.r, m.u0, w * fma(-U, cg, g.mU));
             d_mom<ADD, T, DIM>(N5, g0, g1, g2, m.u0, V, e, g.mV, kg);
         }
         // flux moments of the side terms of Eq. (2.5) over the half space
@@ -1229,20 +1259,23 @@ GKS_HD void side_terms(const Side<T>& S, const FluxParams<T>& P, T* W0, T* W0n, 
 }
 
 // F and dF/dt (per unit time; Sec. 2.2) at one interface point in the local
-// frame.  Both sides must be physical (the caller applies the fallback).
+// frame.  state(0, L, p) and state(1, R, p) form a side's primitive variables
+// (prim_state) and apply the caller's fallback where it is not physical.
 // need_F = false: only dF is formed (the second stage uses nothing else).
 // W0n_lin, W0_lin, W0t_lin: the conventional path's equilibrium normal
 // slope (Eq. 3.12, in 2-D reconstructed to the point), state and tangential
 // slope (2-D: linear reconstructions of line-averaged merges, Step 4),
 // replacing the kinetic merge at the point; nullptr otherwise
-template <typename T, int DIM, bool NONEQ, bool PRFIX>
-GKS_HD void point_flux(const Side<T>& L, const Side<T>& R, const FluxParams<T>& P, T* F, T* dF, bool need_F = true,
+template <typename T, int DIM, bool NONEQ, bool PRFIX, typename State>
+GKS_HD void point_flux(Side<T>& L, Side<T>& R, const FluxParams<T>& P, T* F, T* dF, bool need_F, State&& state,
                        const T* W0n_lin = nullptr, const T* W0_lin = nullptr, const T* W0t_lin = nullptr)
 {
     T W0[4], W0n[4], W0t[4], S3[4], S4[4], S5[4], N4[4], N5[4];
-    T pl, pr;
-    side_terms<true, T, DIM, NONEQ, PRFIX>(L, P, W0, W0n, W0t, S3, S4, S5, N4, N5, pl);
-    side_terms<false, T, DIM, NONEQ, PRFIX>(R, P, W0, W0n, W0t, S3, S4, S5, N4, N5, pr);
+    Prim<T> pl, pr;
+    state(0, L, pl);
+    state(1, R, pr);
+    side_terms<true, T, DIM, NONEQ, PRFIX>(L, pl, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
+    side_terms<false, T, DIM, NONEQ, PRFIX>(R, pr, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
     // the kinetic merge is also the density moment of the side terms (the
     // heat flux needs it even where W0 is replaced below)
     T W0k[4];
@@ -1276,8 +1309,9 @@ GKS_HD void point_flux(const Side<T>& L, const Side<T>& R, const FluxParams<T>& 
     const T r0 = W0[0], ir0 = T(1) / r0;
     const T U0 = W0[1] * ir0;
     const T V0 = (DIM == 2) ? W0[2] * ir0 : T(0);
-    const T q0 = (DIM == 2) ? T(0.5) * (U0 * U0 + V0 * V0) : T(0.5) * U0 * U0;
-    const T p0 = P.gm1 * (W0[3] - r0 * q0);
+    const T hv2 = (DIM == 2) ? T(0.5) * V0 * V0 : T(0);
+    const T q0 = fma(T(0.5) * U0, U0, hv2);
+    const T p0 = P.gm1 * fma(-r0, q0, W0[3]);
     const T Ep = W0[3] + p0, th0 = p0 * ir0;
     Grad<T> n, t, g;
     prim_slope<T, DIM>(W0n, U0, V0, q0, th0, P.gm1, n);
@@ -1285,17 +1319,18 @@ GKS_HD void point_flux(const Side<T>& L, const Side<T>& R, const FluxParams<T>& 
     time_slope<T, DIM>(n, t, U0, V0, th0, P.gm1, g);
     T F0[4], F2[4];
     F0[0] = W0[1];
-    F0[1] = W0[1] * U0 + p0;
+    F0[1] = fma(W0[1], U0, p0);
     F0[2] = (DIM == 2) ? W0[1] * V0 : T(0);
     F0[3] = U0 * Ep;
     {
-        const T mt = g.mU + U0 * g.r;  // d(rho U)
+        const T mt = fma(U0, g.r, g.mU);  // d(rho U)
         F2[0] = mt;
-        F2[1] = U0 * (mt + g.mU) + g.p;
-        F2[2] = (DIM == 2) ? V0 * mt + U0 * g.mV : T(0);
+        F2[1] = fma(U0, mt + g.mU, g.p);
+        F2[2] = (DIM == 2) ? fma(V0, mt, U0 * g.mV) : T(0);
         // rho U H: H d(rho U) + U rho dH, rho dH = U rho dU + V rho dV + cp rho dth
-        const T rdH = (DIM == 2) ? U0 * g.mU + V0 * g.mV + P.cp * g.mT : U0 * g.mU + P.cp * g.mT;
-        F2[3] = (Ep * ir0) * mt + U0 * rdH;
+        T rdH = fma(U0, g.mU, P.cp * g.mT);
+        if constexpr (DIM == 2) rdH = fma(V0, g.mV, rdH);
+        F2[3] = fma(Ep * ir0, mt, U0 * rdH);
     }
 
     if (P.tau_mode == 0) {
@@ -1308,7 +1343,7 @@ GKS_HD void point_flux(const Side<T>& L, const Side<T>& R, const FluxParams<T>& 
     }
     // collision time and time coefficients: is = tau / dt
     T cF[6], cD[6];
-    const T jump = fabs(pl - pr) / (pl + pr);
+    const T jump = fabs(pl.p - pr.p) / (pl.p + pr.p);
     const T dt = P.dt, idt = T(1) / dt;
     const T is = (P.tau_mode == 1) ? P.c1 + P.c2 * jump : P.mu * idt / p0 + P.c2 * jump;
     time_coeffs<T>(T(1) / is, is, cF, cD);
@@ -1319,12 +1354,12 @@ GKS_HD void point_flux(const Side<T>& L, const Side<T>& R, const FluxParams<T>& 
         m.u0 = T(1);
         m.u1 = U0;
         u_moments(m, U0, th0, true);
-        const T e = (DIM == 2) ? T(0.5) * (V0 * V0) + P.hkv * th0 : P.hkv * th0;
-        const T kn = (DIM == 2) ? V0 * n.mV + P.hkv * n.mT : P.hkv * n.mT;
+        const T e = fma(P.hkv, th0, hv2);
+        const T kn = kappa<DIM>(V0, n, P.hkv);
         d_mom<false, T, DIM>(F1, d_u2(m, n), d_u3(m, n), d_u4(m, n), m.u2, V0, e, n.mV, kn);
         if constexpr (DIM == 2)
-            d_cross<T>(F1, t.r * U0 + t.mU, d_u2(m, t), d_u3(m, t), U0, m.u2, m.u3, V0, th0, e, t.mV, t.mT,
-                       V0 * t.mV + P.hkv * t.mT);
+            d_cross<T>(F1, fma(t.r, U0, t.mU), d_u2(m, t), d_u3(m, t), U0, m.u2, m.u3, V0, th0, e, t.mV, t.mT,
+                       kappa<DIM>(V0, t, P.hkv));
     }
     // Prandtl correction: F_E += (1/Pr - 1) q, q the heat flux relative to
     // (U0, V0) expanded in raw moments of the same time-dependent f.
@@ -1346,7 +1381,7 @@ GKS_HD void point_flux(const Side<T>& L, const Side<T>& R, const FluxParams<T>& 
         const T c0 = c[0] * s1, c1 = c[1] * s2, c2 = c[2] * s2, c3 = c[3] * s1, c4 = c[4] * s2, c5 = c[5] * s2;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            o[i] = c0 * F0[i] + c1 * F1[i] + c2 * F2[i] + c3 * S3[i] + c4 * S4[i] + c5 * S5[i];
+            o[i] = fma(c0, F0[i], fma(c1, F1[i], fma(c2, F2[i], fma(c3, S3[i], fma(c4, S4[i], c5 * S5[i])))));
         if constexpr (PRFIX) {
             T Mo[4];
 #pragma unroll
@@ -1358,6 +1393,18 @@ GKS_HD void point_flux(const Side<T>& L, const Side<T>& R, const FluxParams<T>& 
     // qF_k = cF_k dt^{p_k - 1}, qD_k = 4 cD_k dt^{p_k - 2}
     if (need_F) combine(cF, T(1), dt, F);
     combine(cD, T(4) * idt, T(4), dF);
+}
+
+// the same for two physical sides
+template <typename T, int DIM>
+struct PlainState {
+    T gm1;
+    GKS_HD void operator()(int, Side<T>& S, Prim<T>& p) const { prim_state<T, DIM>(S.W, gm1, p); }
+};
+template <typename T, int DIM, bool NONEQ, bool PRFIX>
+GKS_HD void point_flux(Side<T>& L, Side<T>& R, const FluxParams<T>& P, T* F, T* dF)
+{
+    point_flux<T, DIM, NONEQ, PRFIX>(L, R, P, F, dF, true, PlainState<T, DIM>{P.gm1});
 }
 
 }  // namespace gks

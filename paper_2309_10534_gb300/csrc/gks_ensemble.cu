@@ -159,20 +159,15 @@ __device__ void stage_chunk(ChunkSmem<T, NT>& sm, double* W, float* Wf, T* Ws, T
             R.W[slot[v]] = sm.R[v][0][f];
             R.Wn[slot[v]] = sm.R[v][1][f];
         }
-        if (!physical<T, 1>(L.W, fp.gm1)) {
+        auto state = [&](int side, Side<T>& S, Prim<T>& p) {
+            if (prim_state<T, 1>(S.W, fp.gm1, p)) return;
 #pragma unroll
-            for (int v = 0; v < 3; ++v) { L.W[slot[v]] = sm.q[v][f + 2]; L.Wn[slot[v]] = T(0); }
+            for (int v = 0; v < 3; ++v) { S.W[slot[v]] = sm.q[v][f + 2 + side]; S.Wn[slot[v]] = T(0); }
             ++nfb;
-            if (!physical<T, 1>(L.W, fp.gm1)) err |= 2u;
-        }
-        if (!physical<T, 1>(R.W, fp.gm1)) {
-#pragma unroll
-            for (int v = 0; v < 3; ++v) { R.W[slot[v]] = sm.q[v][f + 3]; R.Wn[slot[v]] = T(0); }
-            ++nfb;
-            if (!physical<T, 1>(R.W, fp.gm1)) err |= 2u;
-        }
+            if (!prim_state<T, 1>(S.W, fp.gm1, p)) err |= 2u;
+        };
         T F[4], dF[4];
-        point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, stage == 1);
+        point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, stage == 1, state);
 #pragma unroll
         for (int v = 0; v < 3; ++v) stage_comb<T>(stage, F[slot[v]], dF[slot[v]], tdt, sm.G[0][v][f], sm.G[1][v][f]);
     }

@@ -312,18 +312,13 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(GridDev g, Stage1DArgs a, Fl
             R.W[slot[v]] = sR[v][0][f];
             R.Wn[slot[v]] = sR[v][1][f];
         }
-        if (!physical<T, 1>(L.W, fp.gm1)) {
+        auto state = [&](int side, Side<T>& S, Prim<T>& p) {
+            if (prim_state<T, 1>(S.W, fp.gm1, p)) return;
 #pragma unroll
-            for (int v = 0; v < 3; ++v) { L.W[slot[v]] = sq[v][f + 2]; L.Wn[slot[v]] = T(0); }
+            for (int v = 0; v < 3; ++v) { S.W[slot[v]] = sq[v][f + 2 + side]; S.Wn[slot[v]] = T(0); }
             ++nfb;
-            if (!physical<T, 1>(L.W, fp.gm1)) err |= 2u;
-        }
-        if (!physical<T, 1>(R.W, fp.gm1)) {
-#pragma unroll
-            for (int v = 0; v < 3; ++v) { R.W[slot[v]] = sq[v][f + 3]; R.Wn[slot[v]] = T(0); }
-            ++nfb;
-            if (!physical<T, 1>(R.W, fp.gm1)) err |= 2u;
-        }
+            if (!prim_state<T, 1>(S.W, fp.gm1, p)) err |= 2u;
+        };
         T F[4], dF[4];
         if constexpr (rec_conventional(REC)) {
             // conventional path: equilibrium slope from the cell averages
@@ -333,9 +328,9 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(GridDev g, Stage1DArgs a, Fl
             for (int v = 0; v < 3; ++v)
                 w0n[slot[v]] = (T(1.25) * (sq[v][f + 3] - sq[v][f + 2]) - T(1.0 / 12.0) * (sq[v][f + 4] - sq[v][f + 1]))
                              * idx_;
-            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, w0n);
+            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state, w0n);
         } else {
-            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1);
+            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state);
         }
         const T tdt = s_scal[0];
 #pragma unroll
@@ -658,18 +653,13 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
         }
         T F[4] = {T(0), T(0), T(0), T(0)}, dF[4] = {T(0), T(0), T(0), T(0)};
         if (valid) {
-            if (!physical<T, 2>(L.W, fp.gm1)) {
+            auto state = [&](int side, Side<T>& S, Prim<T>& p) {
+                if (prim_state<T, 2>(S.W, fp.gm1, p)) return;
 #pragma unroll
-                for (int v = 0; v < 4; ++v) { L.W[v] = sm.w[v][r + 2][f + 2]; L.Wn[v] = L.Wt[v] = T(0); }
+                for (int v = 0; v < 4; ++v) { S.W[v] = sm.w[v][r + 2][f + 2 + side]; S.Wn[v] = S.Wt[v] = T(0); }
                 ++nfb;
-                if (!physical<T, 2>(L.W, fp.gm1)) err |= 2u;
-            }
-            if (!physical<T, 2>(R.W, fp.gm1)) {
-#pragma unroll
-                for (int v = 0; v < 4; ++v) { R.W[v] = sm.w[v][r + 2][f + 3]; R.Wn[v] = R.Wt[v] = T(0); }
-                ++nfb;
-                if (!physical<T, 2>(R.W, fp.gm1)) err |= 2u;
-            }
+                if (!prim_state<T, 2>(S.W, fp.gm1, p)) err |= 2u;
+            };
             if constexpr (CONV) {
                 // Step 4: the equilibrium state and slopes at this lane's Gauss
                 // point, linear (quartic) reconstructions of the rows' merges
@@ -689,13 +679,13 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
                 // a non-physical linear state (the quartic across a
                 // discontinuity) falls back to the kinetic merge at the point
                 if (physical<T, 2>(w0g, fp.gm1)) {
-                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, w0n, w0g, w0t);
+                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state, w0n, w0g, w0t);
                 } else {
                     ++nfb;
-                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1);
+                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state);
                 }
             } else {
-                point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1);
+                point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state);
             }
         }
         // the stage's combinations at both points, averaged (weights 1/2): each
