@@ -206,11 +206,10 @@ gks_status fill_ghosts_f64(gks_ctx* c, double* arr, cudaStream_t st)
 
 }  // namespace rt
 }  // namespace gks
-using gks::rt::enqueue_ghosts;
-
 namespace {
 
-gks_status enqueue_stage(gks_ctx* c, int stage, int with_sigma, cudaStream_t st)
+// with_commit: the last kernel reduces the CFL rate and commits the step
+gks_status enqueue_stage(gks_ctx* c, int stage, int with_commit, cudaStream_t st)
 {
     const HostFlux hf = host_flux(c);
     const TenoParams tn = teno_params(c, false), tt = teno_params(c, true);
@@ -218,7 +217,7 @@ gks_status enqueue_stage(gks_ctx* c, int stage, int with_sigma, cudaStream_t st)
     if (c->desc.dim == 1) {
         Stage1DArgs a{};
         a.stage = stage;
-        a.with_sigma = with_sigma;
+        a.with_sigma = a.commit = with_commit;
         a.idx = 1.0 / c->g.dx;
         if (f32) {
             // float32 W* (Wsf) and accumulator increment (inc1)
@@ -260,7 +259,7 @@ gks_status enqueue_stage(gks_ctx* c, int stage, int with_sigma, cudaStream_t st)
             a.nn = c->desc.ny; a.nt = c->desc.nx; a.sn = c->g.pitch; a.st = 1;
             a.ihn = 1.0 / c->g.dy; a.iht = 1.0 / c->g.dx;
         }
-        a.with_sigma = (pass == 1) ? with_sigma : 0;
+        a.with_sigma = a.commit = (pass == 1) ? with_commit : 0;
         const int pi = prof_begin(c, st, 0);
         cudaError_t e = f32 ? launch_sweep_f32(c->g, a, hf, tn, tt, c->ds, st)
                             : launch_sweep_f64(c->g, a, hf, tn, tt, c->ds, st);
@@ -309,25 +308,21 @@ gks_status enqueue_sigma(gks_ctx* c, cudaStream_t st)
     return GKS_OK;
 }
 
-gks_status enqueue_commit(gks_ctx* c, int init, cudaStream_t st)
+gks_status enqueue_first_dt(gks_ctx* c, cudaStream_t st)
 {
     const int pi = prof_begin(c, st, 2);
-    k_commit<<<1, 32, 0, st>>>(c->ds, init);
+    k_commit<<<1, 32, 0, st>>>(c->ds);
     CK(cudaGetLastError());
     prof_end(c, st, pi);
     ++c->launches;
     return GKS_OK;
 }
 
-// one S2O4 step: ghosts(W), stage 1, ghosts(W*), stage 2 (+ CFL rate), commit
+// one S2O4 step: stage 1, stage 2 (+ CFL rate and commit)
 gks_status enqueue_step(gks_ctx* c, cudaStream_t st)
 {
-    gks_status s;
-    if ((s = enqueue_ghosts(c, c->W, st))) return s;
-    if ((s = enqueue_stage(c, 1, 0, st))) return s;
-    if ((s = enqueue_ghosts(c, c->Ws, st))) return s;
-    if ((s = enqueue_stage(c, 2, 1, st))) return s;
-    return enqueue_commit(c, 0, st);
+    const gks_status s = enqueue_stage(c, 1, 0, st);
+    return s ? s : enqueue_stage(c, 2, 1, st);
 }
 
 gks_status sync_state(gks_ctx* c)
@@ -732,8 +727,6 @@ gks_status gks_stage(gks_ctx* c, int stage, double dt)
     k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 0, dt, 0.0, 0);
     CK(cudaGetLastError());
     ++c->launches;
-    gks_status s = enqueue_ghosts(c, stage == 1 ? c->W : c->Ws, c->stream);
-    if (s) return s;
     return enqueue_stage(c, stage, 0, c->stream);
 }
 
@@ -752,7 +745,7 @@ gks_status gks_step(gks_ctx* c, double dt)
         CK(cudaGetLastError());
         ++c->launches;
         if ((s = enqueue_sigma(c, c->stream))) return s;
-        if ((s = enqueue_commit(c, 1, c->stream))) return s;
+        if ((s = enqueue_first_dt(c, c->stream))) return s;
     }
     // else: the previous CFL step's commit already chose dt from this state
     s = enqueue_step(c, c->stream);
@@ -778,7 +771,7 @@ gks_status gks_advance_to(gks_ctx* c, double t_end, long long max_steps, long lo
     CK(cudaGetLastError());
     ++c->launches;
     if ((s = enqueue_sigma(c, c->stream))) return s;
-    if ((s = enqueue_commit(c, 1, c->stream))) return s;
+    if ((s = enqueue_first_dt(c, c->stream))) return s;
     if ((s = build_graph(c))) return s;
     for (;;) {
         CK(cudaGraphLaunch(c->graph, c->stream));

@@ -8,20 +8,17 @@
 namespace gks {
 
 // ------------------------------------------------------------------ ghosts
-// One thread per ghost cell.  x ghosts of interior rows use the x rule; rows
-// of y ghosts use the y rule to pick an interior row, then the x rule for
-// x-ghost columns (the same values as filling x first, then y over the full
-// ghosted width).
-// State-setting rules (inflow, wall after x0, moving shock) write their state;
-// toff: the array's time is t + toff dt (0 for W, 1/2 for W*).
+// The ghost layers in memory, for callers that read them there (the adjoint,
+// the selection count); the stage kernels form their own.  One thread per
+// ghost cell (cell_source).
 template <typename E>
-__global__ void k_fill_ghosts(GridDev g, E* __restrict__ W, const DevState* ds, double toff)
+__global__ void k_fill_ghosts(const __grid_constant__ GridDev g, E* __restrict__ W, const DevState* ds, double toff)
 {
     if (ds && ds->done) return;
     const int gx = g.nx + 2 * NG;
     const int nv = g.dim + 2;
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    int i, j;
+    int i, j;  // ghosted position
     if (g.dim == 1) {
         if (idx >= 2 * NG) return;
         j = 0;
@@ -40,37 +37,14 @@ __global__ void k_fill_ghosts(GridDev g, E* __restrict__ W, const DevState* ds, 
             i = k < NG ? k : g.nx + k;
         }
     }
-    bool fxn = false, fxa = false, fyn = false, fya = false;
-    const double t = ds ? ds->t + toff * ds->dt : 0.0;
-    const double xc = g.ox + (i - NG + 0.5) * g.dx, yc = g.oy + (j - NG + 0.5) * g.dy;
-    int sj = j;
-    if (g.dim == 2 && (j < NG || j >= NG + g.ny)) {
-        const int by = g.bc[2 + (j >= NG + g.ny)];
-        const double* st = ghost_state(g, by, xc, yc, t);
-        if (st) {
-            for (int v = 0; v < nv; ++v)
-                W[(long long)v * g.plane + (long long)j * g.pitch + i] = (E)st[v == nv - 1 ? 3 : v];
-            return;
-        }
-        sj = ghost_src(by, g.ny, j, fyn, fya);
-    }
-    int si = i;
-    const double* sx = nullptr;  // x ghost column under an inflow rule
-    if (i < NG || i >= NG + g.nx) {
-        const int bx = g.bc[(i >= NG + g.nx)];
-        sx = ghost_state(g, bx, xc, yc, t);
-        if (!sx) si = ghost_src(bx, g.nx, i, fxn, fxa);
-    }
+    const int r0 = g.dim == 2 ? NG : 0;  // ghost rows below the interior
+    const CellSrc s = g.dim == 2 ? cell_source<true>(g, i - NG, j - NG, ds, toff)
+                                 : cell_source<false>(g, i - NG, 0, ds, toff);
     for (int v = 0; v < nv; ++v) {
-        E val = sx ? (E)sx[v == nv - 1 ? 3 : v] : W[(long long)v * g.plane + (long long)sj * g.pitch + si];
-        // x rule flips the x velocity (v=1) for symmetry, both for no-slip
-        const int vx = 1, vy = (g.dim == 2) ? 2 : -1;
-        bool neg = false;
-        if (v == vx && (fxn || fxa)) neg = !neg;
-        if (v == vy && fxa) neg = !neg;
-        if (v == vy && (fyn || fya)) neg = !neg;
-        if (v == vx && fya) neg = !neg;
-        W[(long long)v * g.plane + (long long)j * g.pitch + i] = neg ? -val : val;
+        E val = s.state ? (E)state_value(g, s.state, v)
+                        : W[(long long)v * g.plane + (long long)(s.j + r0) * g.pitch + s.i + NG];
+        if ((v == 1 && s.n1) || (v == 2 && g.dim == 2 && s.n2)) val = -val;
+        W[(long long)v * g.plane + (long long)j * g.pitch + i] = val;
     }
 }
 
@@ -89,7 +63,7 @@ __global__ void __launch_bounds__(256) k_sigma(GridDev g, const double* __restri
         for (int v = 0; v < nv; ++v) w[v] = W[(long long)v * g.plane + off];
         s = fmax(s, cell_sigma<T>(w, g.dim, (T)g.gamma, (T)g.mu, (T)h, err));
     }
-    block_commit<256, T>(s, true, err, 0u, ds);
+    block_commit<256, T>(s, true, err, 0u, ds, false);
 }
 
 // float32 shadow of a float64 array (same layout)
@@ -110,23 +84,10 @@ __global__ void k_accumulator(const double* __restrict__ W, const float* __restr
     for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) A[i] = W[i] - (double)inc[i];
 }
 
-// After the last kernel of a step: advance t by dt, pick the next dt
-// (CFL from the reduced sigma, clipped to t_end), detect completion.
-// init = 1: only pick dt from sigma (before the first step).
-__global__ void k_commit(DevState* ds, int init)
+// the first dt of a call, from k_sigma's rate
+__global__ void k_commit(DevState* ds)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    if (ds->done) return;
-    if (!init) {
-        ds->t += ds->dt;
-        ds->steps += 1;
-    }
-    const double sig = __longlong_as_double((long long)ds->sigma);
-    ds->sigma = 0ull;
-    double dt = ds->fixed_dt ? ds->dt : ds->cfl / sig;
-    if (ds->t + dt > ds->t_end) dt = ds->t_end - ds->t;
-    ds->dt = dt;
-    if (!(ds->t < ds->t_end) || (ds->max_steps > 0 && ds->steps >= ds->max_steps)) ds->done = 1u;
+    if (threadIdx.x == 0 && blockIdx.x == 0) commit_step(ds, true);
 }
 
 }  // namespace gks

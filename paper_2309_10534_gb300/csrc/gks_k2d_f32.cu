@@ -9,7 +9,7 @@ cudaError_t launch_one(const GridDev& g, const SweepArgs& a, const FluxParams<fl
                        const TenoParams& tt, DevState* ds, cudaStream_t st)
 {
     constexpr int TN = SWEEP_TN, TT = SWEEP_TT32;
-    auto kern = k2d_sweep<float, NONEQ, PRFIX, TN, TT, REC>;
+    auto kern = k2d_sweep<float, NONEQ, PRFIX, TN, TT, TT * (TN + 1), 2, REC>;
     const size_t smem = sizeof(SweepSmem<float, TN, TT, rec_conventional(REC)>);
     dim3 grid((a.nn + TN - 1) / TN, (a.nt + TT - 1) / TT);
     kern<<<grid, TT * (TN + 1), smem, st>>>(g, a, fp, teno_t<float>(tn), teno_t<float>(tt), ds);
@@ -18,7 +18,7 @@ cudaError_t launch_one(const GridDev& g, const SweepArgs& a, const FluxParams<fl
 template <bool NONEQ, bool PRFIX, int REC>
 cudaError_t set_smem()
 {
-    return cudaFuncSetAttribute(k2d_sweep<float, NONEQ, PRFIX, SWEEP_TN, SWEEP_TT32, REC>,
+    return cudaFuncSetAttribute(k2d_sweep<float, NONEQ, PRFIX, SWEEP_TN, SWEEP_TT32, SWEEP_TT32 * (SWEEP_TN + 1), 2, REC>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sizeof(SweepSmem<float, SWEEP_TN, SWEEP_TT32, rec_conventional(REC)>));
 }

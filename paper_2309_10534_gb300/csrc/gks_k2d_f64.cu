@@ -9,7 +9,7 @@ cudaError_t launch_one(const GridDev& g, const SweepArgs& a, const FluxParams<do
                        const TenoParams& tt, DevState* ds, cudaStream_t st)
 {
     constexpr int TN = SWEEP_TN, TT = SWEEP_TT64;
-    auto kern = k2d_sweep<double, NONEQ, PRFIX, TN, TT, REC>;
+    auto kern = k2d_sweep<double, NONEQ, PRFIX, TN, TT, TT * (TN + 1), 1, REC>;
     const size_t smem = sizeof(SweepSmem<double, TN, TT, rec_conventional(REC)>);
     dim3 grid((a.nn + TN - 1) / TN, (a.nt + TT - 1) / TT);
     kern<<<grid, TT * (TN + 1), smem, st>>>(g, a, fp, teno_t<double>(tn), teno_t<double>(tt), ds);
@@ -18,7 +18,7 @@ cudaError_t launch_one(const GridDev& g, const SweepArgs& a, const FluxParams<do
 template <bool NONEQ, bool PRFIX, int REC>
 cudaError_t set_smem()
 {
-    return cudaFuncSetAttribute(k2d_sweep<double, NONEQ, PRFIX, SWEEP_TN, SWEEP_TT64, REC>,
+    return cudaFuncSetAttribute(k2d_sweep<double, NONEQ, PRFIX, SWEEP_TN, SWEEP_TT64, SWEEP_TT64 * (SWEEP_TN + 1), 1, REC>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sizeof(SweepSmem<double, SWEEP_TN, SWEEP_TT64, rec_conventional(REC)>));
 }

@@ -7,9 +7,11 @@
 //   W  -- the state W^n (and W^{n+1} after stage 2)
 //   Ws -- the stage state W*
 //   Ac -- the stage accumulator W^n - dt/dx d(F + dt/6 dF)   (Sec. 2.2)
-// Kernels of one step (2-D): ghost(W), sweep-x s1, sweep-y s1, ghost(Ws),
-// sweep-x s2, sweep-y s2 (+ CFL reduction), commit.  1-D: ghost, stage 1,
-// ghost, stage 2, commit.  A sweep computes every face flux of its tile
+// Kernels of one step (2-D): sweep-x s1, sweep-y s1, sweep-x s2, sweep-y s2
+// (+ CFL reduction and commit).  1-D: stage 1, stage 2 (the same).  The blocks
+// at the boundary load their ghost cells by the boundary rules, and the last
+// block of a step's last kernel commits the step: four (two) launches a step
+// instead of seven (five).  A sweep computes every face flux of its tile
 // once, in shared memory, so both neighbours of a face apply bit-identical
 // values and the update is conservative.
 #pragma once
@@ -29,7 +31,7 @@ struct DevState {
     unsigned int err;              // bit 0 non-physical update, bit 1 fallback failed
     unsigned int done;             // 1: t_end or max_steps reached; kernels return early
     unsigned int fixed_dt;         // 1: keep dt (caller-given), 0: CFL time step
-    unsigned int pad;
+    unsigned int ticket;           // blocks of a committing kernel that have finished
 };
 
 // state-setting boundary rules: conserved states (energy in slot 3) and the
@@ -51,14 +53,17 @@ struct GridDev {
 
 constexpr int BC_INFLOW = 5, BC_WALL_AFTER_X0 = 6, BC_MOVING_SHOCK = 7;
 
-// the state a state-setting rule gives the ghost centred at (x, y) at time t,
-// or nullptr where the rule copies from the interior
-__device__ __forceinline__ const double* ghost_state(const GridDev& g, int bc, double x, double y, double t)
+// the state a state-setting rule gives the ghost at interior coordinates
+// (i, j): 1 the inflow state, 2 the pre-shock state, 0 where the rule copies
+// from the interior.  The array's time is t + toff dt (0 for W, 1/2 for W*).
+__device__ __forceinline__ int ghost_state(const GridDev& g, int bc, int i, int j, const DevState* ds, double toff)
 {
-    if (bc == BC_INFLOW) return g.bs.in;
-    if (bc == BC_WALL_AFTER_X0) return (x < g.bs.x0) ? g.bs.in : nullptr;
-    if (bc == BC_MOVING_SHOCK) return (x < g.bs.x0 + (y - g.oy) * g.bs.cot + g.bs.vx * t) ? g.bs.in : g.bs.pre;
-    return nullptr;
+    if (bc < BC_INFLOW) return 0;
+    if (bc == BC_INFLOW) return 1;
+    const double x = g.ox + (i + 0.5) * g.dx;
+    if (bc == BC_WALL_AFTER_X0) return (x < g.bs.x0) ? 1 : 0;
+    const double y = g.oy + (j + 0.5) * g.dy, t = ds ? ds->t + toff * ds->dt : 0.0;
+    return (x < g.bs.x0 + (y - g.oy) * g.bs.cot + g.bs.vx * t) ? 1 : 2;
 }
 
 // ------------------------------------------------------------------ ghosts
@@ -81,6 +86,64 @@ __device__ __forceinline__ int ghost_src(int bc, int n, int g, bool& flip_n, boo
         flip_n = true;
         return low ? 2 * NG - 1 - g : 2 * (NG + n) - 1 - g;
     }
+}
+
+// Where the value of cell (i, j) (interior coordinates, -3 .. n + 2) comes
+// from: a prescribed state, or an interior cell with the momenta's signs.  A
+// y ghost row takes the y rule to pick an interior row, then an x ghost
+// column the x rule (the same values as filling x first, then y over the full
+// ghosted width).
+struct CellSrc {
+    int i, j;     // the interior cell copied
+    int state;    // 0 copy, 1 inflow, 2 pre-shock state
+    bool n1, n2;  // momentum 1 / 2 negated
+};
+template <bool D2>
+__device__ __forceinline__ CellSrc cell_source(const GridDev& g, int i, int j, const DevState* ds, double toff)
+{
+    CellSrc s{i, j, 0, false, false};
+    bool fn, fa;
+    if (D2 && (j < 0 || j >= g.ny)) {
+        const int by = g.bc[j >= g.ny ? 3 : 2];
+        s.state = ghost_state(g, by, i, j, ds, toff);
+        if (s.state) return s;
+        s.j = ghost_src(by, g.ny, j + NG, fn, fa) - NG;
+        s.n1 = fa;
+        s.n2 = fn || fa;
+    }
+    if (i < 0 || i >= g.nx) {
+        const int bx = g.bc[i >= g.nx ? 1 : 0];
+        s.state = ghost_state(g, bx, i, j, ds, toff);
+        if (s.state) return s;
+        s.i = ghost_src(bx, g.nx, i + NG, fn, fa) - NG;
+        s.n1 ^= fn || fa;
+        s.n2 ^= fa;
+    }
+    return s;
+}
+// component v of a prescribed state
+__device__ __forceinline__ double state_value(const GridDev& g, int state, int v)
+{
+    const int k = (v == g.dim + 1) ? 3 : v;
+    return state == 1 ? g.bs.in[k] : g.bs.pre[k];
+}
+
+// ------------------------------------------------------------------ commit
+// After the last kernel of a step: advance t by dt, pick the next dt
+// (CFL from the reduced sigma, clipped to t_end), detect completion.
+// init: only pick dt from sigma (before the first step).
+__device__ __forceinline__ void commit_step(DevState* ds, bool init)
+{
+    if (ds->done) return;
+    if (!init) {
+        ds->t += ds->dt;
+        ds->steps += 1;
+    }
+    const double sig = __longlong_as_double((long long)atomicExch(&ds->sigma, 0ull));
+    double dt = ds->fixed_dt ? ds->dt : ds->cfl / sig;
+    if (ds->t + dt > ds->t_end) dt = ds->t_end - ds->t;
+    ds->dt = dt;
+    if (!(ds->t < ds->t_end) || (ds->max_steps > 0 && ds->steps >= ds->max_steps)) ds->done = 1u;
 }
 
 // ------------------------------------------------------------------ CFL rate
@@ -132,9 +195,11 @@ __device__ __forceinline__ T cell_sigma(const WT* w, int dim, T gamma, T mu, T h
 }
 
 // Block reduction of the CFL rate (only when with_sigma), the error word and
-// the fallback count; one atomic of each per block.
+// the fallback count; one atomic of each per block.  commit: the last block
+// to get here commits the step (every block has read dt and done by then).
 template <int NT, typename T>
-__device__ __forceinline__ void block_commit(T s, bool with_sigma, unsigned int err, unsigned int nfb, DevState* ds)
+__device__ __forceinline__ void block_commit(T s, bool with_sigma, unsigned int err, unsigned int nfb, DevState* ds,
+                                             bool commit)
 {
     __shared__ T red_s[NT / 32];
     __shared__ unsigned int red_e[NT / 32], red_f[NT / 32];
@@ -158,6 +223,14 @@ __device__ __forceinline__ void block_commit(T s, bool with_sigma, unsigned int 
             atomicMax(&ds->sigma, (unsigned long long)__double_as_longlong(sd));
         if (err) atomicOr(&ds->err, err);
         if (nfb) atomicAdd(&ds->fallbacks, (unsigned long long)nfb);
+        if (commit) {
+            __threadfence();  // this block's rate before its ticket
+            if (atomicAdd(&ds->ticket, 1u) + 1u == gridDim.x * gridDim.y) {
+                __threadfence();
+                ds->ticket = 0;
+                commit_step(ds, false);
+            }
+        }
     }
 }
 
@@ -194,9 +267,9 @@ __device__ __forceinline__ double wnew32(double w, float inc, float cx, float dG
 // float32 increment dt/dx d(F + dt/6 dF); the only float64 arithmetic is the
 // final update W^{n+1} = W^n - (increment + dt/dx d(dt/3 dF*)).
 struct Stage1DArgs {
-    const double* src;   // float64 reconstruction input (W; float64 path stage 2: W*), ghosts filled
+    const double* src;   // float64 reconstruction input (W; float64 path stage 2: W*)
     const float* srcf;   // float32 path: stage 1 the float32 shadow of W (or nullptr: src,
-                         // converted), stage 2 W* (float32); ghosts filled
+                         // converted), stage 2 W* (float32)
     double* out0;        // float64 path stage 1: W*; stage 2: the new state
     double* out1;        // float64 path stage 1: accumulator A
     const double* acc;   // float64 path stage 2: accumulator A
@@ -207,12 +280,31 @@ struct Stage1DArgs {
     const double* base;  // float32 path stage 2: W^n
     int stage;
     int with_sigma;      // stage 2: reduce the CFL rate of the new state
+    int commit;          // the last block commits the step
     double idx;          // 1 / dx
 };
 
+// cells i0 - 3 .. i0 + TN + 2 of a block at an end of the grid, ghosts by the
+// boundary rules (out of line: the other blocks keep their registers)
+template <typename T, int TN, typename E>
+__device__ __noinline__ void load_edge_1d(T* sq, const E* src, const GridDev& g, int i0, const DevState* ds, int stage)
+{
+    const int pl = (int)g.plane;
+    for (int k = threadIdx.x; k < 3 * (TN + 6); k += blockDim.x) {
+        const int v = k / (TN + 6), i = i0 - NG + k % (TN + 6);
+        T val = T(0);
+        if (i < g.nx + NG) {  // beyond: padding
+            const CellSrc cs = cell_source<false>(g, i, 0, ds, stage == 1 ? 0.0 : 0.5);
+            val = cs.state ? (T)state_value(g, cs.state, v) : (T)src[v * pl + NG + cs.i];
+            if (v == 1 && cs.n1) val = -val;
+        }
+        sq[k] = val;
+    }
+}
+
 template <typename T, bool NONEQ, bool PRFIX, int TN, int REC = 0>
-__global__ void __launch_bounds__(TN + 2) k1d_stage(GridDev g, Stage1DArgs a, FluxParams<T> fp, TenoT<T> tn,
-                                                    DevState* ds)
+__global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ GridDev g, Stage1DArgs a,
+                                                    FluxParams<T> fp, TenoT<T> tn, DevState* ds)
 {
     if (ds->done) return;
     // TN cells per block, TN + 2 threads: the TN + 2 reconstructed cells,
@@ -235,7 +327,6 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(GridDev g, Stage1DArgs a, Fl
     __shared__ T sG[2][3][TN + 1];                     // face fluxes for the update
     const int i0 = blockIdx.x * TN;
     const int tid = threadIdx.x;
-    const int gx = g.nx + 2 * NG;
     const int slot[3] = {0, 1, 3};
 
     const int pl = (int)g.plane;  // a 1-D plane is one ghosted row
@@ -243,11 +334,15 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(GridDev g, Stage1DArgs a, Fl
     // and the converted float64 source was compiled as both, and every
     // element then paid a float64 -> float32 conversion on the slow float64
     // pipe whichever source it took
+    const bool edge = i0 < NG || i0 + TN + NG > g.nx;
     auto load = [&](auto src) {
+        if (edge) {
+            load_edge_1d<T, TN>(&sq[0][0], src, g, i0, ds, a.stage);
+            return;
+        }
         for (int k = tid; k < 3 * (TN + 6); k += NT) {
             const int v = k / (TN + 6), c = k % (TN + 6);
-            const int gi = i0 + c;  // ghosted index of cell i0 - 3 + c
-            sq[v][c] = gi < gx ? (T)src[v * pl + gi] : T(0);
+            sq[v][c] = (T)src[v * pl + i0 + c];
         }
     };
     if constexpr (sizeof(T) == 4) {
@@ -382,7 +477,7 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(GridDev g, Stage1DArgs a, Fl
             if (a.with_sigma) sig = fmax(sig, cell_sigma<T>(w, 1, s_scal[3], s_scal[4], s_scal[5], err));
         }
     }
-    if (NT % 32 == 0) block_commit<NT, T>(sig, a.with_sigma != 0, err, nfb, ds);
+    if (NT % 32 == 0) block_commit<NT, T>(sig, a.with_sigma != 0, err, nfb, ds, a.commit != 0);
 }
 
 // ------------------------------------------------------------------ 2-D sweep
@@ -398,8 +493,8 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(GridDev g, Stage1DArgs a, Fl
 //   stage 1: W*f = Wf - (inc0 + dt/dy dG1),  inc1 <- inc1 + dt/dy dG2
 //   stage 2: W   = W - (inc1 + inc0 + dt/dy dG)   (and its shadow Wf)
 struct SweepArgs {
-    const double* src;   // reconstruction input (W or W*), ghosts filled
-    const float* srcf;   // float32 path: float32 shadow of src (ghosts filled)
+    const double* src;   // reconstruction input (W or W*)
+    const float* srcf;   // float32 path: float32 shadow of src
     const float* basef;  // float32 path, y sweep of stage 1: float32 shadow of W
     const double* base;  // y sweep: W (stage 1) or A (stage 2)
     double* out0;        // y sweep, stage 1: W*; stage 2: W
@@ -414,6 +509,7 @@ struct SweepArgs {
     double ihn, iht;     // inverse cell sizes along normal / tangential
     double hmin;         // min(dx, dy) for the CFL rate
     int with_sigma;
+    int commit;          // the last block commits the step
 };
 
 // global variable index of local variable v (swap: faces normal to y)
@@ -428,15 +524,40 @@ template <typename T, int TN, int TT, bool CONV = false> struct SweepSmem {
     T w0[CONV ? 2 : 1][4][CONV ? TT + 4 : 1][CONV ? TN + 1 : 1];
 };
 
-template <typename T, bool NONEQ, bool PRFIX, int TN, int TT, int REC = 0>
-__global__ void __launch_bounds__(TT * (TN + 1), (sizeof(T) == 4) ? 1024 / (TT * (TN + 1)) : 1)
-k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, DevState* ds)
+// the cells of a tile that reaches past the boundary, ghosts by the boundary
+// rules (out of line: the other tiles keep their registers)
+template <typename T, int TN, int TT>
+__device__ __noinline__ void load_edge_2d(T* w, const GridDev& g, const SweepArgs& a, int n0, int t0,
+                                          const DevState* ds)
+{
+    constexpr int CN = TN + 6, CT = TT + 4;
+    const bool swap = a.dirn != 0;
+    for (int k = threadIdx.x; k < 4 * CN * CT; k += blockDim.x) {
+        const int v = k / (CN * CT), e = k % (CN * CT);
+        const int ct = swap ? e % CT : e / CN, cn = swap ? e / CT : e % CN;
+        const int in = n0 - NG + cn, it = t0 - 2 + ct;
+        T val = T(0);
+        if (in < a.nn + NG && it < a.nt + 2) {  // beyond: padding
+            const int gv = gvar(v, swap);
+            const CellSrc cs = cell_source<true>(g, swap ? it : in, swap ? in : it, ds, a.stage == 1 ? 0.0 : 0.5);
+            const long long off = (long long)gv * g.plane + (long long)(cs.j + NG) * g.pitch + cs.i + NG;
+            if (cs.state) val = (T)state_value(g, cs.state, gv);
+            else if constexpr (sizeof(T) == 4) val = a.srcf[off];
+            else val = a.src[off];
+            if ((gv == 1 && cs.n1) || (gv == 2 && cs.n2)) val = -val;
+        }
+        w[(v * CT + ct) * CN + cn] = val;
+    }
+}
+
+template <typename T, bool NONEQ, bool PRFIX, int TN, int TT, int NT, int MB, int REC = 0>
+__global__ void __launch_bounds__(NT, MB)
+k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, DevState* ds)
 {
     if (ds->done) return;
-    constexpr int NT = TT * (TN + 1);    // one thread per (face, row) pair
     constexpr int NF = TN + 1;           // faces per tile row
     constexpr int NP = TT * NF;          // (face, row) pairs
-    static_assert(NP == NT, "one (face,row) pair per thread");
+    constexpr int NW = NT / 32;
     constexpr bool CONV = rec_conventional(REC);
     constexpr int RB = rec_base(REC);  // the tangential (per-quantity) reconstruction
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -448,7 +569,7 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
     const bool fy = a.dirn != 0;
     auto sfi = [&](int k, int r, int f) { return fy ? (k * NF + f) * (TT + 1) + r : (k * TT + r) * NF + f; };
 
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // the stage's scalars in the arithmetic type, converted once per block
     // (a float64 -> float32 conversion runs on the slow float64 pipe):
     // dt, dt/h_n, 1/h_n, 1/h_t, gamma, mu, min(h_n, h_t); visible after the
@@ -465,6 +586,7 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
         s_scal[6] = (T)a.hmin;
     }
     const int n0 = blockIdx.x * TN, t0 = blockIdx.y * TT;
+    static_assert(TN == 31, "lanes of a warp along the tile's faces");
     // local frame: normal momentum first; y faces swap the two momentum components
     const bool swap = a.dirn != 0;
     // offsets within one variable plane fit in 32 bits; each variable's plane
@@ -475,22 +597,23 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
     const long long pv3 = 3 * g.plane;
 
     // load cells (normal n0-3 .. n0+TN+2, tangential t0-2 .. t0+TT+1); the
-    // thread index runs fastest along the unit-stride direction
+    // thread index runs fastest along the unit-stride direction; tiles that
+    // reach past the boundary take their ghosts by the boundary rules
     {
-        constexpr int CN = TN + 6, CT = TT + 4, NCELL = CN * CT;
-        for (int k = tid; k < 4 * NCELL; k += NT) {
-            const int v = k / NCELL, e = k % NCELL;
-            int cn, ct;
-            if (a.dirn == 0) { ct = e / CN; cn = e % CN; } else { cn = e / CT; ct = e % CT; }
-            const int in = n0 - 3 + cn, it = t0 - 2 + ct;
-            T val = T(0);
-            if (in < a.nn + 3 && it < a.nt + 2) {  // ghosted extent (negative side is covered by ghosts)
-                const long long pv = v == 0 ? 0 : (v == 1 ? pv1 : (v == 2 ? pv2 : pv3));
-                const int off = org + in * sn + it * st;
-                if constexpr (sizeof(T) == 4) val = (a.srcf + pv)[off];
-                else val = (a.src + pv)[off];
-            }
-            sm.w[v][ct][cn] = val;
+        constexpr int CN = TN + 6, CT = TT + 4;
+        const bool edge = n0 < NG || n0 + TN + NG > a.nn || t0 < 2 || t0 + TT + 2 > a.nt;
+        const T* base;
+        if constexpr (sizeof(T) == 4) base = a.srcf + (org + (n0 - NG) * sn + (t0 - 2) * st);
+        else base = a.src + (org + (n0 - NG) * sn + (t0 - 2) * st);
+        auto cell = [&](int v, int cn, int ct) {
+            const long long pv = v == 0 ? 0 : (v == 1 ? pv1 : (v == 2 ? pv2 : pv3));
+            sm.w[v][ct][cn] = (base + pv)[cn * sn + ct * st];
+        };
+        if (edge) load_edge_2d<T, TN, TT>(&sm.w[0][0][0], g, a, n0, t0, ds);
+        else for (int k = tid; k < 4 * CN * CT; k += NT) {
+            const int v = k / (CN * CT), e = k % (CN * CT);
+            if (!fy) cell(v, e % CN, e / CN);
+            else cell(v, e / CT, e % CT);
         }
     }
     __syncthreads();
@@ -522,10 +645,14 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
     } else if constexpr (sizeof(T) == 4 && REC <= 1) {
         // float32 TENO-D / WENO5-AO: variables (0, 1) and (2, 3) as packed pairs
         const float ih = s_scal[2];
-        constexpr int NC = TN + 2, NR = TT + 4;
-        for (int k = tid; k < 2 * NC * NR; k += NT) {
-            const int vv = 2 * (k / (NC * NR)), e = k % (NC * NR);
-            const int r = e / NC, c = e % NC;
+        // a warp takes one (row, pair): cells 0..31 along the lanes; the 33rd
+        // cells of all rows come last, one per lane
+        constexpr int NL = 2 * (TT + 4);
+        for (int k = warp; k < NL + (NL + 31) / 32; k += NW) {
+            const bool line = k < NL;
+            const int e = line ? k : (k - NL) * 32 + lane, c = line ? lane : 32;
+            if (e >= NL) continue;
+            const int vv = 2 * (e & 1), r = e >> 1;
             f2 q[5];
 #pragma unroll
             for (int s = 0; s < 5; ++s) q[s] = f2(sm.w[vv][r][c + s], sm.w[vv + 1][r][c + s]);
@@ -543,10 +670,12 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
         }
     } else {
         const T ih = s_scal[2];
-        constexpr int NC = TN + 2, NR = TT + 4;
-        for (int k = tid; k < 4 * NC * NR; k += NT) {
-            const int v = k / (NC * NR), e = k % (NC * NR);
-            const int r = e / NC, c = e % NC;
+        constexpr int NL = 4 * (TT + 4);  // (row, variable) lines, as above
+        for (int k = warp; k < NL + (NL + 31) / 32; k += NW) {
+            const bool line = k < NL;
+            const int e = line ? k : (k - NL) * 32 + lane, c = line ? lane : 32;
+            if (e >= NL) continue;
+            const int v = e & 3, r = e >> 2;
             T q[5];
 #pragma unroll
             for (int s = 0; s < 5; ++s) q[s] = sm.w[v][r][c + s];
@@ -605,7 +734,7 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
     const T iht = s_scal[3];
     const T gA = T(-0.28867513459481288), gB = T(0.28867513459481288);  // -+1/(2 sqrt 3)
 #pragma unroll 1
-    for (int task = tid; task < 2 * NP; task += NT) {
+    for (int task = tid; task < 2 * NP; task += NT) {  // 2 NP is a multiple of NT: whole warps
         const int pair = task >> 1, gpi = task & 1;
         const int r = pair / NF, f = pair % NF;
         // faces n0+f <= nn on rows t0+r < nt exist; the rest of the tile is padding
@@ -714,9 +843,11 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
     // phase 3: flux divergence; the y sweep updates the float64 state
     T sig = T(0);
     const T cn = s_scal[1];
-    if (tid < TN * TT) {
+    static_assert((2 * NP) % NT == 0, "whole warps of tasks");
+#pragma unroll 1
+    for (int k = tid; k < TN * TT; k += NT) {
         // x faces: the normal (x) index fastest; y faces: the tangential (x) index
-        const int r = fy ? tid % TT : tid / TN, c = fy ? tid / TT : tid % TN;
+        const int r = fy ? k % TT : k / TN, c = fy ? k / TT : k % TN;
         const int in = n0 + c, it = t0 + r;
         if (in < a.nn && it < a.nt) {
             const int o = org + in * sn + it * st;
@@ -755,12 +886,12 @@ k2d_sweep(GridDev g, SweepArgs a, FluxParams<T> fp, TenoT<T> tnn, TenoT<T> tnt, 
                 }
             }
             if (a.with_sigma) {
-                if constexpr (sizeof(T) == 4) sig = cell_sigma<T, T>(wf, 2, s_scal[4], s_scal[5], s_scal[6], err);
-                else sig = cell_sigma<T>(wn, 2, s_scal[4], s_scal[5], s_scal[6], err);
+                if constexpr (sizeof(T) == 4) sig = fmax(sig, cell_sigma<T, T>(wf, 2, s_scal[4], s_scal[5], s_scal[6], err));
+                else sig = fmax(sig, cell_sigma<T>(wn, 2, s_scal[4], s_scal[5], s_scal[6], err));
             }
         }
     }
-    block_commit<NT, T>(sig, a.with_sigma != 0, err, nfb, ds);
+    block_commit<NT, T>(sig, a.with_sigma != 0, err, nfb, ds, a.commit != 0);
 }
 
 }  // namespace gks

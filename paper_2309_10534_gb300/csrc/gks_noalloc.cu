@@ -98,23 +98,9 @@ cudaError_t scratch_address(double** out)
     return cudaSuccess;
 }
 
-// ghost source along a line of n interior cells (same rules as the library's
-// ghost fill): periodic, zero gradient, mirror (velocity negated)
-__device__ int ghost_source(int bc, int n, int g, bool& flip)
-{
-    flip = false;
-    if (g >= NG && g < NG + n) return g;
-    const bool low = g < NG;
-    if (bc == GKS_BC_PERIODIC) return NG + (((g - NG) % n) + n) % n;
-    if (bc == GKS_BC_ZEROGRAD) return low ? NG : NG + n - 1;
-    flip = true;  // symmetry, reflect, no-slip: 1-D velocity negated
-    return low ? 2 * NG - 1 - g : 2 * (NG + n) - 1 - g;
-}
-
-// copy the caller's interior [3][nx] into the ghosted scratch row, fill the
-// ghosts, and reset the step state (everything that must start at zero)
-__global__ void k_load(const double* __restrict__ Win, double* __restrict__ W, int nx, int bc0, int bc1,
-                       DevState* ds, double dt)
+// copy the caller's interior [3][nx] into the scratch row and reset the step
+// state (everything that must start at zero)
+__global__ void k_load(const double* __restrict__ Win, double* __restrict__ W, int nx, DevState* ds, double dt)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {
@@ -123,27 +109,8 @@ __global__ void k_load(const double* __restrict__ Win, double* __restrict__ W, i
         ds->fixed_dt = 1u;
         ds->t_end = INFINITY;
     }
-    if (i >= nx + 2 * NG) return;
-    bool flip;
-    const int src = ghost_source(i < NG ? bc0 : bc1, nx, i, flip);
-    for (int v = 0; v < 3; ++v) {
-        const double val = Win[(long long)v * nx + (src - NG)];
-        W[(long long)v * PITCH + i] = (flip && v == 1) ? -val : val;
-    }
-}
-
-template <typename E>
-__global__ void k_ghosts(E* __restrict__ W, int nx, int bc0, int bc1)
-{
-    const int k = threadIdx.x;
-    if (k >= 2 * NG) return;
-    const int i = k < NG ? k : nx + k;
-    bool flip;
-    const int src = ghost_source(k < NG ? bc0 : bc1, nx, i, flip);
-    for (int v = 0; v < 3; ++v) {
-        const E val = W[(long long)v * PITCH + src];
-        W[(long long)v * PITCH + i] = (flip && v == 1) ? -val : val;
-    }
+    if (i >= nx) return;
+    for (int v = 0; v < 3; ++v) W[(long long)v * PITCH + NG + i] = Win[(long long)v * nx + i];
 }
 
 __global__ void k_store(const double* __restrict__ W, double* __restrict__ Wout, int nx)
@@ -217,7 +184,7 @@ extern "C" gks_status gks_step1d_noalloc(const double* W_in, double* W_out, int 
     // the same scratch regions
     float* Wsf = reinterpret_cast<float*>(Ws);
     float* incf = reinterpret_cast<float*>(Ac);
-    k_load<<<(nx + 2 * NG + 127) / 128, 128, 0, st>>>(W_in, W, nx, bc[0], bc[1], ds, dt);
+    k_load<<<(nx + 127) / 128, 128, 0, st>>>(W_in, W, nx, ds, dt);
     Stage1DArgs a1{};
     a1.idx = 1.0 / dx;
     a1.src = W;
@@ -225,8 +192,6 @@ extern "C" gks_status gks_step1d_noalloc(const double* W_in, double* W_out, int 
     else { a1.out0 = Ws; a1.out1 = Ac; }
     a1.stage = 1;
     if (launch_stage1d(f32, g, a1, hf, tn, ds, st) != cudaSuccess) return GKS_ECUDA;
-    if (f32) k_ghosts<float><<<1, 32, 0, st>>>(Wsf, nx, bc[0], bc[1]);
-    else k_ghosts<double><<<1, 32, 0, st>>>(Ws, nx, bc[0], bc[1]);
     Stage1DArgs a2{};
     a2.idx = 1.0 / dx;
     if (f32) { a2.srcf = Wsf; a2.base = W; a2.accf = incf; }
