@@ -545,8 +545,8 @@ GKS_HD void point_flux_vjp(const Side<T>& L, const Side<T>& R, const FluxParams<
     Prim<T> pl, pr;
     prim_state<T, 2>(L.W, P.gm1, pl);
     prim_state<T, 2>(R.W, P.gm1, pr);
-    side_terms<true, T, 2, false, false>(L, pl, P, W0, W0n, W0t, d4, d5, d6, d7, d8);
-    side_terms<false, T, 2, false, false>(R, pr, P, W0, W0n, W0t, d4, d5, d6, d7, d8);
+    side_terms<true, false, T, 2, false, false>(L, pl, P, W0, W0n, W0t, d4, d5, d6, d7, d8);
+    side_terms<false, true, T, 2, false, false>(R, pr, P, W0, W0n, W0t, d4, d5, d6, d7, d8);
     T gW0[4] = {T(0), T(0), T(0), T(0)}, gW0n[4] = {T(0), T(0), T(0), T(0)}, gW0t[4] = {T(0), T(0), T(0), T(0)};
     equilibrium_vjp(W0, W0n, W0t, P.gm1, gF, gdF, gW0, gW0n, gW0t);
     side_vjp(L, true, P, gW0, gW0n, gW0t, gL);

@@ -1187,13 +1187,12 @@ GKS_HD void merge_values(const T* Wl, const T* Wr, const FluxParams<T>& P, T* W0
 }
 
 // One side's contributions to the equilibrium state (kinetic merge,
-// Eqs. 2.6, 3.25, 3.26) and to the non-equilibrium terms of Eq. (2.5); the
-// left side (u > 0) sets the sums, the right side (u < 0) adds to them.
-template <bool UPPER, typename T, int DIM, bool NONEQ, bool PRFIX>
+// Eqs. 2.6, 3.25, 3.26) and to the non-equilibrium terms of Eq. (2.5): the
+// left side (UPPER, u > 0) or the right one; ADD to the sums, or set them.
+template <bool UPPER, bool ADD, typename T, int DIM, bool NONEQ, bool PRFIX>
 GKS_HD void side_terms(const Side<T>& S, const Prim<T>& pr, const FluxParams<T>& P, T* W0, T* W0n, T* W0t, T* S3, T* S4, T* S5, T* N4,
                        T* N5)
 {
-    constexpr bool ADD = !UPPER;
     const T r = pr.r, U = pr.U, V = pr.V, q = pr.q, hv2 = pr.hv2;
     const T th = pr.p * pr.ir;               // 1/(2 lambda)
     const T sl = M<T>::rsqrt_(T(2) * th);    // sqrt(lambda)
@@ -1258,6 +1257,70 @@ GKS_HD void side_terms(const Side<T>& S, const Prim<T>& pr, const FluxParams<T>&
     }
 }
 
+// The equilibrium state g0: rho0 <u psi>_0 (F0) is the Euler flux of W0,
+// rho0 <u A0 psi>_0 (F2) its time derivative, and rho0 <u (a0n u + a0t v)
+// psi>_0 (F1) is d_n rho0 <u^2 psi>_0 + d_t rho0 <u v psi>_0
+template <typename T> struct Equilibrium {
+    T U, V, q, p;   // velocities, |U|^2/2, pressure
+    Grad<T> g;      // time slopes
+    T F0[4], F1[4], F2[4];
+};
+template <typename T, int DIM, bool NONEQ>
+GKS_HD void equilibrium(const T* W0, const T* W0n, const T* W0t, const FluxParams<T>& P, Equilibrium<T>& E)
+{
+    const T r0 = W0[0], ir0 = T(1) / r0;
+    const T U0 = W0[1] * ir0;
+    const T V0 = (DIM == 2) ? W0[2] * ir0 : T(0);
+    const T hv2 = (DIM == 2) ? T(0.5) * V0 * V0 : T(0);
+    const T q0 = fma(T(0.5) * U0, U0, hv2);
+    const T p0 = P.gm1 * fma(-r0, q0, W0[3]);
+    const T Ep = W0[3] + p0, th0 = p0 * ir0;
+    E.U = U0;
+    E.V = V0;
+    E.q = q0;
+    E.p = p0;
+    Grad<T> n, t;
+    Grad<T>& g = E.g;
+    prim_slope<T, DIM>(W0n, U0, V0, q0, th0, P.gm1, n);
+    if constexpr (DIM == 2) prim_slope<T, DIM>(W0t, U0, V0, q0, th0, P.gm1, t);
+    time_slope<T, DIM>(n, t, U0, V0, th0, P.gm1, g);
+    E.F0[0] = W0[1];
+    E.F0[1] = fma(W0[1], U0, p0);
+    E.F0[2] = (DIM == 2) ? W0[1] * V0 : T(0);
+    E.F0[3] = U0 * Ep;
+    const T mt = fma(U0, g.r, g.mU);  // d(rho U)
+    E.F2[0] = mt;
+    E.F2[1] = fma(U0, mt + g.mU, g.p);
+    E.F2[2] = (DIM == 2) ? fma(V0, mt, U0 * g.mV) : T(0);
+    // rho U H: H d(rho U) + U rho dH, rho dH = U rho dU + V rho dV + cp rho dth
+    T rdH = fma(U0, g.mU, P.cp * g.mT);
+    if constexpr (DIM == 2) rdH = fma(V0, g.mV, rdH);
+    E.F2[3] = fma(Ep * ir0, mt, U0 * rdH);
+    if constexpr (NONEQ) {
+        UMom<T> m;
+        m.u0 = T(1);
+        m.u1 = U0;
+        u_moments(m, U0, th0, true);
+        const T e = fma(P.hkv, th0, hv2);
+        const T kn = kappa<DIM>(V0, n, P.hkv);
+        d_mom<false, T, DIM>(E.F1, d_u2(m, n), d_u3(m, n), d_u4(m, n), m.u2, V0, e, n.mV, kn);
+        if constexpr (DIM == 2)
+            d_cross<T>(E.F1, fma(t.r, U0, t.mU), d_u2(m, t), d_u3(m, t), U0, m.u2, m.u3, V0, th0, e, t.mV, t.mT,
+                       kappa<DIM>(V0, t, P.hkv));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) E.F1[i] = T(0);
+    }
+}
+
+// collision time over dt (Sec. 5), from the sides' pressures and p0
+template <typename T>
+GKS_HD T tau_over_dt(const FluxParams<T>& P, T pl, T pr, T p0, T idt)
+{
+    const T jump = fabs(pl - pr) / (pl + pr);
+    return (P.tau_mode == 1) ? P.c1 + P.c2 * jump : P.mu * idt / p0 + P.c2 * jump;
+}
+
 // F and dF/dt (per unit time; Sec. 2.2) at one interface point in the local
 // frame.  state(0, L, p) and state(1, R, p) form a side's primitive variables
 // (prim_state) and apply the caller's fallback where it is not physical.
@@ -1274,8 +1337,8 @@ GKS_HD void point_flux(Side<T>& L, Side<T>& R, const FluxParams<T>& P, T* F, T* 
     Prim<T> pl, pr;
     state(0, L, pl);
     state(1, R, pr);
-    side_terms<true, T, DIM, NONEQ, PRFIX>(L, pl, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
-    side_terms<false, T, DIM, NONEQ, PRFIX>(R, pr, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
+    side_terms<true, false, T, DIM, NONEQ, PRFIX>(L, pl, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
+    side_terms<false, true, T, DIM, NONEQ, PRFIX>(R, pr, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
     // the kinetic merge is also the density moment of the side terms (the
     // heat flux needs it even where W0 is replaced below)
     T W0k[4];
@@ -1304,34 +1367,9 @@ GKS_HD void point_flux(Side<T>& L, Side<T>& R, const FluxParams<T>& P, T* F, T* 
         for (int i = 0; i < 4; ++i) W0t[i] = W0t_lin[i];
     }
 
-    // equilibrium state g0: rho0 <u psi>_0 is the Euler flux of W0 and
-    // rho0 <u A0 psi>_0 its time derivative
-    const T r0 = W0[0], ir0 = T(1) / r0;
-    const T U0 = W0[1] * ir0;
-    const T V0 = (DIM == 2) ? W0[2] * ir0 : T(0);
-    const T hv2 = (DIM == 2) ? T(0.5) * V0 * V0 : T(0);
-    const T q0 = fma(T(0.5) * U0, U0, hv2);
-    const T p0 = P.gm1 * fma(-r0, q0, W0[3]);
-    const T Ep = W0[3] + p0, th0 = p0 * ir0;
-    Grad<T> n, t, g;
-    prim_slope<T, DIM>(W0n, U0, V0, q0, th0, P.gm1, n);
-    if constexpr (DIM == 2) prim_slope<T, DIM>(W0t, U0, V0, q0, th0, P.gm1, t);
-    time_slope<T, DIM>(n, t, U0, V0, th0, P.gm1, g);
-    T F0[4], F2[4];
-    F0[0] = W0[1];
-    F0[1] = fma(W0[1], U0, p0);
-    F0[2] = (DIM == 2) ? W0[1] * V0 : T(0);
-    F0[3] = U0 * Ep;
-    {
-        const T mt = fma(U0, g.r, g.mU);  // d(rho U)
-        F2[0] = mt;
-        F2[1] = fma(U0, mt + g.mU, g.p);
-        F2[2] = (DIM == 2) ? fma(V0, mt, U0 * g.mV) : T(0);
-        // rho U H: H d(rho U) + U rho dH, rho dH = U rho dU + V rho dV + cp rho dth
-        T rdH = fma(U0, g.mU, P.cp * g.mT);
-        if constexpr (DIM == 2) rdH = fma(V0, g.mV, rdH);
-        F2[3] = fma(Ep * ir0, mt, U0 * rdH);
-    }
+    Equilibrium<T> E;
+    equilibrium<T, DIM, NONEQ>(W0, W0n, W0t, P, E);
+    const T *F0 = E.F0, *F1 = E.F1, *F2 = E.F2;
 
     if (P.tau_mode == 0) {
 #pragma unroll
@@ -1341,26 +1379,10 @@ GKS_HD void point_flux(Side<T>& L, Side<T>& R, const FluxParams<T>& P, T* F, T* 
         }
         return;
     }
-    // collision time and time coefficients: is = tau / dt
     T cF[6], cD[6];
-    const T jump = fabs(pl.p - pr.p) / (pl.p + pr.p);
     const T dt = P.dt, idt = T(1) / dt;
-    const T is = (P.tau_mode == 1) ? P.c1 + P.c2 * jump : P.mu * idt / p0 + P.c2 * jump;
+    const T is = tau_over_dt(P, pl.p, pr.p, E.p, idt);
     time_coeffs<T>(T(1) / is, is, cF, cD);
-
-    T F1[4] = {T(0), T(0), T(0), T(0)};  // rho0 <u (a0n u + a0t v) psi>_0 = d_n rho0 <u^2 psi>_0 + d_t rho0 <u v psi>_0
-    if constexpr (NONEQ) {
-        UMom<T> m;
-        m.u0 = T(1);
-        m.u1 = U0;
-        u_moments(m, U0, th0, true);
-        const T e = fma(P.hkv, th0, hv2);
-        const T kn = kappa<DIM>(V0, n, P.hkv);
-        d_mom<false, T, DIM>(F1, d_u2(m, n), d_u3(m, n), d_u4(m, n), m.u2, V0, e, n.mV, kn);
-        if constexpr (DIM == 2)
-            d_cross<T>(F1, fma(t.r, U0, t.mU), d_u2(m, t), d_u3(m, t), U0, m.u2, m.u3, V0, th0, e, t.mV, t.mT,
-                       kappa<DIM>(V0, t, P.hkv));
-    }
     // Prandtl correction: F_E += (1/Pr - 1) q, q the heat flux relative to
     // (U0, V0) expanded in raw moments of the same time-dependent f.
     // Density moments: rho0 <psi>_0 = W0, rho0 <(a_n u + a_t v) psi>_0 =
@@ -1368,13 +1390,15 @@ GKS_HD void point_flux(Side<T>& L, Side<T>& R, const FluxParams<T>& P, T* F, T* 
     // merge), N4, N5.
     T W0time[4] = {T(0), T(0), T(0), T(0)};
     T cf = T(0), uk = T(0);
+    const T U0 = E.U, V0 = E.V;
     if constexpr (PRFIX) {
+        const Grad<T>& g = E.g;
         W0time[0] = g.r;
         W0time[1] = g.mU + U0 * g.r;
         W0time[2] = g.mV + V0 * g.r;
-        W0time[3] = q0 * g.r + U0 * g.mU + V0 * g.mV + (P.cp - T(1)) * g.p;  // 1/(gamma - 1) = cp - 1
-        cf = q0 + U0 * U0;
-        uk = U0 * q0;
+        W0time[3] = E.q * g.r + U0 * g.mU + V0 * g.mV + (P.cp - T(1)) * g.p;  // 1/(gamma - 1) = cp - 1
+        cf = E.q + U0 * U0;
+        uk = U0 * E.q;
     }
     auto combine = [&](const T* c, T s1, T s2, T* o) {
         // q_k = c_k s1 for p_k = 1 (k = 0, 3), c_k s2 for p_k = 2

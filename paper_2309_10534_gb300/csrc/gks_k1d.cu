@@ -8,6 +8,13 @@ template <typename T, bool NONEQ, bool PRFIX, int REC>
 cudaError_t launch_one(const GridDev& g, const Stage1DArgs& a, const HostFlux& hf, const TenoParams& tn,
                        DevState* ds, cudaStream_t st)
 {
+    if constexpr (!PRFIX && REC != REC_TENO_CHAR) {
+        if (hf.merge == 0 && g.nx <= (sizeof(T) == 8 ? STAGE1D_WIDE_NX64 : STAGE1D_WIDE_NX32)) {
+            k1d_stage_wide<T, NONEQ, REC><<<(g.nx + WIDE_TN - 1) / WIDE_TN, 96, 0, st>>>(
+                g, a, make_flux_params<T>(hf), teno_t<T>(tn), ds);
+            return cudaGetLastError();
+        }
+    }
     constexpr int TN = STAGE1D_TN;
     dim3 grid((g.nx + TN - 1) / TN);
     k1d_stage<T, NONEQ, PRFIX, TN, REC><<<grid, TN + 2, 0, st>>>(g, a, make_flux_params<T>(hf), teno_t<T>(tn), ds);

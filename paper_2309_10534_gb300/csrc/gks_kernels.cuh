@@ -480,6 +480,230 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
     if (NT % 32 == 0) block_commit<NT, T>(sig, a.with_sigma != 0, err, nfb, ds, a.commit != 0);
 }
 
+// ------------------------------------------------------------------ 1-D stage, short grids
+// The same stage for grids too short to fill the chip, where a step lasts as
+// long as one warp's chain of operations (a dependent float64 operation takes
+// over 100 cycles, a float32 stage ~1500 instructions): three warps on 30
+// cells split the chain, so that no lane runs more than a third of it.
+// Phase 1: warp v reconstructs variable v.  Phase 2: warps 0 and 1 the left
+// and the right side's moments; then warp 0 the equilibrium fluxes while warp
+// 1 forms the time coefficients; then warp v combines component v.  The
+// heat-flux correction, the averaged merge and characteristic variables take
+// k1d_stage.
+constexpr int WIDE_TN = 30;
+
+template <typename T, bool NONEQ, int REC>
+__global__ void __launch_bounds__(96) k1d_stage_wide(const __grid_constant__ GridDev g, Stage1DArgs a,
+                                                     FluxParams<T> fp, TenoT<T> tn, DevState* ds)
+{
+    if (ds->done) return;
+    constexpr int TN = WIDE_TN, NS = 16;
+    __shared__ T sq[3][TN + 6];
+    __shared__ T sL[3][2][32], sR[3][2][32];  // [var][value, slope][face]
+    __shared__ T sS[2][NS][32];               // a side's W0, W0n, S3, S4, S5 (3 each), pressure
+    __shared__ T sF[3][3][32], sC[12][32];    // F0, F1, F2; time coefficients
+    __shared__ T sG[2][3][32];
+    __shared__ double s_cx;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * TN;
+    const int pl = (int)g.plane;
+    constexpr int slot[3] = {0, 1, 3};
+    const double dt = ds->dt;
+    fp.dt = (T)dt;
+    const T ih = (T)a.idx;
+    if (threadIdx.x == 0) s_cx = dt * a.idx;
+    auto load = [&](auto src) {  // warp v loads variable v
+        for (int c = lane; c < TN + 6; c += 32) {
+            const int i = i0 - NG + c;
+            T val = T(0);
+            if (i >= 0 && i < g.nx) {
+                val = (T)src[warp * pl + NG + i];
+            } else if (i < g.nx + NG) {  // a ghost; beyond: padding
+                const CellSrc cs = cell_source<false>(g, i, 0, ds, a.stage == 1 ? 0.0 : 0.5);
+                val = cs.state ? (T)state_value(g, cs.state, warp) : (T)src[warp * pl + NG + cs.i];
+                if (warp == 1 && cs.n1) val = -val;
+            }
+            sq[warp][c] = val;
+        }
+    };
+    if constexpr (sizeof(T) == 4) {
+        if (a.srcf) load(a.srcf);
+        else load(a.src);
+    } else {
+        load(a.src);
+    }
+    // the update's other inputs, ahead of their use (warp 0: cell i0 + lane)
+    const int i = i0 + lane, o = i + NG;
+    const bool own = warp == 0 && lane < TN && i < g.nx;
+    double base[3] = {0.0, 0.0, 0.0};
+    T acc[3] = {T(0), T(0), T(0)};
+    if (own) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            if constexpr (sizeof(T) == 4) {
+                if (a.stage == 2) { base[v] = a.base[v * pl + o]; acc[v] = a.accf[v * pl + o]; }
+            } else {
+                base[v] = a.stage == 1 ? a.src[v * pl + o] : a.acc[v * pl + o];
+            }
+        }
+    }
+    __syncwarp();
+    {
+        T q[5], vp, dp, vm, dm;
+#pragma unroll
+        for (int s = 0; s < 5; ++s) q[s] = sq[warp][lane + s];
+        if constexpr (sizeof(T) == 4 && REC == 0) {
+            // as recon_cell3: (rho, rho u) in the packed form, E in the scalar one
+            if (warp < 2) {
+                f2 qq[5], x, y, z, w;
+#pragma unroll
+                for (int s = 0; s < 5; ++s) qq[s] = f2(q[s]);
+                packed_faces<0>(qq, tn, x, y, z, w);
+                vp = x.x(), dp = y.x(), vm = z.x(), dm = w.x();
+            } else {
+                TenoSel<T> S;
+                teno_select(q, tn, S);
+                teno_faces(q, S, vp, dp, vm, dm);
+            }
+        } else {
+            TenoSel<T> S;
+            rec_select<REC>(q, tn, S);
+            rec_faces<REC>(q, S, vp, dp, vm, dm);
+        }
+        sL[warp][0][lane] = vp;
+        sL[warp][1][lane] = dp * ih;
+        if (lane >= 1) {
+            sR[warp][0][lane - 1] = vm;
+            sR[warp][1][lane - 1] = dm * ih;
+        }
+    }
+    __syncthreads();
+    // phase 2: face lane between interior cells i0 + lane - 1 and i0 + lane
+    const bool face = lane <= TN && i0 + lane <= g.nx;
+    unsigned int nfb = 0, err = 0;
+    if (warp < 2 && face) {
+        const int f = lane;
+        Side<T> S;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) S.W[k] = S.Wn[k] = S.Wt[k] = T(0);
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            S.W[slot[v]] = warp ? sR[v][0][f] : sL[v][0][f];
+            S.Wn[slot[v]] = warp ? sR[v][1][f] : sL[v][1][f];
+        }
+        Prim<T> p;
+        if (!prim_state<T, 1>(S.W, fp.gm1, p)) {
+#pragma unroll
+            for (int v = 0; v < 3; ++v) { S.W[slot[v]] = sq[v][f + 2 + warp]; S.Wn[slot[v]] = T(0); }
+            ++nfb;
+            if (!prim_state<T, 1>(S.W, fp.gm1, p)) err |= 2u;
+        }
+        T W0[4], W0n[4], W0t[4], S3[4], S4[4], S5[4];
+        if (warp == 0) side_terms<true, false, T, 1, NONEQ, false>(S, p, fp, W0, W0n, W0t, S3, S4, S5, nullptr, nullptr);
+        else side_terms<false, false, T, 1, NONEQ, false>(S, p, fp, W0, W0n, W0t, S3, S4, S5, nullptr, nullptr);
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            sS[warp][v][f] = W0[slot[v]];
+            sS[warp][3 + v][f] = W0n[slot[v]];
+            if constexpr (NONEQ) {
+                sS[warp][6 + v][f] = S3[slot[v]];
+                sS[warp][9 + v][f] = S4[slot[v]];
+                sS[warp][12 + v][f] = S5[slot[v]];
+            }
+        }
+        sS[warp][15][f] = p.p;
+    }
+    __syncthreads();
+    if (warp < 2 && face) {
+        const int f = lane;
+        T W0[4] = {sS[0][0][f] + sS[1][0][f], sS[0][1][f] + sS[1][1][f], T(0), sS[0][2][f] + sS[1][2][f]};
+        if (warp == 0) {
+            T W0n[4] = {T(0), T(0), T(0), T(0)}, W0t[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+                if constexpr (rec_conventional(REC))  // Eq. (3.12), as k1d_stage
+                    W0n[slot[v]] = (T(1.25) * (sq[v][f + 3] - sq[v][f + 2])
+                                    - T(1.0 / 12.0) * (sq[v][f + 4] - sq[v][f + 1])) * ih;
+                else W0n[slot[v]] = sS[0][3 + v][f] + sS[1][3 + v][f];
+            }
+            Equilibrium<T> E;
+            equilibrium<T, 1, NONEQ>(W0, W0n, W0t, fp, E);
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+                sF[0][v][f] = E.F0[slot[v]];
+                sF[1][v][f] = E.F1[slot[v]];
+                sF[2][v][f] = E.F2[slot[v]];
+            }
+        } else if (fp.tau_mode != 0) {
+            T p0 = T(1);
+            if (fp.tau_mode == 2) p0 = fp.gm1 * (W0[3] - T(0.5) * W0[1] * W0[1] / W0[0]);
+            T cF[6], cD[6];
+            const T is = tau_over_dt(fp, sS[0][15][f], sS[1][15][f], p0, T(1) / fp.dt);
+            time_coeffs<T>(T(1) / is, is, cF, cD);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                sC[k][f] = cF[k];
+                sC[6 + k][f] = cD[k];
+            }
+        }
+    }
+    __syncthreads();
+    if (face) {
+        const int f = lane, v = warp;
+        T F = T(0), dF;
+        if (fp.tau_mode == 0) {
+            F = sF[0][v][f];
+            dF = sF[2][v][f];
+        } else {
+            const T x[6] = {sF[0][v][f], sF[1][v][f], sF[2][v][f], sS[0][6 + v][f] + sS[1][6 + v][f],
+                            sS[0][9 + v][f] + sS[1][9 + v][f], sS[0][12 + v][f] + sS[1][12 + v][f]};
+            const T tdt = fp.dt, i4 = T(4) / tdt;
+            // q_k = c_k s1 for p_k = 1 (k = 0, 3), c_k s2 for p_k = 2
+            auto combine = [&](int c, T s1, T s2) {
+                T r = (sC[c + 5][f] * s2) * x[5];
+                r = fma(sC[c + 4][f] * s2, x[4], r);
+                r = fma(sC[c + 3][f] * s1, x[3], r);
+                r = fma(sC[c + 2][f] * s2, x[2], r);
+                r = fma(sC[c + 1][f] * s2, x[1], r);
+                return fma(sC[c][f] * s1, x[0], r);
+            };
+            if (a.stage == 1) F = combine(0, T(1), tdt);
+            dF = combine(6, i4, T(4));
+        }
+        stage_comb<T>(a.stage, F, dF, fp.dt, sG[0][v][f], sG[1][v][f]);
+    }
+    __syncthreads();
+    T sig = T(0);
+    if (own) {
+        const double cx = s_cx;
+        const T cxt = (T)cx;
+        const int c = lane;
+        T w[4];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            const T d0 = sG[0][v][c + 1] - sG[0][v][c];
+            if constexpr (sizeof(T) == 4) {
+                if (a.stage == 1) {
+                    a.out0f[v * pl + o] = wstar32(sq[v][c + 3], cxt, d0);
+                    a.out1f[v * pl + o] = cxt * (sG[1][v][c + 1] - sG[1][v][c]);
+                } else {
+                    const double r = wnew32(base[v], acc[v], cxt, d0);
+                    a.out0[v * pl + o] = r;
+                    w[v] = (T)r;
+                    if (a.out0f) a.out0f[v * pl + o] = w[v];
+                }
+            } else {
+                const double r = upd64(base[v], cx, (double)d0);
+                a.out0[v * pl + o] = r;
+                if (a.stage == 1) a.out1[v * pl + o] = upd64(base[v], cx, (double)(sG[1][v][c + 1] - sG[1][v][c]));
+                w[v] = (T)r;
+            }
+        }
+        if (a.with_sigma) sig = cell_sigma<T, T>(w, 1, (T)g.gamma, (T)g.mu, (T)g.dx, err);
+    }
+    block_commit<96, T>(sig, a.with_sigma != 0, err, nfb, ds, a.commit != 0);
+}
+
 // ------------------------------------------------------------------ 2-D sweep
 // One stage = x sweep (pass 0) then y sweep (pass 1).  The x sweep stores its
 // flux-divergence increments dt/dx dG in the kernel's arithmetic type (inc0,

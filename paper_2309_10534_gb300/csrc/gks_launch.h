@@ -18,6 +18,9 @@ constexpr int SWEEP_TT64 = 8;
 // cells per block of the 1-D stage (TN + 2 = 128 threads: one per
 // reconstructed cell, face and updated cell)
 constexpr int STAGE1D_TN = 126;
+// up to these many cells a 1-D stage takes k1d_stage_wide
+constexpr int STAGE1D_WIDE_NX64 = 9120;
+constexpr int STAGE1D_WIDE_NX32 = 9120;
 
 struct HostFlux {
     double gamma, K, ntot, c1, c2, mu, prfac;
