@@ -252,6 +252,7 @@ gks_status enqueue_stage(gks_ctx* c, int stage, int with_commit, cudaStream_t st
         a.inc0 = c->inc0;
         a.inc1 = c->inc1;
         a.hmin = fmin(c->g.dx, c->g.dy);
+        a.sms = c->sms;
         if (pass == 0) {
             a.nn = c->desc.nx; a.nt = c->desc.ny; a.sn = 1; a.st = c->g.pitch;
             a.ihn = 1.0 / c->g.dx; a.iht = 1.0 / c->g.dy;
@@ -504,6 +505,8 @@ gks_status gks_create(const gks_grid_desc* d, gks_ctx** out)
     c->desc = *d;
     if (d->dim == 1) c->desc.ny = 1;
     c->nv = d->dim + 2;
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
     c->gas = {1.4, 0.0, 1.0};
     c->sch.cfl = 0.5;
     c->sch.c1 = 0.01;

@@ -17,7 +17,7 @@ struct gks_ctx {
     gks::GridDev g{};
     gks_gas gas{};
     gks_scheme sch{};
-    int nv = 0;
+    int nv = 0, sms = 1;
     double *W = nullptr, *Ws = nullptr, *Ac = nullptr;
     void *inc0 = nullptr, *inc1 = nullptr;  // 2-D: x-sweep increments, working precision;
                                              // 1-D float32: inc1 = accumulator increment

@@ -1,0 +1,16 @@
+// gks_k2d_f64_t4.cu -- the 2-D sweep in double, tiles of 4 rows.
+#include "gks_k2d.cuh"
+
+namespace gks {
+
+cudaError_t sweep_f64_t4_prepare()
+{
+    return SweepTile<double, 4, 128, 2>::prepare();
+}
+cudaError_t sweep_f64_t4(const GridDev& g, const SweepArgs& a, const HostFlux& hf, const TenoParams& tn,
+                        const TenoParams& tt, DevState* ds, cudaStream_t st)
+{
+    return SweepTile<double, 4, 128, 2>::launch(g, a, hf, tn, tt, ds, st);
+}
+
+}  // namespace gks

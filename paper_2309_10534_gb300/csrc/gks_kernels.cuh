@@ -734,6 +734,7 @@ struct SweepArgs {
     double hmin;         // min(dx, dy) for the CFL rate
     int with_sigma;
     int commit;          // the last block commits the step
+    int sms;             // multiprocessors of the device (tile choice)
 };
 
 // global variable index of local variable v (swap: faces normal to y)

@@ -9,12 +9,9 @@
 
 namespace gks {
 
-// tile of the 2-D sweep: TN cells along the face normal (TN + 1 faces) x TT
-// rows, one thread per (face, row) pair; float32 blocks hold 64 registers per
-// thread (1024 / threads blocks per SM)
+// tile of the 2-D sweep: TN cells along the face normal (TN + 1 faces, the
+// lanes of a warp) x rows by the grid's size (gks_k2d_select.cu)
 constexpr int SWEEP_TN = 31;
-constexpr int SWEEP_TT32 = 16;
-constexpr int SWEEP_TT64 = 8;
 // cells per block of the 1-D stage (TN + 2 = 128 threads: one per
 // reconstructed cell, face and updated cell)
 constexpr int STAGE1D_TN = 126;
