@@ -39,6 +39,10 @@ int gks_host_physical(int dim, int precision, double gamma, const double *W);
 int gks_host_teno(int precision, const double *q, double eps, int qpow, double ct1, double ct2,
                   double *faces, double *gauss);
 
+/* The float32 kernels' conversions of n values each way (integer arithmetic;
+ * float32 denormals become zero). */
+int gks_host_convert(const double *x, float *narrowed, const float *y, double *widened, int n);
+
 /* TENO-D selection of one stencil as 4 bits (bit 0: large stencil, bits 1-3:
  * the kept sub-stencils): in float64, and as the float64 kernels decide it in
  * float32 first (0: not decided there, the float64 selection is taken). */

@@ -314,11 +314,11 @@ __global__ void __launch_bounds__(128, (sizeof(T) == 4) ? 4 : 1) k_adj_gauss(Gri
             // one float64 subtraction per difference
             const double p1 = fc < a.nn ? a.lam1[b + fc * a.sn] : 0.0;
             const double m1 = fc >= 1 ? a.lam1[b + (fc - 1) * a.sn] : 0.0;
-            T e1 = (T)(p1 - m1), e2 = T(0);
+            T e1 = from_f64<T>(p1 - m1), e2 = T(0);
             if (a.lam2) {
                 const double p2 = fc < a.nn ? a.lam2[b + fc * a.sn] : 0.0;
                 const double m2 = fc >= 1 ? a.lam2[b + (fc - 1) * a.sn] : 0.0;
-                e2 = (T)(p2 - m2);
+                e2 = from_f64<T>(p2 - m2);
             }
             mF[h] = T(0.5) * (cF1 * e1 + cF2 * e2);
             mD[h] = T(0.5) * (cD1 * e1 + cD2 * e2);
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(256) k_adj_gather(GridDev g, AdjDir a)
             const int i = j + 2 - s;  // cell i's stencil position s is cell i - 2 + s = j
             if (i >= -1 && i <= a.nn) acc += D[(long long)(s * 4 + v) * DP + didx(a, i, r)];
         }
-        a.gW[(long long)gvar_(v, swap) * g.plane + org + j * a.sn + r * a.st] += (double)acc;
+        a.gW[(long long)gvar_(v, swap) * g.plane + org + j * a.sn + r * a.st] += to_f64(acc);
     }
 }
 
@@ -520,7 +520,7 @@ __global__ void k_sum3(const double* __restrict__ a, const double* __restrict__ 
 
 __global__ void k_shadow(const double* __restrict__ W, float* __restrict__ Wf, long long n)
 {
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) Wf[i] = (float)W[i];
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) Wf[i] = narrow(W[i]);
 }
 
 int blocks_for(long long n) { return (int)std::min<long long>((n + 255) / 256, 4096); }

@@ -69,19 +69,19 @@ __global__ void __launch_bounds__(256) k_sigma(GridDev g, const double* __restri
 // float32 shadow of a float64 array (same layout)
 __global__ void k_to_float(const double* __restrict__ W, float* __restrict__ Wf, long long n)
 {
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) Wf[i] = (float)W[i];
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) Wf[i] = narrow(W[i]);
 }
 
 // float64 views of the float32 path's stage buffers (gks_get_buffer):
 // W* from its float32 form, the accumulator from W and its increment
 __global__ void k_widen(const float* __restrict__ src, double* __restrict__ dst, long long n)
 {
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) dst[i] = (double)src[i];
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) dst[i] = widen(src[i]);
 }
 __global__ void k_accumulator(const double* __restrict__ W, const float* __restrict__ inc, double* __restrict__ A,
                               long long n)
 {
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) A[i] = W[i] - (double)inc[i];
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) A[i] = W[i] - widen(inc[i]);
 }
 
 // the first dt of a call, from k_sigma's rate

@@ -96,6 +96,57 @@ GKS_HD float quick_div(float a, float b)
 }
 GKS_HD int imax(int a, int b) { return a > b ? a : b; }
 
+// float32 <-> float64 on the integer pipe.  A conversion instruction occupies
+// GB300's float64 pipe for 64 cycles a warp, which made the float32 kernels'
+// one float64 update per value (a subtraction between two conversions) wait
+// on that pipe; these take about ten integer operations and the same bits:
+// widening is exact, narrowing rounds to nearest even, and float32 denormals
+// are zero, as everywhere in those kernels.
+GKS_HD unsigned float_bits(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    unsigned u;
+    memcpy(&u, &x, 4);
+    return u;
+#endif
+}
+GKS_HD double make_double(unsigned hi, unsigned lo)
+{
+#ifdef __CUDA_ARCH__
+    return __hiloint2double((int)hi, (int)lo);
+#else
+    const uint64_t b = ((uint64_t)hi << 32) | lo;
+    double x;
+    memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+GKS_HD double widen(float x)
+{
+    const unsigned u = float_bits(x), e = u & 0x7f800000u;
+    unsigned hi = ((u & 0x7fffffffu) >> 3) + (896u << 20);  // exponent bias 127 -> 1023
+    hi = e == 0u ? 0u : (e == 0x7f800000u ? (hi | 0x7ff00000u) : hi);
+    return make_double(hi | (u & 0x80000000u), e == 0u ? 0u : u << 29);
+}
+GKS_HD float narrow(double x)
+{
+    const unsigned hi = (unsigned)hi_word(x), lo = lo_word(x);
+    const int e = (int)((hi >> 20) & 0x7ffu);
+    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+    unsigned v = ((unsigned)(e - 896) << 23) + m;
+    v += ((lo & 0x1fffffffu) + 0x0fffffffu + (v & 1u)) >> 29;  // a carry runs into the exponent, up to infinity
+    if (e <= 896) v = 0u;
+    if (e >= 1151) v = (e == 0x7ff && (m | lo) != 0u) ? 0x7fffffffu : 0x7f800000u;
+    return as_float(v | (hi & 0x80000000u));
+}
+// a float64 value in the kernel's arithmetic type, and back
+template <typename T> GKS_HD T from_f64(double x) { return x; }
+template <> GKS_HD float from_f64<float>(double x) { return narrow(x); }
+GKS_HD double to_f64(double x) { return x; }
+GKS_HD double to_f64(float x) { return widen(x); }
+
 // integer power by squaring (q of Eq. 4.5 is a small positive integer)
 template <typename T>
 GKS_HD T ipow(T x, int q)

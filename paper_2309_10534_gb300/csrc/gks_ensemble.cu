@@ -190,7 +190,7 @@ __device__ void stage_chunk(ChunkSmem<T, NT>& sm, double* W, float* Wf, T* Ws, T
                 for (int v = 0; v < 3; ++v) {
                     const double r = wnew32(Wv[v][i], Av[v][i], cxt, sm.G[0][v][c + 1] - sm.G[0][v][c]);
                     Wv[v][i] = r;
-                    w[v] = (T)r;
+                    w[v] = narrow(r);
                     Wfv[v][i] = w[v];
                 }
                 sig = fmax(sig, cell_sigma<T, T>(w, 1, gamma, mu, hcell, err));
@@ -215,7 +215,7 @@ __device__ void stage_chunk(ChunkSmem<T, NT>& sm, double* W, float* Wf, T* Ws, T
 }
 
 template <typename T, int NT, bool NONEQ, bool PRFIX>
-__global__ void __launch_bounds__(NT) k_batch(BatchDev b, FluxParams<T> fp, TenoT<T> tn)
+__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1024 : 512) / NT) k_batch(BatchDev b, FluxParams<T> fp, TenoT<T> tn)
 {
     __shared__ ChunkSmem<T, NT> sm;
     __shared__ T red[NT / 32];
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(NT) k_batch(BatchDev b, FluxParams<T> fp, Teno
         // to float32, which becomes the shadow the stage-1 loads read)
         T sig = T(0);
         for (int i = tid; i < n; i += NT) {
-            const T w0[3] = {(T)W[i], (T)W[b.total + i], (T)W[2 * b.total + i]};
+            const T w0[3] = {from_f64<T>(W[i]), from_f64<T>(W[b.total + i]), from_f64<T>(W[2 * b.total + i])};
             if constexpr (sizeof(T) == 4) {
                 Wf[i] = w0[0];
                 Wf[b.total + i] = w0[1];
@@ -548,6 +548,8 @@ gks_status gks_batch_create(int count, const int* ncells, const double* lengths,
     if (!b) return GKS_ENOMEM;
     b->count = count;
     b->precision = precision;
+    // as many 256-thread blocks as are resident (64 / 128 registers a thread)
+    b->blocks_per_sm = precision == GKS_FP32_FLUX ? 4 : 2;
     b->n.assign(ncells, ncells + count);
     b->len.assign(lengths, lengths + count);
     b->off.resize(count);

@@ -198,6 +198,16 @@ int weno_ao_packed(const double* q, double eps_ao, double d_hi, double d_lo, dou
 
 }  // namespace
 
+extern "C" int gks_host_convert(const double* x, float* narrowed, const float* y, double* widened, int n)
+{
+    if (!x || !narrowed || !y || !widened || n < 0) return -1;
+    for (int k = 0; k < n; ++k) {
+        narrowed[k] = gks::narrow(x[k]);
+        widened[k] = gks::widen(y[k]);
+    }
+    return 0;
+}
+
 extern "C" int gks_host_teno_code(const double* q, double eps, int qpow, double ct1, double ct2, int* code64,
                                   int* code32)
 {

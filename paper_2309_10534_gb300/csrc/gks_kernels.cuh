@@ -257,7 +257,7 @@ __device__ __forceinline__ double upd64(double w, double cx, double dG) { return
 __device__ __forceinline__ float wstar32(float w, float cx, float dG) { return fmaf(-cx, dG, w); }
 __device__ __forceinline__ double wnew32(double w, float inc, float cx, float dG)
 {
-    return w - (double)fmaf(cx, dG, inc);
+    return w - widen(fmaf(cx, dG, inc));
 }
 
 // ------------------------------------------------------------------ 1-D stage
@@ -266,6 +266,8 @@ __device__ __forceinline__ double wnew32(double w, float inc, float cx, float dG
 // so it is formed and kept in float32, and the accumulator is kept as the
 // float32 increment dt/dx d(F + dt/6 dF); the only float64 arithmetic is the
 // final update W^{n+1} = W^n - (increment + dt/dx d(dt/3 dF*)).
+template <typename T> __device__ __forceinline__ T load_as(double x) { return from_f64<T>(x); }
+template <typename T> __device__ __forceinline__ T load_as(float x) { return x; }
 struct Stage1DArgs {
     const double* src;   // float64 reconstruction input (W; float64 path stage 2: W*)
     const float* srcf;   // float32 path: stage 1 the float32 shadow of W (or nullptr: src,
@@ -295,7 +297,7 @@ __device__ __noinline__ void load_edge_1d(T* sq, const E* src, const GridDev& g,
         T val = T(0);
         if (i < g.nx + NG) {  // beyond: padding
             const CellSrc cs = cell_source<false>(g, i, 0, ds, stage == 1 ? 0.0 : 0.5);
-            val = cs.state ? (T)state_value(g, cs.state, v) : (T)src[v * pl + NG + cs.i];
+            val = cs.state ? (T)state_value(g, cs.state, v) : load_as<T>(src[v * pl + NG + cs.i]);
             if (v == 1 && cs.n1) val = -val;
         }
         sq[k] = val;
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
         }
         for (int k = tid; k < 3 * (TN + 6); k += NT) {
             const int v = k / (TN + 6), c = k % (TN + 6);
-            sq[v][c] = (T)src[v * pl + i0 + c];
+            sq[v][c] = load_as<T>(src[v * pl + i0 + c]);
         }
     };
     if constexpr (sizeof(T) == 4) {
@@ -454,7 +456,7 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
                     const int gi = v * pl + o;
                     const double r = wnew32(a.base[gi], a.accf[gi], cxt, sG[0][v][c + 1] - sG[0][v][c]);
                     a.out0[gi] = r;
-                    w[v] = (T)r;
+                    w[v] = narrow(r);
                     if (a.out0f) a.out0f[gi] = w[v];
                 }
                 if (a.with_sigma) sig = fmax(sig, cell_sigma<T, T>(w, 1, s_scal[3], s_scal[4], s_scal[5], err));
@@ -517,10 +519,10 @@ __global__ void __launch_bounds__(96) k1d_stage_wide(const __grid_constant__ Gri
             const int i = i0 - NG + c;
             T val = T(0);
             if (i >= 0 && i < g.nx) {
-                val = (T)src[warp * pl + NG + i];
+                val = load_as<T>(src[warp * pl + NG + i]);
             } else if (i < g.nx + NG) {  // a ghost; beyond: padding
                 const CellSrc cs = cell_source<false>(g, i, 0, ds, a.stage == 1 ? 0.0 : 0.5);
-                val = cs.state ? (T)state_value(g, cs.state, warp) : (T)src[warp * pl + NG + cs.i];
+                val = cs.state ? (T)state_value(g, cs.state, warp) : load_as<T>(src[warp * pl + NG + cs.i]);
                 if (warp == 1 && cs.n1) val = -val;
             }
             sq[warp][c] = val;
@@ -689,7 +691,7 @@ __global__ void __launch_bounds__(96) k1d_stage_wide(const __grid_constant__ Gri
                 } else {
                     const double r = wnew32(base[v], acc[v], cxt, d0);
                     a.out0[v * pl + o] = r;
-                    w[v] = (T)r;
+                    w[v] = narrow(r);
                     if (a.out0f) a.out0f[v * pl + o] = w[v];
                 }
             } else {
@@ -1095,9 +1097,9 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
                         a.out0f[go] = a.basef[go] - (inc0[go] + d0);
                         inc1[go] = inc1[go] + d1;
                     } else {
-                        const double res = a.base[go] - (double)(inc1[go] + inc0[go] + d0);
+                        const double res = a.base[go] - widen(inc1[go] + inc0[go] + d0);
                         a.out0[go] = res;
-                        wf[v] = (float)res;  // local order; the CFL rate only needs |U|
+                        wf[v] = narrow(res);  // local order; the CFL rate only needs |U|
                         a.out0f[go] = wf[v];
                     }
                 } else if (a.stage == 1) {

@@ -425,6 +425,20 @@ def host_teno(q, precision="fp64", eps=1e-40, q_pow=7, ct1=1e-7, ct2=1e-5):
     return f, g, bool(r)
 
 
+def host_convert(x, y):
+    """(float32 of the float64 array x, float64 of the float32 array y) by the
+    float32 kernels' integer conversions."""
+    x, y = np.ascontiguousarray(x, dtype=np.float64), np.ascontiguousarray(y, dtype=np.float32)
+    if x.shape != y.shape:
+        raise ValueError("x and y must have the same shape")
+    a, b = np.empty(x.shape, dtype=np.float32), np.empty(x.shape)
+    f = _replica().gks_host_convert
+    f.argtypes, f.restype = [_vp, _vp, _vp, _vp, C.c_int], C.c_int
+    if f(x.ctypes.data_as(_vp), a.ctypes.data_as(_vp), y.ctypes.data_as(_vp), b.ctypes.data_as(_vp), x.size):
+        raise ValueError("bad argument")
+    return a, b
+
+
 def host_teno_code(q, eps=1e-40, q_pow=7, ct1=1e-7, ct2=1e-5):
     """(float64 selection, the float64 kernels' float32 decision or 0) of one
     stencil as 4-bit codes."""
