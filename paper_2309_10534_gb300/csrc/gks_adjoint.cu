@@ -18,9 +18,9 @@
 //                 (the forward sweep's phase 1)
 //   k_adj_gauss   per face segment and Gauss point: tangential TENO-D to the
 //                 Gauss point (forward), the reverse of the point flux, then
-//                 the transposed tangential reconstruction; writes, per face
-//                 segment, its contributions to the five line rows of its
-//                 tangential stencil
+//                 the transposed tangential reconstruction; sums, per tile,
+//                 the contributions to each line row, and writes the tile's
+//                 own rows and the two rows beyond each of its edges
 //   k_adj_normal  per cell: gathers the line cotangents of its two faces and
 //                 applies the transposed normal reconstruction; writes its
 //                 contributions to the five cells of its stencil
@@ -65,10 +65,11 @@ struct AdjDir {
     // float32 conversion in every thread would run on the slow float64 pipe)
     float fcF1, fcD1, fcF2, fcD2, fihn, fiht;
     void* lines;          // [NQ][faces nn+1][rows nt+4]
-    void* contrib;        // [5][NQ][faces nn+1][rows nt]
+    void* contrib;        // line cotangents: [NQ][faces nn+1][rows ntp], then [NQ][faces][tiles][4] edge rows
     void* dcell;          // [5][4][cells nn+2][rows nt+4]
     double* gW;           // ghosted gradient accumulator
     int dirn, nn, nt;
+    int tiles, ntp;       // Gauss-row tiles of adj_tile(dirn) rows, rows padded to whole tiles
     long long sn, st;     // element strides along normal / tangential
     double ihn, iht;
 };
@@ -81,9 +82,20 @@ __device__ __forceinline__ long long lidx(const AdjDir& a, int f, int r)
 {
     return a.dirn == 0 ? (long long)(r + 2) * (a.nn + 1) + f : (long long)f * (a.nt + 4) + (r + 2);
 }
-__device__ __forceinline__ long long cidx(const AdjDir& a, int f, int r)
+// A k_adj_gauss block holds 128 face segments (float64: 64, as a block's time
+// is its share of the float64 pipe): 16 along the unit stride.  Rows of its
+// tile along the tangential direction:
+template <typename T> constexpr int ADJ_PAIRS = sizeof(T) == 4 ? 128 : 64;
+__host__ __device__ constexpr int adj_tile(int dirn, bool f32) { return dirn == 0 ? (f32 ? 8 : 4) : 16; }
+// line cotangents: own rows of a tile, and its edge rows e = 0, 1 (the two
+// rows before it) and 2, 3 (after it)
+__device__ __forceinline__ long long midx(const AdjDir& a, int f, int r)
 {
-    return a.dirn == 0 ? (long long)r * (a.nn + 1) + f : (long long)f * a.nt + r;
+    return a.dirn == 0 ? (long long)r * (a.nn + 1) + f : (long long)f * a.ntp + r;
+}
+__device__ __forceinline__ long long eidx(const AdjDir& a, int f, int tile, int e)
+{
+    return a.dirn == 0 ? (long long)(tile * 4 + e) * (a.nn + 1) + f : (long long)f * (a.tiles * 4) + tile * 4 + e;
 }
 __device__ __forceinline__ long long didx(const AdjDir& a, int i, int r)
 {
@@ -237,9 +249,18 @@ __global__ void __launch_bounds__(256) k_adj_lines(GridDev g, AdjDir a, TenoT<T>
 // ---- Gauss points: forward tangential TENO-D, reverse point flux, transposed
 // tangential TENO-D.  Two adjacent lanes hold the two Gauss points of one face
 // segment; lane 0 finishes the left side's quantities, lane 1 the right's.
+//
+// A face segment contributes to the five line rows of its stencil.  Writing
+// the five contributions of 16 quantities (80 values per segment, read once
+// by k_adj_normal) was most of both kernels' memory traffic; the block's 128
+// segments now add theirs up in shared memory, and 1.25 to 1.5 values per
+// segment and quantity go out.
 template <typename T>
-__global__ void __launch_bounds__(128, (sizeof(T) == 4) ? 4 : 1) k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
+__global__ void __launch_bounds__(2 * ADJ_PAIRS<T>, (sizeof(T) == 4) ? 2 : 1)
+k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
 {
+    constexpr int NP = ADJ_PAIRS<T>;
+    __shared__ T sc[8][5][NP];  // [side, variable][stencil position][segment]
     const int gp = threadIdx.x & 1;
     const int x = (blockIdx.x * blockDim.x + threadIdx.x) >> 1, y = blockIdx.y * blockDim.y + threadIdx.y;
     int f, r;
@@ -250,50 +271,50 @@ __global__ void __launch_bounds__(128, (sizeof(T) == 4) ? 4 : 1) k_adj_gauss(Gri
     const bool swap = a.dirn != 0;
     const long long org = (long long)NG * g.pitch + NG;
     const long long LP = (long long)(a.nn + 1) * (a.nt + 4);
-    const long long CP = (long long)(a.nn + 1) * a.nt;
     const T* Lq = static_cast<const T*>(a.lines);
-    const T gpos = gp ? T(0.28867513459481288) : T(-0.28867513459481288);
     const T iht = scal<T>(a.iht, a.fiht);
 
     // forward, as the forward sweep: lane gp reconstructs side gp (0: left,
     // 1: right) at both Gauss points, keeps its own point and hands the other
-    // point's values to its partner
+    // point's values to its partner; L is the own side, R the partner's
     Side<T> L, R;
     unsigned codes = 0;  // selections of the own side: 4 bits per quantity kk * 4 + v
-    const T gA = T(-0.28867513459481288), gB = T(0.28867513459481288);
+    const T gs = gp ? T(0.28867513459481288) : T(-0.28867513459481288);
+    {
+        const int ls = a.dirn == 0 ? a.nn + 1 : 1;  // element stride of line rows
+        const T* Lp = Lq + (long long)(8 * gp) * LP + lidx(a, fc, rc - 2);
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        // the side's value and normal-slope streams as one pair, as the forward
-        T q[2][5];
-        T va[2], da[2], vb[2], db[2];
+        for (int v = 0; v < 4; ++v) {
+            // the side's value and normal-slope streams as one pair, as the forward
+            T q[2][5];
+            T va[2], da[2], vb[2], db[2];
+            const T *pv = Lp + v * LP, *ps = Lp + (4 + v) * LP;
 #pragma unroll
-        for (int l = 0; l < 2; ++l)
-#pragma unroll
-            for (int s = 0; s < 5; ++s) q[l][s] = Lq[((2 * gp + l) * 4 + v) * LP + lidx(a, fc, rc - 2 + s)];
-        const unsigned c2 = fwd_gauss2(q[0], q[1], tt, gA, gB, va, da, vb, db);
-        codes |= (c2 & 15u) << (4 * v);
-        codes |= (c2 >> 4) << (4 * (4 + v));
-        T own = gp ? vb[0] : va[0], got = __shfl_xor_sync(0xffffffffu, gp ? va[0] : vb[0], 1);
-        L.W[v] = gp ? got : own;
-        R.W[v] = gp ? own : got;
-        own = (gp ? db[0] : da[0]) * iht;
-        got = __shfl_xor_sync(0xffffffffu, (gp ? da[0] : db[0]) * iht, 1);
-        L.Wt[v] = gp ? got : own;
-        R.Wt[v] = gp ? own : got;
-        own = gp ? vb[1] : va[1];
-        got = __shfl_xor_sync(0xffffffffu, gp ? va[1] : vb[1], 1);
-        L.Wn[v] = gp ? got : own;
-        R.Wn[v] = gp ? own : got;
+            for (int s = 0; s < 5; ++s) {
+                q[0][s] = pv[s * ls];
+                q[1][s] = ps[s * ls];
+            }
+            const unsigned c2 = fwd_gauss2(q[0], q[1], tt, -gs, gs, vb, db, va, da);
+            codes |= (c2 & 15u) << (4 * v);
+            codes |= (c2 >> 4) << (4 * (4 + v));
+            L.W[v] = va[0];
+            R.W[v] = __shfl_xor_sync(0xffffffffu, vb[0], 1);
+            L.Wt[v] = da[0] * iht;
+            R.Wt[v] = __shfl_xor_sync(0xffffffffu, db[0], 1) * iht;
+            L.Wn[v] = va[1];
+            R.Wn[v] = __shfl_xor_sync(0xffffffffu, vb[1], 1);
+        }
     }
     // positivity fallback, as the forward: the adjacent cell average, zero slopes
     const bool fbL = valid && !physical<T, 2>(L.W, fp.gm1);
     const bool fbR = valid && !physical<T, 2>(R.W, fp.gm1);
+    const int cL = fc - 1 + gp, cR = fc - gp;  // normal index of the cell beside the face on the own / partner's side
     if (fbL || fbR) {
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const long long b = (long long)gvar_(v, swap) * g.plane + org + rc * a.st;
-            if (fbL) { L.W[v] = load_src<T>(a, b + (fc - 1) * a.sn); L.Wn[v] = L.Wt[v] = T(0); }
-            if (fbR) { R.W[v] = load_src<T>(a, b + fc * a.sn); R.Wn[v] = R.Wt[v] = T(0); }
+            if (fbL) { L.W[v] = load_src<T>(a, b + cL * a.sn); L.Wn[v] = L.Wt[v] = T(0); }
+            if (fbR) { R.W[v] = load_src<T>(a, b + cR * a.sn); R.Wn[v] = R.Wt[v] = T(0); }
         }
     }
     // face cotangents (each Gauss point carries weight 1/2).  The
@@ -337,59 +358,68 @@ __global__ void __launch_bounds__(128, (sizeof(T) == 4) ? 4 : 1) k_adj_gauss(Gri
     Side<T> gL, gR;
 #pragma unroll
     for (int v = 0; v < 4; ++v) gL.W[v] = gL.Wn[v] = gL.Wt[v] = gR.W[v] = gR.Wn[v] = gR.Wt[v] = T(0);
-    if (valid) point_flux_vjp(L, R, fp, gF, gdF, gL, gR);
+    if (valid) point_flux_vjp(L, R, gp ? T(-1) : T(1), fp, gF, gdF, gL, gR);
     if (fbL || fbR) {
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const long long b = (long long)gvar_(v, swap) * g.plane + org + rc * a.st;
             if (fbL) {
-                atomicAdd(&a.gW[b + (fc - 1) * a.sn], (double)gL.W[v]);
+                atomicAdd(&a.gW[b + cL * a.sn], (double)gL.W[v]);
                 gL.W[v] = gL.Wn[v] = gL.Wt[v] = T(0);
             }
             if (fbR) {
-                atomicAdd(&a.gW[b + fc * a.sn], (double)gR.W[v]);
+                atomicAdd(&a.gW[b + cR * a.sn], (double)gR.W[v]);
                 gR.W[v] = gR.Wn[v] = gR.Wt[v] = T(0);
             }
         }
     }
-    // exchange: lane 0 keeps the left side (receives its + point), lane 1 the right
-    Side<T>& mine = gp ? gR : gL;
-    const Side<T>& other = gp ? gL : gR;
+    // exchange: each lane keeps its own side and receives that side's
+    // cotangents at the partner's point
     T oW[4], oWn[4], oWt[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-        oW[v] = __shfl_xor_sync(0xffffffffu, other.W[v], 1);
-        oWn[v] = __shfl_xor_sync(0xffffffffu, other.Wn[v], 1);
-        oWt[v] = __shfl_xor_sync(0xffffffffu, other.Wt[v], 1);
+        oW[v] = __shfl_xor_sync(0xffffffffu, gR.W[v], 1);
+        oWn[v] = __shfl_xor_sync(0xffffffffu, gR.Wn[v], 1);
+        oWt[v] = __shfl_xor_sync(0xffffffffu, gR.Wt[v], 1);
     }
-    if (!valid) return;
-    const T gm = gA, gpl = gB;
-    T* C = static_cast<T*>(a.contrib);
+    const int pair = threadIdx.y * 16 + (threadIdx.x >> 1), tid = threadIdx.y * 32 + threadIdx.x;
+    const int TT = adj_tile(a.dirn, sizeof(T) == 4), NF = NP / TT;  // the tile's rows and faces
+    const int tile = a.dirn == 0 ? blockIdx.y : blockIdx.x, f0 = (a.dirn == 0 ? blockIdx.x : blockIdx.y) * NF;
+    const long long MP = (long long)(a.nn + 1) * a.ntp, EP = (long long)(a.nn + 1) * a.tiles * 4;
+    T* M = static_cast<T*>(a.contrib);
+    T* Eg = M + NQ * MP;
 #pragma unroll 1
-    for (int kk = 0; kk < 2; ++kk) {
-        const int k = 2 * gp + kk;  // lane 0: k = 0, 1 (left), lane 1: k = 2, 3 (right)
+    for (int kk = 0; kk < 2; ++kk) {  // values, then normal slopes, of both sides
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const int qi = k * 4 + v;
             TenoSel<T> S;
             sel_decode((codes >> (4 * (kk * 4 + v))) & 15u, S);
-            // cotangents at the - point and the + point
-            T gvm, gdm, gvp, gdp;
-            if (kk == 0) {
-                const T a0 = mine.W[v], d0 = mine.Wt[v] * iht, a1 = oW[v], d1 = oWt[v] * iht;
-                gvm = gp ? a1 : a0; gdm = gp ? d1 : d0;
-                gvp = gp ? a0 : a1; gdp = gp ? d0 : d1;
-            } else {
-                gvm = gp ? oWn[v] : mine.Wn[v];
-                gvp = gp ? mine.Wn[v] : oWn[v];
-                gdm = gdp = T(0);
-            }
-            T gq[5] = {T(0), T(0), T(0), T(0), T(0)};
-            teno_gauss_T(S, gm, gvm, gdm, gq);
-            teno_gauss_T(S, gpl, gvp, gdp, gq);
+            T gq[5];
+            if (kk == 0) teno_gauss_pm_T(S, gs, oW[v], oWt[v] * iht, gL.W[v], gL.Wt[v] * iht, gq);
+            else teno_gauss_pm_T(S, gs, oWn[v], T(0), gL.Wn[v], T(0), gq);
 #pragma unroll
-            for (int s = 0; s < 5; ++s) C[(long long)(s * NQ + qi) * CP + cidx(a, f, r)] = gq[s];
+            for (int s = 0; s < 5; ++s) sc[gp * 4 + v][s][pair] = valid ? gq[s] : T(0);
         }
+        __syncthreads();
+        // line row l - 2 of the tile from the segments of rows l - s; 16
+        // segments of a row (dirn 0) or of a face (dirn 1) are adjacent
+        for (int k = tid; k < 8 * (TT + 4) * NF; k += 2 * NP) {
+            int l, fl, qq;
+            if (a.dirn == 0) { fl = k % 16; l = (k / 16) % (NP / 16 + 4); qq = k / (NP + 64); }
+            else { l = k % 20; fl = (k / 20) % (NP / 16); qq = k / (20 * (NP / 16)); }
+            const int f2_ = f0 + fl;
+            if (f2_ > a.nn) continue;
+            T acc = T(0);
+#pragma unroll
+            for (int s = 0; s < 5; ++s) {
+                const int rl = l - s;
+                if (rl >= 0 && rl < TT) acc += sc[qq][s][a.dirn == 0 ? rl * 16 + fl : fl * 16 + rl];
+            }
+            const int qi = (2 * (qq >> 2) + kk) * 4 + (qq & 3);
+            if (l >= 2 && l < TT + 2) M[qi * MP + midx(a, f2_, tile * TT + l - 2)] = acc;
+            else Eg[qi * EP + eidx(a, f2_, tile, l < 2 ? l : l - TT)] = acc;
+        }
+        __syncthreads();
     }
 }
 
@@ -402,19 +432,28 @@ __global__ void __launch_bounds__(256) k_adj_normal(GridDev g, AdjDir a, TenoT<T
     if (i > a.nn || r >= a.nt + 2) return;
     const bool swap = a.dirn != 0;
     const long long org = (long long)NG * g.pitch + NG;
-    const long long CP = (long long)(a.nn + 1) * a.nt;
+    const long long MP = (long long)(a.nn + 1) * a.ntp, EP = (long long)(a.nn + 1) * a.tiles * 4;
     const long long DP = (long long)(a.nn + 2) * (a.nt + 4);
-    const T* C = static_cast<const T*>(a.contrib);
+    const T* M = static_cast<const T*>(a.contrib);
+    const T* Eg = M + NQ * MP;
     T* D = static_cast<T*>(a.dcell);
     const T ih = scal<T>(a.ihn, a.fihn);
-    // line row r receives from Gauss row r - s + 2 at stencil position s
+    // line row r: its tile's sum, and the edge rows of the tiles beside it
+    const int TT = adj_tile(a.dirn, sizeof(T) == 4);
+    int own = -1, e1 = -1, e2 = -1, t1 = 0, t2 = 0;  // own row; edge rows of tiles t1, t2
+    if (r < 0) { t1 = 0; e1 = r + 2; }
+    else if (r >= a.ntp) { t1 = a.tiles - 1; e1 = 2 + r - a.ntp; }
+    else {
+        const int tl = r / TT, m = r - tl * TT;
+        own = r;
+        if (m >= TT - 2 && tl + 1 < a.tiles) { t1 = tl + 1; e1 = m - (TT - 2); }
+        if (m < 2 && tl > 0) { t2 = tl - 1; e2 = 2 + m; }
+    }
     auto gline = [&](int q, int f) {
         T acc = T(0);
-#pragma unroll
-        for (int s = 0; s < 5; ++s) {
-            const int rg = r - s + 2;
-            if (rg >= 0 && rg < a.nt) acc += C[(long long)(s * NQ + q) * CP + cidx(a, f, rg)];
-        }
+        if (e1 >= 0) acc += Eg[q * EP + eidx(a, f, t1, e1)];
+        if (own >= 0) acc += M[q * MP + midx(a, f, own)];
+        if (e2 >= 0) acc += Eg[q * EP + eidx(a, f, t2, e2)];
         return acc;
     };
     {
@@ -476,6 +515,34 @@ __global__ void __launch_bounds__(256) k_adj_gather(GridDev g, AdjDir a)
 // ---- transpose of the ghost fill: y ghost rows first (over the full ghosted
 // width), then the x ghost columns of the interior rows.  One thread per
 // (column or row, variable) walks its six ghost cells in a fixed order.
+// The six ghosts and their source cells are read at once and added up in a
+// fixed order in registers (one after the other through memory they cost a
+// round trip each).  tang, norm: the line holds the tangential / the normal
+// momentum of these ghosts.
+__device__ __forceinline__ void fold_line(double* P, long long stride, int n, int bc0, int bc1, bool tang, bool norm)
+{
+    double x[2 * NG], s[2 * NG];
+    int src[2 * NG];
+#pragma unroll
+    for (int k = 0; k < 2 * NG; ++k) {
+        const int j = k < NG ? k : n + k;
+        bool fn, fa;
+        src[k] = ghost_src(k < NG ? bc0 : bc1, n, j, fn, fa);
+        const double y = P[j * stride];
+        x[k] = ((norm && (fn || fa)) || (tang && fa)) ? -y : y;
+        s[k] = P[src[k] * stride];
+    }
+#pragma unroll
+    for (int k = 0; k < 2 * NG; ++k) {
+        s[k] += x[k];
+#pragma unroll
+        for (int m = k + 1; m < 2 * NG; ++m)
+            if (src[m] == src[k]) s[m] = s[k];  // the same source again: go on from its sum
+        P[src[k] * stride] = s[k];
+        P[(k < NG ? k : n + k) * stride] = 0.0;
+    }
+}
+
 __global__ void k_fold_y(GridDev g, double* gW)
 {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -483,15 +550,7 @@ __global__ void k_fold_y(GridDev g, double* gW)
     if (idx >= 4 * gx) return;
     const int v = idx / gx, i = idx % gx;
     double* P = gW + (long long)v * g.plane + i;
-    for (int k = 0; k < 2 * NG; ++k) {
-        const int j = k < NG ? k : g.ny + k;
-        bool fn, fa;
-        const int sj = ghost_src(g.bc[2 + (j >= NG + g.ny)], g.ny, j, fn, fa);
-        const bool neg = (v == 2 && (fn || fa)) || (v == 1 && fa);
-        const double x = P[(long long)j * g.pitch];
-        P[(long long)sj * g.pitch] += neg ? -x : x;
-        P[(long long)j * g.pitch] = 0.0;
-    }
+    fold_line(P, g.pitch, g.ny, g.bc[2], g.bc[3], v == 1, v == 2);
 }
 
 __global__ void k_fold_x(GridDev g, double* gW)
@@ -500,15 +559,7 @@ __global__ void k_fold_x(GridDev g, double* gW)
     if (idx >= 4 * g.ny) return;
     const int v = idx / g.ny, j = NG + idx % g.ny;
     double* P = gW + (long long)v * g.plane + (long long)j * g.pitch;
-    for (int k = 0; k < 2 * NG; ++k) {
-        const int i = k < NG ? k : g.nx + k;
-        bool fn, fa;
-        const int si = ghost_src(g.bc[(i >= NG + g.nx)], g.nx, i, fn, fa);
-        const bool neg = (v == 1 && (fn || fa)) || (v == 2 && fa);
-        const double x = P[i];
-        P[si] += neg ? -x : x;
-        P[i] = 0.0;
-    }
+    fold_line(P, 1, g.nx, g.bc[0], g.bc[1], v == 2, v == 1);
 }
 
 // out = a + b + c (whole ghosted arrays)
@@ -534,8 +585,10 @@ struct gks_adjoint {
     double dt = 0.0;
     bool have_forward = false;
     std::vector<double*> ckpt;   // W at steps 0, k, 2k, ... (ghosted)
-    std::vector<double*> seg;    // W of the segment being reversed
-    std::vector<void*> segs;     // its W* (float32 on the float32 path), from the recomputation
+    // the stage inputs W and W* of the segment being reversed, from the
+    // recomputation, as the adjoint kernels read them: in the kernels'
+    // precision, ghosts filled
+    std::vector<void*> seg, segs;
     double* WN = nullptr;        // final state of the forward pass
     double *lam = nullptr, *lams = nullptr, *gacc = nullptr, *nxt = nullptr;
     void *lines = nullptr, *contrib = nullptr, *dcell = nullptr;
@@ -565,7 +618,12 @@ gks_status adj_scratch(gks_adjoint* A)
     const long long nx = c->desc.nx, ny = c->desc.ny;
     const size_t es = c->desc.precision == GKS_FP32_FLUX ? 4 : 8;
     const long long lines = std::max((nx + 1) * (ny + 4), (ny + 1) * (nx + 4)) * NQ;
-    const long long contrib = std::max((nx + 1) * ny, (ny + 1) * nx) * 5 * NQ;
+    long long contrib = 0;  // line cotangents: own rows of whole tiles and four edge rows per tile
+    for (int d = 0; d < 2; ++d) {
+        const long long nn = d == 0 ? nx : ny, nt = d == 0 ? ny : nx, tt = adj_tile(d, es == 4);
+        const long long tiles = (nt + tt - 1) / tt;
+        contrib = std::max(contrib, (nn + 1) * tiles * (tt + 4) * NQ);
+    }
     const long long dcell = std::max((nx + 2) * (ny + 4), (ny + 2) * (nx + 4)) * 20;
     CK(cudaMalloc(&A->lines, lines * es));
     CK(cudaMalloc(&A->contrib, contrib * es));
@@ -605,12 +663,12 @@ gks_status sweep_vjp_t(gks_adjoint* A, AdjDir d)
         const int ex = d.dirn == 0 ? nnorm : ntan, ey = d.dirn == 0 ? ntan : nnorm;
         return dim3((unsigned)((ex * xmul + blk.x - 1) / blk.x), (unsigned)((ey + blk.y - 1) / blk.y));
     };
-    const dim3 b256(32, 8), b128(32, 4);
+    const dim3 b256(32, 8), bg(32, ADJ_PAIRS<T> / 16);
     // the per-cell kernels take the two variable pairs in blockIdx.z
     dim3 gcell = grid_for(d.nn + 2, d.nt + 4, b256, 1);
     gcell.z = 2;
     k_adj_lines<T><<<gcell, b256, 0, st>>>(g, d, tn);
-    k_adj_gauss<T><<<grid_for(d.nn + 1, d.nt, b128, 2), b128, 0, st>>>(g, d, fp, tt);
+    k_adj_gauss<T><<<grid_for(d.nn + 1, d.nt, bg, 2), bg, 0, st>>>(g, d, fp, tt);
     k_adj_normal<T><<<gcell, b256, 0, st>>>(g, d, tn);
     k_adj_gather<T><<<grid_for(d.nn + 6, d.nt + 4, b256, 1), b256, 0, st>>>(g, d);
     CK(cudaGetLastError());
@@ -619,16 +677,16 @@ gks_status sweep_vjp_t(gks_adjoint* A, AdjDir d)
 }
 
 // adds to A->gacc the transposed flux Jacobian of both directions at the
-// stage input (src), with face cotangents from lam1, lam2
-gks_status stage_vjp(gks_adjoint* A, bool stage2_input, const double* lam1, const double* lam2, double cF1,
+// stage input, with face cotangents from lam1, lam2
+gks_status stage_vjp(gks_adjoint* A, const void* input, const double* lam1, const double* lam2, double cF1,
                      double cD1, double cF2, double cD2)
 {
     gks_ctx* c = A->c;
     const bool f32 = c->desc.precision == GKS_FP32_FLUX;
     for (int dirn = 0; dirn < 2; ++dirn) {
         AdjDir d{};
-        d.src = stage2_input ? c->Ws : c->W;
-        d.srcf = stage2_input ? c->Wsf : c->Wf;
+        d.src = static_cast<const double*>(input);
+        d.srcf = static_cast<const float*>(input);
         d.lam1 = lam1;
         d.lam2 = lam2;
         const double h = dirn == 0 ? c->g.dx : c->g.dy;
@@ -648,6 +706,9 @@ gks_status stage_vjp(gks_adjoint* A, bool stage2_input, const double* lam1, cons
             d.nn = c->desc.ny; d.nt = c->desc.nx; d.sn = c->g.pitch; d.st = 1;
             d.ihn = 1.0 / c->g.dy; d.iht = 1.0 / c->g.dx;
         }
+        const int tt = adj_tile(dirn, f32);
+        d.tiles = (d.nt + tt - 1) / tt;
+        d.ntp = d.tiles * tt;
         d.fcF1 = (float)d.cF1;
         d.fcD1 = (float)d.cD1;
         d.fcF2 = (float)d.cF2;
@@ -665,30 +726,26 @@ gks_status stage_vjp(gks_adjoint* A, bool stage2_input, const double* lam1, cons
     return GKS_OK;
 }
 
-size_t wstar_bytes(const gks_ctx* c)
+// bytes of a state in the kernels' precision
+size_t work_bytes(const gks_ctx* c)
 {
     return (size_t)c->nv * c->g.plane * (c->Wsf ? sizeof(float) : sizeof(double));
 }
 
 // A->lam <- (dW^{n+1}/dW^n)^T A->lam at the ghosted state Wn with its stage
 // state Ws (as the forward pass computed it)
-gks_status adjoint_step(gks_adjoint* A, const double* Wn, const void* Ws)
+gks_status adjoint_step(gks_adjoint* A, const void* Wn, const void* Ws)
 {
     gks_ctx* c = A->c;
     const double dt = A->dt;
     gks_status s;
-    if ((s = load_state(A, Wn))) return s;
-    void* ws = c->Wsf ? static_cast<void*>(c->Wsf) : static_cast<void*>(c->Ws);
-    CK(cudaMemcpyAsync(ws, Ws, wstar_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
-    if ((s = rt::enqueue_ghosts(c, c->W, c->stream))) return s;
-    if ((s = rt::enqueue_ghosts(c, c->Ws, c->stream))) return s;
     // lam* = [d dF/dW*]^T (dt^2/(3h) Delta lam)
     CK(cudaMemsetAsync(A->gacc, 0, c->arr_bytes, c->stream));
-    if ((s = stage_vjp(A, true, A->lam, nullptr, 0.0, dt * dt / 3.0, 0.0, 0.0))) return s;
+    if ((s = stage_vjp(A, Ws, A->lam, nullptr, 0.0, dt * dt / 3.0, 0.0, 0.0))) return s;
     std::swap(A->lams, A->gacc);
     // stage 1 at W^n with the cotangents of A (lam) and of W* (lam*)
     CK(cudaMemsetAsync(A->gacc, 0, c->arr_bytes, c->stream));
-    if ((s = stage_vjp(A, false, A->lam, A->lams, dt, dt * dt / 6.0, 0.5 * dt, dt * dt / 8.0))) return s;
+    if ((s = stage_vjp(A, Wn, A->lam, A->lams, dt, dt * dt / 6.0, 0.5 * dt, dt * dt / 8.0))) return s;
     const long long n = (long long)c->nv * c->g.plane;
     k_sum3<<<blocks_for(n), 256, 0, c->stream>>>(A->lam, A->lams, A->gacc, A->nxt, n);
     CK(cudaGetLastError());
@@ -712,9 +769,8 @@ gks_status reserve(gks_adjoint* A, int nsteps)
         A->ckpt.push_back(p);
     }
     while ((int)A->seg.size() < A->k) {
-        double* p = nullptr;
-        void* q = nullptr;
-        if (cudaMalloc(&p, c->arr_bytes) != cudaSuccess || cudaMalloc(&q, wstar_bytes(c)) != cudaSuccess) {
+        void *p = nullptr, *q = nullptr;
+        if (cudaMalloc(&p, work_bytes(c)) != cudaSuccess || cudaMalloc(&q, work_bytes(c)) != cudaSuccess) {
             cudaFree(p);
             cudaGetLastError();
             return rt::fail(c, GKS_ENOMEM, "no device memory for a %d-step segment", A->k);
@@ -776,7 +832,7 @@ void gks_adjoint_destroy(gks_adjoint* A)
     if (!A) return;
     if (A->seg_exec) cudaGraphExecDestroy(A->seg_exec);
     for (double* p : A->ckpt) cudaFree(p);
-    for (double* p : A->seg) cudaFree(p);
+    for (void* p : A->seg) cudaFree(p);
     for (void* p : A->segs) cudaFree(p);
     cudaFree(A->WN);
     cudaFree(A->lam);
@@ -819,11 +875,14 @@ gks_status run_segment(gks_adjoint* A, int len)
 {
     gks_ctx* c = A->c;
     gks_status s;
+    const void* w = c->Wf ? static_cast<const void*>(c->Wf) : static_cast<const void*>(c->W);
     const void* ws = c->Wsf ? static_cast<const void*>(c->Wsf) : static_cast<const void*>(c->Ws);
     for (int n = 0; n < len; ++n) {
-        CK(cudaMemcpyAsync(A->seg[n], c->W, c->arr_bytes, cudaMemcpyDeviceToDevice, c->stream));
+        CK(cudaMemcpyAsync(A->seg[n], w, work_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
+        if ((s = rt::fill_ghosts(c, A->seg[n], c->stream))) return s;
         if ((s = gks_stage(c, 1, A->dt))) return s;
-        CK(cudaMemcpyAsync(A->segs[n], ws, wstar_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
+        CK(cudaMemcpyAsync(A->segs[n], ws, work_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
+        if ((s = rt::fill_ghosts(c, A->segs[n], c->stream))) return s;
         if (n + 1 < len && (s = gks_stage(c, 2, A->dt))) return s;
     }
     for (int n = len - 1; n >= 0; --n)

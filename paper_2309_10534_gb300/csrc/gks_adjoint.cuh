@@ -21,81 +21,63 @@
 namespace gks {
 
 // ------------------------------------------------------------------ TENO-D, frozen selection
-// transpose of the quadratic coefficients b_k, c_k of teno_select
+// Both transposes go through the first differences the reconstruction is
+// formed from (TenoSel): cotangents of A, B, C, D (or of the sub-stencils'
+// coefficients) -> of e_1 .. e_4 -> of the five cells; gq is set.
 template <typename T>
-GKS_HD void teno_bc_T(const T* gb, const T* gc, T* gq)
+GKS_HD void teno_e_T(T ge1, T ge2, T ge3, T ge4, T gc, T* gq)
 {
-    // b0 = (q0 - 4 q1 + 3 q2)/2, c0 = (q0 - 2 q1 + q2)/2
-    gq[0] += T(0.5) * (gb[0] + gc[0]);
-    gq[1] += T(-2) * gb[0] - gc[0];
-    gq[2] += T(1.5) * gb[0] + T(0.5) * gc[0];
-    // b1 = (q3 - q1)/2, c1 = (q1 - 2 q2 + q3)/2
-    gq[1] += T(0.5) * (gc[1] - gb[1]);
-    gq[2] -= gc[1];
-    gq[3] += T(0.5) * (gb[1] + gc[1]);
-    // b2 = (-3 q2 + 4 q3 - q4)/2, c2 = (q2 - 2 q3 + q4)/2
-    gq[2] += T(-1.5) * gb[2] + T(0.5) * gc[2];
-    gq[3] += T(2) * gb[2] - gc[2];
-    gq[4] += T(0.5) * (gc[2] - gb[2]);
+    gq[0] = -ge1;
+    gq[1] = ge1 - ge2;
+    gq[2] = gc + (ge2 - ge3);
+    gq[3] = ge3 - ge4;
+    gq[4] = ge4;
+}
+// kept sub-stencils: cotangents of 2 sum w b and 2 sum w c (teno_small)
+template <typename T>
+GKS_HD void teno_small_T(const TenoSel<T>& S, T gb, T gc, T g2, T* gq)
+{
+    const T b0 = S.w[0] * gb, b1 = S.w[1] * gb, b2 = S.w[2] * gb;
+    const T c0 = S.w[0] * gc, c1 = S.w[1] * gc, c2 = S.w[2] * gc;
+    // B0 = 3 e2 - e1, A = e2 + e3, B2 = 3 e3 - e4; C0 = e2 - e1, C = e3 - e2, C2 = e4 - e3
+    teno_e_T(-b0 - c0, T(3) * b0 + b1 + (c0 - c1), T(3) * b2 + b1 + (c1 - c2), c2 - b2, g2, gq);
+}
+// large stencil: cotangents of A, B, C, D
+template <typename T>
+GKS_HD void teno_large_T(T gA, T gB, T gC, T gD, T g2, T* gq)
+{
+    teno_e_T(gB - gD, gA - gC, gA + gC, gB + gD, g2, gq);
 }
 
-// transpose of the quartic's Legendre-type coefficients u1..u4 of teno_select
-template <typename T>
-GKS_HD void teno_u_T(T gu1, T gu2, T gu3, T gu4, T* gq)
-{
-    const T a = gu1 * T(1.0 / 120.0), b = gu2 * T(1.0 / 56.0), c = gu3 * T(1.0 / 12.0), d = gu4 * T(1.0 / 24.0);
-    gq[0] += T(11) * a - T(3) * b - c + d;
-    gq[1] += T(-82) * a + T(40) * b + T(2) * c - T(4) * d;
-    gq[2] += T(-74) * b + T(6) * d;
-    gq[3] += T(82) * a + T(40) * b - T(2) * c - T(4) * d;
-    gq[4] += T(-11) * a - T(3) * b + c + d;
-}
-
-// transpose of teno_faces: cotangents of (vp, dp, vm, dm), added to gq[0..4]
+// transpose of teno_faces: cotangents of (vp, dp, vm, dm) -> gq[0..4]
 template <typename T>
 GKS_HD void teno_faces_T(const TenoSel<T>& S, T gvp, T gdp, T gvm, T gdm, T* gq)
 {
-    if (S.large) {  // Eqs. (4.8), (4.9) and their mirror
-        gq[0] += (T(2) * gvp - T(3) * gvm) * T(1.0 / 60.0) + gdm * T(1.0 / 12.0);
-        gq[1] += (T(-13) * gvp + T(27) * gvm) * T(1.0 / 60.0) + (gdp - T(15) * gdm) * T(1.0 / 12.0);
-        gq[2] += T(47) * (gvp + gvm) * T(1.0 / 60.0) + T(15) * (gdm - gdp) * T(1.0 / 12.0);
-        gq[3] += (T(27) * gvp - T(13) * gvm) * T(1.0 / 60.0) + (T(15) * gdp - gdm) * T(1.0 / 12.0);
-        gq[4] += (T(-3) * gvp + T(2) * gvm) * T(1.0 / 60.0) - gdp * T(1.0 / 12.0);
-        return;
+    const T ge = gvp + gvm, go = gvp - gvm, gde = gdp + gdm, gdo = gdp - gdm;
+    if (S.large) {
+        // even = q2 + (13 C - D)/120, odd = (7 A - B)/24, deven = (13 A - B)/24, dodd = (15 C - D)/24
+        const T e = T(1.0 / 120.0) * ge, o = T(1.0 / 24.0) * go, d = T(1.0 / 24.0) * gde, p = T(1.0 / 24.0) * gdo;
+        teno_large_T(T(7) * o + T(13) * d, -(o + d), T(13) * e + T(15) * p, -(e + p), ge, gq);
+    } else {
+        // even = q2 + sc/12, odd = sb/4, deven = sb/2, dodd = sc/2
+        teno_small_T(S, T(0.25) * go + T(0.5) * gde, T(1.0 / 12.0) * ge + T(0.5) * gdo, ge, gq);
     }
-    // vp = q2 + sum w (b/2 + c/6), vm = q2 + sum w (c/6 - b/2),
-    // dp = sum w (b + c), dm = sum w (b - c)
-    const T sb = T(0.5) * (gvp - gvm) + gdp + gdm;
-    const T sc = (gvp + gvm) * T(1.0 / 6.0) + gdp - gdm;
-    T gb[3], gc[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        gb[k] = S.w[k] * sb;
-        gc[k] = S.w[k] * sc;
-    }
-    gq[2] += gvp + gvm;
-    teno_bc_T(gb, gc, gq);
 }
 
-// transpose of teno_gauss at xi = g: cotangents of (v, d), added to gq[0..4]
+// transpose of teno_gauss_pm: cotangents of the values and derivatives at
+// xi = -g (gvm, gdm) and +g (gvp, gdp) -> gq[0..4]
 template <typename T>
-GKS_HD void teno_gauss_T(const TenoSel<T>& S, T g, T gv, T gd, T* gq)
+GKS_HD void teno_gauss_pm_T(const TenoSel<T>& S, T g, T gvm, T gdm, T gvp, T gdp, T* gq)
 {
-    gq[2] += gv;
+    const T gE = gvp + gvm, gO = g * (gvp - gvm), gEd = gdp + gdm, gOd = g * (gdp - gdm);
     if (S.large) {
-        // v = q2 + u1 g - u3 g/15 - u4/180, d = u1 + 2 u2 g + u3/10 - (2/21) u4 g
-        teno_u_T(g * gv + gd, T(2) * g * gd, g * gv * T(-1.0 / 15.0) + T(0.1) * gd,
-                 gv * T(-1.0 / 180.0) - T(2.0 / 21.0) * g * gd, gq);
-        return;
+        // E = q2 - R/4320, O = (43 A - 7 B)/72, Ed = P/12, Od = (12 C - D)/9, P = 7 A - B, R = D - 3 C
+        const T r = T(-1.0 / 4320.0) * gE, o = T(1.0 / 72.0) * gO, p = T(1.0 / 12.0) * gEd, d = T(1.0 / 9.0) * gOd;
+        teno_large_T(T(43) * o + T(7) * p, -(T(7) * o + p), T(12) * d - T(3) * r, r - d, gE, gq);
+    } else {
+        // E = q2, O = Ed = sb/2, Od = sc
+        teno_small_T(S, T(0.5) * (gO + gEd), gOd, gE, gq);
     }
-    // v = q2 + sum w b g, d = sum w (b + 2 c g)
-    T gb[3], gc[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        gb[k] = S.w[k] * (g * gv + gd);
-        gc[k] = S.w[k] * T(2) * g * gd;
-    }
-    teno_bc_T(gb, gc, gq);
 }
 
 // ------------------------------------------------------------------ kinetic layer (2-D)
@@ -151,14 +133,13 @@ GKS_HD void prim_vjp(T r, T ir, T U, T V, T q, T th, T gm1, PrimCot<T> c, T* gW)
 
 // Reverse of side_terms (NONEQ = false, 2-D): cotangents of the side's
 // contributions to W0, W0_n, W0_t -> cotangents of the side's W, Wn, Wt.
-template <bool UPPER, typename T>
-GKS_HD void side_vjp(const Side<T>& S, const Prim<T>& s, const FluxParams<T>& P, const T* gW0, const T* gW0n,
+template <typename T>
+GKS_HD void side_vjp(const Side<T>& S, const Prim<T>& s, T sg, const FluxParams<T>& P, const T* gW0, const T* gW0n,
                      const T* gW0t, Side<T>& gS)
 {
     // ---- forward values
     const T r = s.r, ir = s.ir, U = s.U, V = s.V, q = s.q;
     const T th = s.p * ir, sl = M<T>::rsqrt_(T(2) * th), hit = sl * sl;
-    const T sg = UPPER ? T(1) : T(-1);
     T u0, gz;
     half_space_start<T>(sl * U, sg, u0, gz);
     const T w = (sg * T(0.56418958354775628)) * (sl * gz), wt = th * w;
@@ -289,19 +270,19 @@ GKS_HD void equilibrium_vjp(const T* W0, const T* W0n, const T* W0t, const FluxP
 // Reverse of point_flux<T, 2, false, false> (tau = 0): cotangents of F and
 // dF/dt at one Gauss point -> cotangents of both sides.
 template <typename T>
-GKS_HD void point_flux_vjp(const Side<T>& L, const Side<T>& R, const FluxParams<T>& P, const T* gF, const T* gdF,
+GKS_HD void point_flux_vjp(const Side<T>& L, const Side<T>& R, T sg, const FluxParams<T>& P, const T* gF, const T* gdF,
                            Side<T>& gL, Side<T>& gR)
 {
     T W0[4], W0n[4], W0t[4];
     Prim<T> pl, pr;
     prim_state<T, 2>(L.W, P.gm1, pl);
     prim_state<T, 2>(R.W, P.gm1, pr);
-    side_terms<true, false, T, 2, false, false>(L, pl, P, W0, W0n, W0t, nullptr, nullptr, nullptr, nullptr, nullptr);
-    side_terms<false, true, T, 2, false, false>(R, pr, P, W0, W0n, W0t, nullptr, nullptr, nullptr, nullptr, nullptr);
+    side_terms<false, T, 2, false, false>(L, pl, sg, P, W0, W0n, W0t, nullptr, nullptr, nullptr, nullptr, nullptr);
+    side_terms<true, T, 2, false, false>(R, pr, -sg, P, W0, W0n, W0t, nullptr, nullptr, nullptr, nullptr, nullptr);
     T gW0[4] = {T(0), T(0), T(0), T(0)}, gW0n[4] = {T(0), T(0), T(0), T(0)}, gW0t[4] = {T(0), T(0), T(0), T(0)};
     equilibrium_vjp(W0, W0n, W0t, P, gF, gdF, gW0, gW0n, gW0t);
-    side_vjp<true>(L, pl, P, gW0, gW0n, gW0t, gL);
-    side_vjp<false>(R, pr, P, gW0, gW0n, gW0t, gR);
+    side_vjp(L, pl, sg, P, gW0, gW0n, gW0t, gL);
+    side_vjp(R, pr, -sg, P, gW0, gW0n, gW0t, gR);
 }
 
 }  // namespace gks

@@ -171,23 +171,20 @@ cudaError_t prof_harvest(gks_ctx* c)
 }
 
 // ---------------------------------------------------------------- launches
-// Ghost layers of W or W*.  On the float32 path the stage kernels read W* in
-// float32 (and, in 2-D, W through its float32 shadow), so those ghosts are
-// filled instead of the float64 ones.
 }  // namespace
 
 namespace gks {
 namespace rt {
 
-gks_status enqueue_ghosts(gks_ctx* c, double* arr, cudaStream_t st)
+gks_status fill_ghosts(gks_ctx* c, void* arr, cudaStream_t st)
 {
     const int gx = c->desc.nx + 2 * NG;
     const int n = (c->desc.dim == 1) ? 2 * NG : 2 * NG * gx + 2 * NG * c->desc.ny;
     const int pi = prof_begin(c, st, 1);
-    float* shadow = (arr == c->Ws) ? c->Wsf : (arr == c->W ? c->Wf : nullptr);
-    const double toff = (arr == c->Ws) ? 0.5 : 0.0;  // W* belongs to t + dt/2
-    if (shadow) k_fill_ghosts<float><<<(n + 127) / 128, 128, 0, st>>>(c->g, shadow, c->ds, toff);
-    else k_fill_ghosts<double><<<(n + 127) / 128, 128, 0, st>>>(c->g, arr, c->ds, toff);
+    if (c->desc.precision == GKS_FP32_FLUX)
+        k_fill_ghosts<float><<<(n + 127) / 128, 128, 0, st>>>(c->g, static_cast<float*>(arr), nullptr, 0.0);
+    else
+        k_fill_ghosts<double><<<(n + 127) / 128, 128, 0, st>>>(c->g, static_cast<double*>(arr), nullptr, 0.0);
     CK(cudaGetLastError());
     prof_end(c, st, pi);
     ++c->launches;

@@ -54,8 +54,9 @@ namespace rt {
 
 // records a formatted message in the context and returns s
 gks_status fail(gks_ctx* c, gks_status s, const char* fmt, ...);
-// fill the ghost layers of W or W* (the float32 shadow on the 2-D float32 path)
-gks_status enqueue_ghosts(gks_ctx* c, double* arr, cudaStream_t st);
+// fill the ghost layers of a state in the kernels' precision (float32 on the
+// float32 path) by the copying boundary rules
+gks_status fill_ghosts(gks_ctx* c, void* arr, cudaStream_t st);
 // fill the ghost layers of a float64 array at the state's time (whatever the
 // context's precision; diagnostics that read W itself)
 gks_status fill_ghosts_f64(gks_ctx* c, double* arr, cudaStream_t st);

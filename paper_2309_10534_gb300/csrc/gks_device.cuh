@@ -342,14 +342,16 @@ GKS_HD unsigned teno_code(const T t[4], T ct1, T ct2, int q)
     m = m < t[3] ? m : t[3];
     T p[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const T r = m * (T(1) / t[j]);
-        if (q == 7) {
-            const T r2 = r * r, r3 = r2 * r;
+    for (int j = 0; j < 4; ++j) p[j] = m * (T(1) / t[j]);
+    if (q == 7) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const T r = p[j], r2 = r * r, r3 = r2 * r;
             p[j] = r3 * r3 * r;
-        } else {
-            p[j] = ipow(r, q);
         }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[j] = ipow(p[j], q);
     }
     const T s012 = p[0] + p[1] + p[2];
     // first selection (Eqs. 4.6, 4.7): keep the large stencil when chi_{3,1} >= C_T1
@@ -410,15 +412,15 @@ GKS_HD unsigned teno_code_f32(const double q[5], const TenoT<double>& P)
                       + ((float)(781.0 / 720.0) * u3 * u3 + ((float)(1421461.0 / 327600.0) * R * R + eps4)));
     const float m = fminf(fminf(t0, t1), fminf(t2, t3));
     float p[4] = {quick_div(m, t0), quick_div(m, t1), quick_div(m, t2), quick_div(m, t3)};
+    if (P.q == 7) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float r = p[j];
-        if (P.q == 7) {
-            const float r2 = r * r, r3 = r2 * r;
+        for (int j = 0; j < 4; ++j) {
+            const float r = p[j], r2 = r * r, r3 = r2 * r;
             p[j] = r3 * r3 * r;
-        } else {
-            p[j] = ipow(r, P.q);
         }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[j] = ipow(p[j], P.q);
     }
     const float s012 = p[0] + p[1] + p[2];
     const float lim = P.fct1 * (s012 + p[3]), thr = P.fct2 * s012;
@@ -1239,9 +1241,10 @@ GKS_HD void merge_values(const T* Wl, const T* Wr, const FluxParams<T>& P, T* W0
 
 // One side's contributions to the equilibrium state (kinetic merge,
 // Eqs. 2.6, 3.25, 3.26) and to the non-equilibrium terms of Eq. (2.5): the
-// left side (UPPER, u > 0) or the right one; ADD to the sums, or set them.
-template <bool UPPER, bool ADD, typename T, int DIM, bool NONEQ, bool PRFIX>
-GKS_HD void side_terms(const Side<T>& S, const Prim<T>& pr, const FluxParams<T>& P, T* W0, T* W0n, T* W0t, T* S3, T* S4, T* S5, T* N4,
+// left side (sg = 1, u > 0) or the right one (sg = -1, u < 0); ADD to the
+// sums, or set them.
+template <bool ADD, typename T, int DIM, bool NONEQ, bool PRFIX>
+GKS_HD void side_terms(const Side<T>& S, const Prim<T>& pr, T sg, const FluxParams<T>& P, T* W0, T* W0n, T* W0t, T* S3, T* S4, T* S5, T* N4,
                        T* N5)
 {
     const T r = pr.r, U = pr.U, V = pr.V, q = pr.q, hv2 = pr.hv2;
@@ -1250,7 +1253,6 @@ GKS_HD void side_terms(const Side<T>& S, const Prim<T>& pr, const FluxParams<T>&
 
     // half-space u-moments: u > 0 (left state) or u < 0 (right state);
     // w = +- g(u = 0), the boundary value in the derivatives of u_0, u_1
-    const T sg = UPPER ? T(1) : T(-1);
     UMom<T> m;
     T gz;
     half_space_start<T>(sl * U, sg, m.u0, gz);
@@ -1373,7 +1375,8 @@ GKS_HD T tau_over_dt(const FluxParams<T>& P, T pl, T pr, T p0, T idt)
 }
 
 // F and dF/dt (per unit time; Sec. 2.2) at one interface point in the local
-// frame.  state(0, L, p) and state(1, R, p) form a side's primitive variables
+// frame, from the left and right sides (sg = 1; the other way round with
+// sg = -1).  state(0, L, p) and state(1, R, p) form a side's primitive variables
 // (prim_state) and apply the caller's fallback where it is not physical.
 // need_F = false: only dF is formed (the second stage uses nothing else).
 // W0n_lin, W0_lin, W0t_lin: the conventional path's equilibrium normal
@@ -1381,15 +1384,15 @@ GKS_HD T tau_over_dt(const FluxParams<T>& P, T pl, T pr, T p0, T idt)
 // slope (2-D: linear reconstructions of line-averaged merges, Step 4),
 // replacing the kinetic merge at the point; nullptr otherwise
 template <typename T, int DIM, bool NONEQ, bool PRFIX, typename State>
-GKS_HD void point_flux(Side<T>& L, Side<T>& R, const FluxParams<T>& P, T* F, T* dF, bool need_F, State&& state,
+GKS_HD void point_flux(Side<T>& L, Side<T>& R, T sg, const FluxParams<T>& P, T* F, T* dF, bool need_F, State&& state,
                        const T* W0n_lin = nullptr, const T* W0_lin = nullptr, const T* W0t_lin = nullptr)
 {
     T W0[4], W0n[4], W0t[4], S3[4], S4[4], S5[4], N4[4], N5[4];
     Prim<T> pl, pr;
     state(0, L, pl);
     state(1, R, pr);
-    side_terms<true, false, T, DIM, NONEQ, PRFIX>(L, pl, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
-    side_terms<false, true, T, DIM, NONEQ, PRFIX>(R, pr, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
+    side_terms<false, T, DIM, NONEQ, PRFIX>(L, pl, sg, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
+    side_terms<true, T, DIM, NONEQ, PRFIX>(R, pr, -sg, P, W0, W0n, W0t, S3, S4, S5, N4, N5);
     // the kinetic merge is also the density moment of the side terms (the
     // heat flux needs it even where W0 is replaced below)
     T W0k[4];
@@ -1479,7 +1482,7 @@ struct PlainState {
 template <typename T, int DIM, bool NONEQ, bool PRFIX>
 GKS_HD void point_flux(Side<T>& L, Side<T>& R, const FluxParams<T>& P, T* F, T* dF)
 {
-    point_flux<T, DIM, NONEQ, PRFIX>(L, R, P, F, dF, true, PlainState<T, DIM>{P.gm1});
+    point_flux<T, DIM, NONEQ, PRFIX>(L, R, T(1), P, F, dF, true, PlainState<T, DIM>{P.gm1});
 }
 
 }  // namespace gks

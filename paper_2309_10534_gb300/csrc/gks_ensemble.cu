@@ -167,7 +167,7 @@ __device__ void stage_chunk(ChunkSmem<T, NT>& sm, double* W, float* Wf, T* Ws, T
             if (!prim_state<T, 1>(S.W, fp.gm1, p)) err |= 2u;
         };
         T F[4], dF[4];
-        point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, stage == 1, state);
+        point_flux<T, 1, NONEQ, PRFIX>(L, R, T(1), fp, F, dF, stage == 1, state);
 #pragma unroll
         for (int v = 0; v < 3; ++v) stage_comb<T>(stage, F[slot[v]], dF[slot[v]], tdt, sm.G[0][v][f], sm.G[1][v][f]);
     }

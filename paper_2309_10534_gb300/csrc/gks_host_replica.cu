@@ -112,10 +112,10 @@ int teno_vjp_t(const double* q, double eps, int qpow, double ct1, double ct2, co
     const gks::TenoParams P{eps, qpow, ct1, ct2};
     gks::TenoSel<T> S;
     gks::teno_select(qq, gks::teno_t<T>(P), S);
+    T h[5];
     gks::teno_faces_T(S, (T)gfaces[0], (T)gfaces[1], (T)gfaces[2], (T)gfaces[3], g);
-    gks::teno_gauss_T(S, T(-0.28867513459481288), (T)ggauss[0], (T)ggauss[1], g);
-    gks::teno_gauss_T(S, T(0.28867513459481288), (T)ggauss[2], (T)ggauss[3], g);
-    for (int k = 0; k < 5; ++k) gq[k] = (double)g[k];
+    gks::teno_gauss_pm_T(S, T(0.28867513459481288), (T)ggauss[0], (T)ggauss[1], (T)ggauss[2], (T)ggauss[3], h);
+    for (int k = 0; k < 5; ++k) gq[k] = (double)(g[k] + h[k]);
     return S.large ? 1 : 0;
 }
 
@@ -141,7 +141,7 @@ int flux_vjp_t(double gamma, const double* Wl, const double* Wln, const double* 
         f[k] = (T)gF[k];
         d[k] = (T)gdF[k];
     }
-    gks::point_flux_vjp(L, R, p, f, d, gL, gR);
+    gks::point_flux_vjp(L, R, T(1), p, f, d, gL, gR);
     for (int k = 0; k < 4; ++k) {
         gl[k] = gL.W[k]; gl[4 + k] = gL.Wn[k]; gl[8 + k] = gL.Wt[k];
         gr[k] = gR.W[k]; gr[4 + k] = gR.Wn[k]; gr[8 + k] = gR.Wt[k];

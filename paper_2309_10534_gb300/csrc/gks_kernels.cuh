@@ -425,9 +425,9 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
             for (int v = 0; v < 3; ++v)
                 w0n[slot[v]] = (T(1.25) * (sq[v][f + 3] - sq[v][f + 2]) - T(1.0 / 12.0) * (sq[v][f + 4] - sq[v][f + 1]))
                              * idx_;
-            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state, w0n);
+            point_flux<T, 1, NONEQ, PRFIX>(L, R, T(1), fp, F, dF, a.stage == 1, state, w0n);
         } else {
-            point_flux<T, 1, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state);
+            point_flux<T, 1, NONEQ, PRFIX>(L, R, T(1), fp, F, dF, a.stage == 1, state);
         }
         const T tdt = s_scal[0];
 #pragma unroll
@@ -601,8 +601,7 @@ __global__ void __launch_bounds__(96) k1d_stage_wide(const __grid_constant__ Gri
             if (!prim_state<T, 1>(S.W, fp.gm1, p)) err |= 2u;
         }
         T W0[4], W0n[4], W0t[4], S3[4], S4[4], S5[4];
-        if (warp == 0) side_terms<true, false, T, 1, NONEQ, false>(S, p, fp, W0, W0n, W0t, S3, S4, S5, nullptr, nullptr);
-        else side_terms<false, false, T, 1, NONEQ, false>(S, p, fp, W0, W0n, W0t, S3, S4, S5, nullptr, nullptr);
+        side_terms<false, T, 1, NONEQ, false>(S, p, warp ? T(-1) : T(1), fp, W0, W0n, W0t, S3, S4, S5, nullptr, nullptr);
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
             sS[warp][v][f] = W0[slot[v]];
@@ -742,9 +741,13 @@ struct SweepArgs {
 // global variable index of local variable v (swap: faces normal to y)
 __device__ __forceinline__ int gvar(int v, bool swap) { return (swap && (v == 1 || v == 2)) ? 3 - v : v; }
 
+template <typename T> struct alignas(2 * sizeof(T)) Pair2 {
+    T v, s;
+};
+
 template <typename T, int TN, int TT, bool CONV = false> struct SweepSmem {
     T w[4][TT + 4][TN + 6];           // cells: tangential rows t0-2.., normal n0-3..
-    T rec[4][4][TT + 4][TN + 1];      // [vL, sL, vR, sR][var][row][face]
+    Pair2<T> rec[2][4][TT + 4][TN + 1];  // [side][var][row][face]: value and normal slope
     T flux[8 * (TN + 1) * (TT + 1)];  // face fluxes for the update (layout: sfi)
     // conventional path: line-averaged equilibrium state and its normal
     // slope per face and row (Step 2)
@@ -863,10 +866,8 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
             char_face<T, 2>(w, tnn, fp.gm1, vl, dl, vr, dr);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                sm.rec[0][v][r][f] = vl[v];
-                sm.rec[1][v][r][f] = dl[v] * ih;
-                sm.rec[2][v][r][f] = vr[v];
-                sm.rec[3][v][r][f] = dr[v] * ih;
+                sm.rec[0][v][r][f] = {vl[v], dl[v] * ih};
+                sm.rec[1][v][r][f] = {vr[v], dr[v] * ih};
             }
         }
     } else if constexpr (sizeof(T) == 4 && REC <= 1) {
@@ -887,12 +888,12 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
             packed_faces<REC>(q, tnn, vp, dp, vm, dm);
             const f2 dpi = dp * f2(ih), dmi = dm * f2(ih);
             if (c <= TN) {
-                sm.rec[0][vv][r][c] = vp.x(); sm.rec[0][vv + 1][r][c] = vp.y();
-                sm.rec[1][vv][r][c] = dpi.x(); sm.rec[1][vv + 1][r][c] = dpi.y();
+                sm.rec[0][vv][r][c] = {vp.x(), dpi.x()};
+                sm.rec[0][vv + 1][r][c] = {vp.y(), dpi.y()};
             }
             if (c >= 1) {
-                sm.rec[2][vv][r][c - 1] = vm.x(); sm.rec[2][vv + 1][r][c - 1] = vm.y();
-                sm.rec[3][vv][r][c - 1] = dmi.x(); sm.rec[3][vv + 1][r][c - 1] = dmi.y();
+                sm.rec[1][vv][r][c - 1] = {vm.x(), dmi.x()};
+                sm.rec[1][vv + 1][r][c - 1] = {vm.y(), dmi.y()};
             }
         }
     } else {
@@ -910,8 +911,8 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
             rec_select<REC>(q, tnn, S);
             T vp, dp, vm, dm;
             rec_faces<REC>(q, S, vp, dp, vm, dm);
-            if (c <= TN) { sm.rec[0][v][r][c] = vp; sm.rec[1][v][r][c] = dp * ih; }
-            if (c >= 1) { sm.rec[2][v][r][c - 1] = vm; sm.rec[3][v][r][c - 1] = dm * ih; }
+            if (c <= TN) sm.rec[0][v][r][c] = {vp, dp * ih};
+            if (c >= 1) sm.rec[1][v][r][c - 1] = {vm, dm * ih};
         }
     }
     __syncthreads();
@@ -930,7 +931,7 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
             if (n0 + f > a.nn || t0 - 2 + r > a.nt + 1) continue;
             T wl[4], wr[4], w0[4];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) { wl[v] = sm.rec[0][v][r][f]; wr[v] = sm.rec[2][v][r][f]; }
+            for (int v = 0; v < 4; ++v) { wl[v] = sm.rec[0][v][r][f].v; wr[v] = sm.rec[1][v][r][f].v; }
             if (!physical<T, 2>(wl, fp.gm1)) {
 #pragma unroll
                 for (int v = 0; v < 4; ++v) wl[v] = sm.w[v][r][f + 2];
@@ -955,8 +956,11 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     // phase 2: per (face segment, Gauss point): tangential TENO-D of the line
     // averages to the Gauss point, then merge + flux.  The two lanes of a face
     // segment split the work: lane gpi reconstructs side gpi (0: left, 1:
-    // right) at both Gauss points, keeps its own point and hands the other
-    // point's values to its partner; after the flux they average (weights 1/2).
+    // right) at both Gauss points, keeps its own point (xi = -g for lane 0, +g
+    // for lane 1: one signed g, no selection) and hands the other point's
+    // values to its partner.  A lane's own side goes first into the flux,
+    // whose sign says which of the two that is; after it they average
+    // (weights 1/2).
     const T tdt = s_scal[0];
     const T iht = s_scal[3];
     const T gA = T(-0.28867513459481288), gB = T(0.28867513459481288);  // -+1/(2 sqrt 3)
@@ -966,51 +970,52 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
         const int r = pair / NF, f = pair % NF;
         // faces n0+f <= nn on rows t0+r < nt exist; the rest of the tile is padding
         const bool valid = (n0 + f <= a.nn) && (t0 + r < a.nt);
-        Side<T> L, R;
+        const T gs = gpi ? gB : gA;
+        Side<T> L, R;  // own side, partner's side
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             // line averages of the side's value (W) and normal slope (Wn) at
-            // the two Gauss points: value and tangential derivative of W,
-            // value of Wn
+            // the own (a) and the partner's (b) Gauss point: value and
+            // tangential derivative of W, value of Wn
             T wa, wda, wb, wdb, na, nb;
             if constexpr (sizeof(T) == 4 && RB <= 1) {
                 // both streams as one packed pair (x: W, y: Wn)
                 f2 q[5];
 #pragma unroll
-                for (int s = 0; s < 5; ++s) q[s] = f2(sm.rec[2 * gpi][v][r + s][f], sm.rec[2 * gpi + 1][v][r + s][f]);
+                for (int s = 0; s < 5; ++s) {
+                    const Pair2<T> p = sm.rec[gpi][v][r + s][f];
+                    q[s] = f2(p.v, p.s);
+                }
                 f2 va, da, vb, db;
-                packed_gauss<RB>(q, tnt, gA, gB, va, da, vb, db);
+                packed_gauss<RB>(q, tnt, -gs, gs, vb, db, va, da);
                 wa = va.x(), wda = da.x(), wb = vb.x(), wdb = db.x(), na = va.y(), nb = vb.y();
             } else {
-                T q[5];
+                T q[5], qs[5];
                 TenoSel<T> S;
                 T dn;
 #pragma unroll
-                for (int s = 0; s < 5; ++s) q[s] = sm.rec[2 * gpi][v][r + s][f];
+                for (int s = 0; s < 5; ++s) {
+                    const Pair2<T> p = sm.rec[gpi][v][r + s][f];
+                    q[s] = p.v;
+                    qs[s] = p.s;
+                }
                 rec_select<RB>(q, tnt, S);
-                rec_gauss_pm<RB>(S, gB, wa, wda, wb, wdb);  // gA = -gB
-#pragma unroll
-                for (int s = 0; s < 5; ++s) q[s] = sm.rec[2 * gpi + 1][v][r + s][f];
-                rec_select<RB>(q, tnt, S);
-                rec_gauss_pm<RB>(S, gB, na, dn, nb, dn);
+                rec_gauss_pm<RB>(S, gs, wb, wdb, wa, wda);
+                rec_select<RB>(qs, tnt, S);
+                rec_gauss_pm<RB>(S, gs, nb, dn, na, dn);
             }
-            // own side at own point; the partner's point goes to the partner
-            T own = gpi ? wb : wa, got = __shfl_xor_sync(0xffffffffu, gpi ? wa : wb, 1);
-            L.W[v] = gpi ? got : own;
-            R.W[v] = gpi ? own : got;
-            own = (gpi ? wdb : wda) * iht;
-            got = __shfl_xor_sync(0xffffffffu, (gpi ? wda : wdb) * iht, 1);
-            L.Wt[v] = gpi ? got : own;
-            R.Wt[v] = gpi ? own : got;
-            own = gpi ? nb : na;
-            got = __shfl_xor_sync(0xffffffffu, gpi ? na : nb, 1);
-            L.Wn[v] = gpi ? got : own;
-            R.Wn[v] = gpi ? own : got;
+            L.W[v] = wa;
+            R.W[v] = __shfl_xor_sync(0xffffffffu, wb, 1);
+            L.Wt[v] = wda * iht;
+            R.Wt[v] = __shfl_xor_sync(0xffffffffu, wdb, 1) * iht;
+            L.Wn[v] = na;
+            R.Wn[v] = __shfl_xor_sync(0xffffffffu, nb, 1);
         }
         T F[4] = {T(0), T(0), T(0), T(0)}, dF[4] = {T(0), T(0), T(0), T(0)};
         if (valid) {
-            auto state = [&](int side, Side<T>& S, Prim<T>& p) {
+            auto state = [&](int k, Side<T>& S, Prim<T>& p) {
                 if (prim_state<T, 2>(S.W, fp.gm1, p)) return;
+                const int side = k ^ gpi;  // 0: left, 1: right
 #pragma unroll
                 for (int v = 0; v < 4; ++v) { S.W[v] = sm.w[v][r + 2][f + 2 + side]; S.Wn[v] = S.Wt[v] = T(0); }
                 ++nfb;
@@ -1020,28 +1025,27 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
                 // Step 4: the equilibrium state and slopes at this lane's Gauss
                 // point, linear (quartic) reconstructions of the rows' merges
                 T w0g[4], w0t[4], w0n[4];
-                const T gme = gpi ? gB : gA;
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     T q[5], dd;
 #pragma unroll
                     for (int s = 0; s < 5; ++s) q[s] = sm.w0[0][v][r + s][f];
-                    quartic_gauss(q, gme, w0g[v], dd);
+                    quartic_gauss(q, gs, w0g[v], dd);
                     w0t[v] = dd * iht;
 #pragma unroll
                     for (int s = 0; s < 5; ++s) q[s] = sm.w0[1][v][r + s][f];
-                    quartic_gauss(q, gme, w0n[v], dd);
+                    quartic_gauss(q, gs, w0n[v], dd);
                 }
                 // a non-physical linear state (the quartic across a
                 // discontinuity) falls back to the kinetic merge at the point
                 if (physical<T, 2>(w0g, fp.gm1)) {
-                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state, w0n, w0g, w0t);
+                    point_flux<T, 2, NONEQ, PRFIX>(L, R, gpi ? T(-1) : T(1), fp, F, dF, a.stage == 1, state, w0n, w0g, w0t);
                 } else {
                     ++nfb;
-                    point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state);
+                    point_flux<T, 2, NONEQ, PRFIX>(L, R, gpi ? T(-1) : T(1), fp, F, dF, a.stage == 1, state);
                 }
             } else {
-                point_flux<T, 2, NONEQ, PRFIX>(L, R, fp, F, dF, a.stage == 1, state);
+                point_flux<T, 2, NONEQ, PRFIX>(L, R, gpi ? T(-1) : T(1), fp, F, dF, a.stage == 1, state);
             }
         }
         // the stage's combinations at both points, averaged (weights 1/2): each

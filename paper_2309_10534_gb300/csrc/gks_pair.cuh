@@ -111,14 +111,16 @@ GKS_HD void teno_select_x2(const f2 q[5], const TenoT<float>& P, TenoSel2& S)
     const f2 m(lane_min4(t[0].x(), t[1].x(), t[2].x(), t[3].x()), lane_min4(t[0].y(), t[1].y(), t[2].y(), t[3].y()));
     f2 p[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const f2 r = m * f2(1.0f / t[j].x(), 1.0f / t[j].y());
-        if (P.q == 7) {
-            const f2 r2 = r * r, r3 = r2 * r;
+    for (int j = 0; j < 4; ++j) p[j] = m * f2(1.0f / t[j].x(), 1.0f / t[j].y());
+    if (P.q == 7) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const f2 r = p[j], r2 = r * r, r3 = r2 * r;
             p[j] = r3 * r3 * r;
-        } else {
-            p[j] = f2(ipow(r.x(), P.q), ipow(r.y(), P.q));
         }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[j] = f2(ipow(p[j].x(), P.q), ipow(p[j].y(), P.q));
     }
     const f2 s012 = p[0] + p[1] + p[2];
     const f2 lim = f2(P.ct1) * (s012 + p[3]);
