@@ -332,6 +332,24 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
     const int slot[3] = {0, 1, 3};
 
     const int pl = (int)g.plane;  // a 1-D plane is one ghosted row
+    // the update's other inputs, requested before the stage's arithmetic: read
+    // in the update they cost its warps a memory round trip each (four steps of
+    // a 2^22-cell float32 tube 1702 -> 1688 us)
+    const int ui = i0 + tid, uo = ui + NG;
+    const bool own = tid < TN && ui < g.nx;
+    double ubase[3] = {0.0, 0.0, 0.0};
+    T uacc[3] = {T(0), T(0), T(0)};
+    if (own && (a.stage == 2 || sizeof(T) == 8)) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            if constexpr (sizeof(T) == 4) {
+                ubase[v] = a.base[v * pl + uo];
+                uacc[v] = a.accf[v * pl + uo];
+            } else {
+                ubase[v] = a.stage == 1 ? a.src[v * pl + uo] : a.acc[v * pl + uo];
+            }
+        }
+    }
     // one loop per source type: a per-element choice between the float32
     // and the converted float64 source was compiled as both, and every
     // element then paid a float64 -> float32 conversion on the slow float64
@@ -438,46 +456,30 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
     T sig = T(0);
     const double cx = dt * a.idx;
     const T cxt = s_scal[1];
-    for (int c = tid; c < TN; c += NT) {
-        const int i = i0 + c;
-        if (i >= g.nx) continue;
-        const int o = i + NG;
-        if constexpr (sizeof(T) == 4) {
-            if (a.stage == 1) {
+    if (own) {
+        const int c = tid, o = uo;
+        T w[4];
 #pragma unroll
-                for (int v = 0; v < 3; ++v) {
-                    a.out0f[v * pl + o] = wstar32(sq[v][c + 3], cxt, sG[0][v][c + 1] - sG[0][v][c]);
+        for (int v = 0; v < 3; ++v) {
+            const T d0 = sG[0][v][c + 1] - sG[0][v][c];
+            if constexpr (sizeof(T) == 4) {
+                if (a.stage == 1) {
+                    a.out0f[v * pl + o] = wstar32(sq[v][c + 3], cxt, d0);
                     a.out1f[v * pl + o] = cxt * (sG[1][v][c + 1] - sG[1][v][c]);
+                } else {
+                    const double r = wnew32(ubase[v], uacc[v], cxt, d0);
+                    a.out0[v * pl + o] = r;
+                    w[v] = narrow(r);
+                    if (a.out0f) a.out0f[v * pl + o] = w[v];
                 }
             } else {
-                T w[3];
-#pragma unroll
-                for (int v = 0; v < 3; ++v) {
-                    const int gi = v * pl + o;
-                    const double r = wnew32(a.base[gi], a.accf[gi], cxt, sG[0][v][c + 1] - sG[0][v][c]);
-                    a.out0[gi] = r;
-                    w[v] = narrow(r);
-                    if (a.out0f) a.out0f[gi] = w[v];
-                }
-                if (a.with_sigma) sig = fmax(sig, cell_sigma<T, T>(w, 1, s_scal[3], s_scal[4], s_scal[5], err));
-            }
-        } else if (a.stage == 1) {
-#pragma unroll
-            for (int v = 0; v < 3; ++v) {
-                const double w = a.src[v * pl + o];
-                a.out0[v * pl + o] = upd64(w, cx, (double)(sG[0][v][c + 1] - sG[0][v][c]));
-                a.out1[v * pl + o] = upd64(w, cx, (double)(sG[1][v][c + 1] - sG[1][v][c]));
-            }
-        } else {
-            double w[4];
-#pragma unroll
-            for (int v = 0; v < 3; ++v) {
-                const double r = upd64(a.acc[v * pl + o], cx, (double)(sG[0][v][c + 1] - sG[0][v][c]));
+                const double r = upd64(ubase[v], cx, (double)d0);
                 a.out0[v * pl + o] = r;
-                w[v] = r;
+                if (a.stage == 1) a.out1[v * pl + o] = upd64(ubase[v], cx, (double)(sG[1][v][c + 1] - sG[1][v][c]));
+                w[v] = (T)r;
             }
-            if (a.with_sigma) sig = fmax(sig, cell_sigma<T>(w, 1, s_scal[3], s_scal[4], s_scal[5], err));
         }
+        if (a.with_sigma) sig = cell_sigma<T, T>(w, 1, s_scal[3], s_scal[4], s_scal[5], err);
     }
     if (NT % 32 == 0) block_commit<NT, T>(sig, a.with_sigma != 0, err, nfb, ds, a.commit != 0);
 }
@@ -749,10 +751,25 @@ template <typename T, int TN, int TT, bool CONV = false> struct SweepSmem {
     T w[4][TT + 4][TN + 6];           // cells: tangential rows t0-2.., normal n0-3..
     Pair2<T> rec[2][4][TT + 4][TN + 1];  // [side][var][row][face]: value and normal slope
     T flux[8 * (TN + 1) * (TT + 1)];  // face fluxes for the update (layout: sfi)
+    // y sweep: the update's inputs, copied while the sweep computes
+    double base[4][TN * TT];             // W or A (float32 stage 1: its float32 shadow, in the first half)
+    T inc[2][4][TN * TT];                // the x sweep's increments
     // conventional path: line-averaged equilibrium state and its normal
     // slope per face and row (Step 2)
     T w0[CONV ? 2 : 1][4][CONV ? TT + 4 : 1][CONV ? TN + 1 : 1];
 };
+
+// 4- or 8-byte copies from global to shared memory that the thread waits for
+// only when it reads them
+template <int B>
+__device__ __forceinline__ void copy_async(void* dst, const void* src)
+{
+    static_assert(B == 4 || B == 8, "cp.async size");
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if constexpr (B == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // the cells of a tile that reaches past the boundary, ghosts by the boundary
 // rules (out of line: the other tiles keep their registers)
@@ -844,6 +861,28 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
             const int v = k / (CN * CT), e = k % (CN * CT);
             if (!fy) cell(v, e % CN, e / CN);
             else cell(v, e / CT, e % CT);
+        }
+    }
+    // y sweep: start copying the update's inputs (read in the update, they
+    // cost its warps a memory round trip: four steps of a 64^2 float32 plane
+    // 292 -> 281 us, two of a 1024^2 plane the same)
+    const bool base_f = sizeof(T) == 4 && a.stage == 1;
+    if (a.pass == 1) {
+        for (int k = tid; k < TN * TT; k += NT) {
+            const int r = fy ? k % TT : k / TN, c = fy ? k / TT : k % TN;
+            const int in = n0 + c, it = t0 + r;
+            if (in < a.nn && it < a.nt) {
+                const int o = org + in * sn + it * st;
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const long long go = (v == 0 ? 0 : (v == 1 ? pv1 : (v == 2 ? pv2 : pv3))) + o;
+                    if (base_f) copy_async<4>(reinterpret_cast<float*>(sm.base[v]) + k, a.basef + go);
+                    else copy_async<8>(&sm.base[v][k], a.base + go);
+                    copy_async<sizeof(T)>(&sm.inc[0][v][k], static_cast<const T*>(a.inc0) + go);
+                    if (a.stage == 1 || sizeof(T) == 4)
+                        copy_async<sizeof(T)>(&sm.inc[1][v][k], static_cast<const T*>(a.inc1) + go);
+                }
+            }
         }
     }
     __syncthreads();
@@ -1071,7 +1110,9 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     }
     __syncthreads();
 
-    // phase 3: flux divergence; the y sweep updates the float64 state
+    // phase 3: flux divergence; the y sweep updates the float64 state.  Each
+    // thread reads the inputs it copied itself
+    copy_wait();
     T sig = T(0);
     const T cn = s_scal[1];
     static_assert((2 * NP) % NT == 0, "whole warps of tasks");
@@ -1098,20 +1139,20 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
                     if (a.stage == 1) inc1[go] = d1;
                 } else if constexpr (sizeof(T) == 4) {
                     if (a.stage == 1) {
-                        a.out0f[go] = a.basef[go] - (inc0[go] + d0);
-                        inc1[go] = inc1[go] + d1;
+                        a.out0f[go] = reinterpret_cast<const float*>(sm.base[v])[k] - (sm.inc[0][v][k] + d0);
+                        inc1[go] = sm.inc[1][v][k] + d1;
                     } else {
-                        const double res = a.base[go] - widen(inc1[go] + inc0[go] + d0);
+                        const double res = sm.base[v][k] - widen(sm.inc[1][v][k] + sm.inc[0][v][k] + d0);
                         a.out0[go] = res;
                         wf[v] = narrow(res);  // local order; the CFL rate only needs |U|
                         a.out0f[go] = wf[v];
                     }
                 } else if (a.stage == 1) {
-                    const double w = a.base[go];
-                    a.out0[go] = w - (double)(inc0[go] + d0);
-                    a.out1[go] = w - (double)(inc1[go] + d1);
+                    const double w = sm.base[v][k];
+                    a.out0[go] = w - (double)(sm.inc[0][v][k] + d0);
+                    a.out1[go] = w - (double)(sm.inc[1][v][k] + d1);
                 } else {
-                    const double res = a.base[go] - (double)(inc0[go] + d0);
+                    const double res = sm.base[v][k] - (double)(sm.inc[0][v][k] + d0);
                     a.out0[go] = res;
                     wn[v] = res;  // local order; the CFL rate only needs |U|
                 }
