@@ -327,6 +327,7 @@ gks_status sync_state(gks_ctx* c)
 {
     CK(cudaMemcpyAsync(c->hs, c->ds, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    c->hs_fresh = true;
     return GKS_OK;
 }
 
@@ -345,7 +346,7 @@ gks_status check_err(gks_ctx* c)
 namespace gks {
 namespace rt {
 
-gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device, bool in)
+gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device, bool in, bool wait)
 {
     // A caller's array [nv][ny][nx] is moved in one contiguous copy (host
     // arrays through a device staging buffer) and scattered into / gathered
@@ -372,7 +373,7 @@ gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device
     if (host && !in)
         CK(cudaMemcpyAsync(const_cast<double*>(W), c->stage, sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost,
                            c->stream));
-    if (on_device != GKS_HOST_PINNED_ASYNC) CK(cudaStreamSynchronize(c->stream));
+    if (wait && on_device != GKS_HOST_PINNED_ASYNC) CK(cudaStreamSynchronize(c->stream));
     return GKS_OK;
 }
 
@@ -382,33 +383,33 @@ using gks::rt::copy_interior;
 
 namespace {
 
-gks_status build_graph(gks_ctx* c)
+gks_status build_graph(gks_ctx* c, gks_ctx::StepGraph& sg, int steps)
 {
-    if (c->graph && c->graph_version == c->param_version) return GKS_OK;
-    if (c->graph) {
-        cudaGraphExecDestroy(c->graph);
-        c->graph = nullptr;
+    if (sg.exec && sg.version == c->param_version) return GKS_OK;
+    if (sg.exec) {
+        cudaGraphExecDestroy(sg.exec);
+        sg.exec = nullptr;
     }
     if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     const long long before = c->launches;
     CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     c->capturing = true;
     gks_status s = GKS_OK;
-    for (int k = 0; k < GRAPH_STEPS && s == GKS_OK; ++k) s = enqueue_step(c, c->cap_stream);
+    for (int k = 0; k < steps && s == GKS_OK; ++k) s = enqueue_step(c, c->cap_stream);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
     c->capturing = false;
-    c->graph_nodes = c->launches - before;
+    sg.nodes = c->launches - before;
     c->launches = before;  // captured, not launched
     if (s != GKS_OK) {
         if (graph) cudaGraphDestroy(graph);
         return s;
     }
     CK(e);
-    e = cudaGraphInstantiate(&c->graph, graph, 0);
+    e = cudaGraphInstantiate(&sg.exec, graph, 0);
     cudaGraphDestroy(graph);
     CK(e);
-    c->graph_version = c->param_version;
+    sg.version = c->param_version;
     return GKS_OK;
 }
 
@@ -583,7 +584,8 @@ gks_status gks_create(const gks_grid_desc* d, gks_ctx** out)
 void gks_destroy(gks_ctx* c)
 {
     if (!c) return;
-    if (c->graph) cudaGraphExecDestroy(c->graph);
+    if (c->graph.exec) cudaGraphExecDestroy(c->graph.exec);
+    if (c->graph1.exec) cudaGraphExecDestroy(c->graph1.exec);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     for (auto& p : c->ev) {
         cudaEventDestroy(p.a);
@@ -660,7 +662,8 @@ gks_status gks_set_state(gks_ctx* c, const double* W, int on_device)
 {
     if (!c || !W) return GKS_EINVAL;
     c->cfl_dt_ready = false;
-    gks_status s = copy_interior(c, c->W, W, on_device, true);
+    c->hs_fresh = false;
+    gks_status s = copy_interior(c, c->W, W, on_device, true, false);
     if (s) return s;
     if (c->Wf) {
         const long long n = (long long)c->nv * c->g.plane;
@@ -723,7 +726,7 @@ gks_status gks_stage(gks_ctx* c, int stage, double dt)
 {
     const NvtxRange range("gks_stage");
     if (!c || (stage != 1 && stage != 2) || !(dt > 0.0) || !std::isfinite(dt)) return GKS_EINVAL;
-    c->cfl_dt_ready = false;
+    c->cfl_dt_ready = c->hs_fresh = false;
     k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 0, dt, 0.0, 0);
     CK(cudaGetLastError());
     ++c->launches;
@@ -735,6 +738,7 @@ gks_status gks_step(gks_ctx* c, double dt)
     const NvtxRange range("gks_step");
     if (!c || !std::isfinite(dt)) return GKS_EINVAL;
     gks_status s;
+    c->hs_fresh = false;
     if (dt > 0.0) {
         c->cfl_dt_ready = false;
         k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 0, dt, 0.0, 0);
@@ -759,23 +763,33 @@ gks_status gks_advance_to(gks_ctx* c, double t_end, long long max_steps, long lo
     if (!c || !std::isfinite(t_end)) return GKS_EINVAL;
     c->cfl_dt_ready = false;
     gks_status s;
-    if ((s = sync_state(c))) return s;
+    if (!c->hs_fresh && (s = sync_state(c))) return s;
     const long long steps0 = c->hs->steps;
     if (!(c->hs->t < t_end)) {
         if (steps_done) *steps_done = 0;
         if (t_out) *t_out = c->hs->t;
         return GKS_OK;
     }
+    c->hs_fresh = false;
     const long long limit = max_steps > 0 ? steps0 + max_steps : 0;
     k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 1, 0.0, t_end, limit);
     CK(cudaGetLastError());
     ++c->launches;
     if ((s = enqueue_sigma(c, c->stream))) return s;
     if ((s = enqueue_first_dt(c, c->stream))) return s;
-    if ((s = build_graph(c))) return s;
+    long long left = limit ? limit - steps0 : GRAPH_STEPS;
     for (;;) {
-        CK(cudaGraphLaunch(c->graph, c->stream));
-        c->launches += c->graph_nodes;
+        // the last few steps of a limited call one by one: a full replay
+        // would launch the steps beyond the limit too, each to return at once
+        const bool single = limit && left < GRAPH_STEPS;
+        gks_ctx::StepGraph& sg = single ? c->graph1 : c->graph;
+        if ((s = build_graph(c, sg, single ? 1 : GRAPH_STEPS))) return s;
+        const int replays = single ? (int)left : 1;
+        for (int k = 0; k < replays; ++k) {
+            CK(cudaGraphLaunch(sg.exec, c->stream));
+            c->launches += sg.nodes;
+        }
+        if (limit) left -= GRAPH_STEPS;
         if ((s = sync_state(c))) return s;
         if ((s = check_err(c))) return s;
         if (c->hs->done) break;

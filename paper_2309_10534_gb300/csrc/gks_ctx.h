@@ -29,9 +29,15 @@ struct gks_ctx {
     gks::DevState* hs = nullptr;      // pinned host mirror
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t graph = nullptr;
-    long long graph_nodes = 0;
-    unsigned long long param_version = 1, graph_version = 0;
+    // captured steps: GRAPH_STEPS of them, and a single one for what is left
+    // of a call's max_steps
+    struct StepGraph {
+        cudaGraphExec_t exec = nullptr;
+        long long nodes = 0;
+        unsigned long long version = 0;
+    } graph, graph1;
+    unsigned long long param_version = 1;
+    bool hs_fresh = false;  // hs holds the device state's time and step count
     long long launches = 0;
     // the device already holds the CFL time step of the current state (set by
     // a CFL step's commit, cleared by anything else that changes W or dt)
@@ -61,7 +67,8 @@ gks_status fill_ghosts(gks_ctx* c, void* arr, cudaStream_t st);
 // context's precision; diagnostics that read W itself)
 gks_status fill_ghosts_f64(gks_ctx* c, double* arr, cudaStream_t st);
 // copy the interior [nv][ny][nx] between a caller's buffer and a ghosted array
-gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device, bool in);
+// (wait = false: the caller synchronises the stream before it returns)
+gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device, bool in, bool wait = true);
 HostFlux host_flux(const gks_ctx* c);
 TenoParams teno_params(const gks_ctx* c, bool tangential);
 
