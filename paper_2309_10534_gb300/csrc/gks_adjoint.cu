@@ -160,9 +160,9 @@ __device__ __forceinline__ unsigned fwd_faces2(const T qa[5], const T qb[5], con
 #pragma unroll
         for (int s = 0; s < 5; ++s) qq[s] = f2(qa[s], qb[s]);
         TenoSel2 S2;
-        teno_select_x2(qq, P, S2);
         f2 a, b, c, d;
-        teno_faces_x2(S2, a, b, c, d);
+        if (teno_select_x2(qq, P, S2)) teno_faces_x2(S2, true, a, b, c, d);
+        else teno_faces_x2(S2, false, a, b, c, d);
         vp[0] = a.x(); dp[0] = b.x(); vm[0] = c.x(); dm[0] = d.x();
         vp[1] = a.y(); dp[1] = b.y(); vm[1] = c.y(); dm[1] = d.y();
         return sel_code_x(S2) | (sel_code_y(S2) << 4);
@@ -188,9 +188,9 @@ __device__ __forceinline__ unsigned fwd_gauss2(const T qa[5], const T qb[5], con
 #pragma unroll
         for (int s = 0; s < 5; ++s) qq[s] = f2(qa[s], qb[s]);
         TenoSel2 S2;
-        teno_select_x2(qq, P, S2);
         f2 a, b, c, d;
-        teno_gauss_pm_x2(S2, gB, a, b, c, d);  // gA = -gB
+        if (teno_select_x2(qq, P, S2)) teno_gauss_pm_x2(S2, true, gB, a, b, c, d);  // gA = -gB
+        else teno_gauss_pm_x2(S2, false, gB, a, b, c, d);
         va[0] = a.x(); da[0] = b.x(); vb[0] = c.x(); db[0] = d.x();
         va[1] = a.y(); da[1] = b.y(); vb[1] = c.y(); db[1] = d.y();
         return sel_code_x(S2) | (sel_code_y(S2) << 4);

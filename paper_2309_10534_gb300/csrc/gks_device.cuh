@@ -335,24 +335,25 @@ GKS_HD void ao_select(const T q[5], const TenoT<T>& P, TenoSel<T>& S)
 // both selections (the second normalises over k = 0..2 only, where d_k = 1/3
 // cancels).
 template <typename T>
+GKS_HD T teno_pow(T r, int q)
+{
+    if (q == 7) {
+        const T r2 = r * r, r3 = r2 * r;
+        return r3 * r3 * r;
+    }
+    return ipow(r, q);
+}
+template <typename T>
 GKS_HD unsigned teno_code(const T t[4], T ct1, T ct2, int q)
 {
     T m = t[0] < t[1] ? t[0] : t[1];
     m = m < t[2] ? m : t[2];
     m = m < t[3] ? m : t[3];
     T p[4];
+    p[3] = teno_pow(m * (T(1) / t[3]), q);
+    if (p[3] >= T(4.001) * ct1) return 1u;  // s012 + p[3] < 4: the first selection is settled
 #pragma unroll
-    for (int j = 0; j < 4; ++j) p[j] = m * (T(1) / t[j]);
-    if (q == 7) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const T r = p[j], r2 = r * r, r3 = r2 * r;
-            p[j] = r3 * r3 * r;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) p[j] = ipow(p[j], q);
-    }
+    for (int j = 0; j < 3; ++j) p[j] = teno_pow(m * (T(1) / t[j]), q);
     const T s012 = p[0] + p[1] + p[2];
     // first selection (Eqs. 4.6, 4.7): keep the large stencil when chi_{3,1} >= C_T1
     if (p[3] >= ct1 * (s012 + p[3])) return 1u;
@@ -411,27 +412,22 @@ GKS_HD unsigned teno_code_f32(const double q[5], const TenoT<double>& P)
                    + ((float)(13.0 / 3.0 * (163.0 / 130.0) * (163.0 / 130.0)) * bq * bq
                       + ((float)(781.0 / 720.0) * u3 * u3 + ((float)(1421461.0 / 327600.0) * R * R + eps4)));
     const float m = fminf(fminf(t0, t1), fminf(t2, t3));
-    float p[4] = {quick_div(m, t0), quick_div(m, t1), quick_div(m, t2), quick_div(m, t3)};
-    if (P.q == 7) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float r = p[j], r2 = r * r, r3 = r2 * r;
-            p[j] = r3 * r3 * r;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) p[j] = ipow(p[j], P.q);
-    }
+    // m: not lost in the scaling, finite; no square over- or underflows in
+    // float64 either
+    if (!(m > 1e-30f && m < 1e30f && h < 1423 && (h > 623 || P.eps4_m > 0.0f))) return 0u;
+    const float up = 1.0f + P.margin, dn = 1.0f - P.margin;
+    float p[4];
+    p[3] = teno_pow(quick_div(m, t3), P.q);
+    if (p[3] > 4.0f * up * P.fct1 && P.fct1 > 1e-25f) return 1u;  // s012 + p[3] < 4
+    p[0] = teno_pow(quick_div(m, t0), P.q);
+    p[1] = teno_pow(quick_div(m, t1), P.q);
+    p[2] = teno_pow(quick_div(m, t2), P.q);
     const float s012 = p[0] + p[1] + p[2];
     const float lim = P.fct1 * (s012 + p[3]), thr = P.fct2 * s012;
-    const float up = 1.0f + P.margin, dn = 1.0f - P.margin;
     const bool large = p[3] > lim * up, small = p[3] < lim * dn;
     const bool clear = (p[0] > thr * up || p[0] < thr * dn) && (p[1] > thr * up || p[1] < thr * dn) &&
                        (p[2] > thr * up || p[2] < thr * dn);
-    // m: not lost in the scaling, finite; the cut-offs well inside float32's
-    // range; no square over- or underflows in float64 either
-    if (!(m > 1e-30f && m < 1e30f && lim > 1e-25f && thr > 1e-25f && h < 1423 && (h > 623 || P.eps4_m > 0.0f)))
-        return 0u;
+    if (!(lim > 1e-25f && thr > 1e-25f)) return 0u;  // the cut-offs well inside float32's range
     if (large) return 1u;
     if (!(small && clear)) return 0u;
     return (p[0] > thr ? 2u : 0u) | (p[1] > thr ? 4u : 0u) | (p[2] > thr ? 8u : 0u);

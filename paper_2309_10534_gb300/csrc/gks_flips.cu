@@ -191,7 +191,7 @@ __global__ void k_flips2d(GridDev g, const double* __restrict__ W, int dirn, Ten
                     TenoSel2 S2;
                     teno_select_x2(qq, nf, S2);
                     f2 a, b, cc, d;
-                    teno_faces_x2(S2, a, b, cc, d);
+                    teno_faces_x2(S2, false, a, b, cc, d);
                     fv[r] = side ? cc : a;
                     fs[r] = (side ? d : b) * f2(ihf);
                 }

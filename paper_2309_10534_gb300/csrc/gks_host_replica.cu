@@ -44,15 +44,21 @@ int teno_packed(const double* q, double eps, int qpow, double ct1, double ct2, d
     for (int k = 0; k < 5; ++k) qq[k] = gks::f2((float)q[k], -(float)q[k]);
     const gks::TenoParams P{eps, qpow, ct1, ct2};
     gks::TenoSel2 S;
-    gks::teno_select_x2(qq, gks::teno_t<float>(P), S);
+    const bool both = gks::teno_select_x2(qq, gks::teno_t<float>(P), S);
     gks::f2 fv[4];
-    gks::teno_faces_x2(S, fv[0], fv[1], fv[2], fv[3]);
+    gks::teno_faces_x2(S, both, fv[0], fv[1], fv[2], fv[3]);
+    if (both) {  // the folded evaluation gives the same bits
+        gks::f2 fw[4];
+        gks::teno_faces_x2(S, false, fw[0], fw[1], fw[2], fw[3]);
+        for (int i = 0; i < 4; ++i)
+            if (fw[i].x() != fv[i].x()) return -2;
+    }
     for (int i = 0; i < 4; ++i) {
         if (fv[i].y() != -fv[i].x()) return -2;
         faces[i] = fv[i].x();
     }
     gks::f2 gv[4];
-    gks::teno_gauss_pm_x2(S, 0.28867513459481288f, gv[0], gv[1], gv[2], gv[3]);
+    gks::teno_gauss_pm_x2(S, both, 0.28867513459481288f, gv[0], gv[1], gv[2], gv[3]);
     for (int i = 0; i < 4; ++i) {
         if (gv[i].y() != -gv[i].x()) return -2;
         gauss[i] = gv[i].x();
