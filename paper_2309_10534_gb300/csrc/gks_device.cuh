@@ -343,7 +343,8 @@ GKS_HD T teno_pow(T r, int q)
     }
     return ipow(r, q);
 }
-template <typename T>
+// QUICK: leave at once where the large stencil is settled by its own power
+template <bool QUICK, typename T>
 GKS_HD unsigned teno_code(const T t[4], T ct1, T ct2, int q)
 {
     T m = t[0] < t[1] ? t[0] : t[1];
@@ -351,7 +352,7 @@ GKS_HD unsigned teno_code(const T t[4], T ct1, T ct2, int q)
     m = m < t[3] ? m : t[3];
     T p[4];
     p[3] = teno_pow(m * (T(1) / t[3]), q);
-    if (p[3] >= T(4.001) * ct1) return 1u;  // s012 + p[3] < 4: the first selection is settled
+    if (QUICK && p[3] >= T(4.001) * ct1) return 1u;  // s012 + p[3] < 4: the first selection is settled
 #pragma unroll
     for (int j = 0; j < 3; ++j) p[j] = teno_pow(m * (T(1) / t[j]), q);
     const T s012 = p[0] + p[1] + p[2];
@@ -389,6 +390,7 @@ GKS_HD float scaled_float(double x, int base)
     return as_float((ex == 0 || ex - base < 1) ? 0u : (v | ((unsigned)hi & 0x80000000u)));
 }
 
+template <bool QUICK>
 GKS_HD unsigned teno_code_f32(const double q[5], const TenoT<double>& P)
 {
     const double d1 = q[1] - q[0], d2 = q[2] - q[1], d3 = q[3] - q[2], d4 = q[4] - q[3];
@@ -418,7 +420,7 @@ GKS_HD unsigned teno_code_f32(const double q[5], const TenoT<double>& P)
     const float up = 1.0f + P.margin, dn = 1.0f - P.margin;
     float p[4];
     p[3] = teno_pow(quick_div(m, t3), P.q);
-    if (p[3] > 4.0f * up * P.fct1 && P.fct1 > 1e-25f) return 1u;  // s012 + p[3] < 4
+    if (QUICK && p[3] > 4.0f * up * P.fct1 && P.fct1 > 1e-25f) return 1u;  // s012 + p[3] < 4
     p[0] = teno_pow(quick_div(m, t0), P.q);
     p[1] = teno_pow(quick_div(m, t1), P.q);
     p[2] = teno_pow(quick_div(m, t2), P.q);
@@ -434,18 +436,18 @@ GKS_HD unsigned teno_code_f32(const double q[5], const TenoT<double>& P)
 }
 
 // TENO-D (Sec. 4.2) of one stencil: differences, selection, weights
-template <typename T>
+template <bool QUICK = true, typename T>
 GKS_HD void teno_select(const T q[5], const TenoT<T>& P, TenoSel<T>& S)
 {
     teno_differences(q, S);
     unsigned code = 0;
 #ifdef __CUDA_ARCH__
-    if constexpr (std::is_same<T, double>::value) code = teno_code_f32(q, P);
+    if constexpr (std::is_same<T, double>::value) code = teno_code_f32<QUICK>(q, P);
 #endif
     if (code == 0) {
         T t[4];
         teno_indicators(S, T(4) * P.eps, t);
-        code = teno_code(t, P.ct1, P.ct2, P.q);
+        code = teno_code<QUICK>(t, P.ct1, P.ct2, P.q);
     }
     S.large = (code & 1u) != 0;
     const int n = ((code >> 1) & 1u) + ((code >> 2) & 1u) + ((code >> 3) & 1u);
@@ -678,10 +680,10 @@ GKS_HD void quartic_gauss(const T q[5], T g, T& v, T& d)
 
 // the scheme's reconstruction: REC 0 = TENO-D, 1 = WENO5-AO, 2 = WENO5-Z and
 // 3 = TENO5 (the conventional path)
-template <int REC, typename T>
+template <int REC, bool QUICK = true, typename T>
 GKS_HD void rec_select(const T q[5], const TenoT<T>& P, TenoSel<T>& S)
 {
-    if constexpr (REC == 0) teno_select(q, P, S);
+    if constexpr (REC == 0) teno_select<QUICK>(q, P, S);
     else if constexpr (REC == 1) ao_select(q, P, S);
     else weno3_select<REC>(q, P, S);
 }

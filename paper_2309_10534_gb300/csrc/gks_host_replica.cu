@@ -223,8 +223,8 @@ extern "C" int gks_host_teno_code(const double* q, double eps, int qpow, double 
     gks::teno_differences(q, S);
     double t[4];
     gks::teno_indicators(S, 4.0 * P.eps, t);
-    *code64 = (int)gks::teno_code(t, P.ct1, P.ct2, P.q);
-    *code32 = (int)gks::teno_code_f32(q, P);
+    *code64 = (int)gks::teno_code<true>(t, P.ct1, P.ct2, P.q);
+    *code32 = (int)gks::teno_code_f32<true>(q, P);
     return 0;
 }
 

@@ -562,16 +562,16 @@ __global__ void __launch_bounds__(96) k1d_stage_wide(const __grid_constant__ Gri
                 f2 qq[5], x, y, z, w;
 #pragma unroll
                 for (int s = 0; s < 5; ++s) qq[s] = f2(q[s]);
-                packed_faces<0>(qq, tn, x, y, z, w);
+                packed_faces<0, false>(qq, tn, x, y, z, w);
                 vp = x.x(), dp = y.x(), vm = z.x(), dm = w.x();
             } else {
                 TenoSel<T> S;
-                teno_select(q, tn, S);
+                teno_select<false>(q, tn, S);
                 teno_faces(q, S, vp, dp, vm, dm);
             }
         } else {
             TenoSel<T> S;
-            rec_select<REC>(q, tn, S);
+            rec_select<REC, false>(q, tn, S);
             rec_faces<REC>(q, S, vp, dp, vm, dm);
         }
         sL[warp][0][lane] = vp;
@@ -769,7 +769,10 @@ __device__ __forceinline__ void copy_async(void* dst, const void* src)
     if constexpr (B == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
     else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
 }
-__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the last N committed groups of this thread are done
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // the cells of a tile that reaches past the boundary, ghosts by the boundary
 // rules (out of line: the other tiles keep their registers)
@@ -854,7 +857,7 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
         else base = a.src + (org + (n0 - NG) * sn + (t0 - 2) * st);
         auto cell = [&](int v, int cn, int ct) {
             const long long pv = v == 0 ? 0 : (v == 1 ? pv1 : (v == 2 ? pv2 : pv3));
-            sm.w[v][ct][cn] = (base + pv)[cn * sn + ct * st];
+            copy_async<sizeof(T)>(&sm.w[v][ct][cn], (base + pv) + (cn * sn + ct * st));
         };
         if (edge) load_edge_2d<T, TN, TT>(&sm.w[0][0][0], g, a, n0, t0, ds);
         else for (int k = tid; k < 4 * CN * CT; k += NT) {
@@ -863,6 +866,7 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
             else cell(v, e / CT, e % CT);
         }
     }
+    copy_commit();
     // y sweep: start copying the update's inputs (read in the update, they
     // cost its warps a memory round trip: four steps of a 64^2 float32 plane
     // 292 -> 281 us, two of a 1024^2 plane the same)
@@ -885,6 +889,8 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
             }
         }
     }
+    copy_commit();
+    copy_wait<1>();  // the tile
     __syncthreads();
     fp.dt = s_scal[0];
 
@@ -1112,7 +1118,7 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
 
     // phase 3: flux divergence; the y sweep updates the float64 state.  Each
     // thread reads the inputs it copied itself
-    copy_wait();
+    copy_wait<0>();
     T sig = T(0);
     const T cn = s_scal[1];
     static_assert((2 * NP) % NT == 0, "whole warps of tasks");

@@ -116,8 +116,11 @@ GKS_HD f2 pair_pow(f2 r, int q)
 // powers are (their sum with p_3 lies below 4, so p_3 >= 4 C_T1 settles Eq.
 // 4.7): in smooth regions three of the four powers and reciprocals, the
 // second selection and the sub-stencils' half of the evaluation (S.w is zero)
-// are then never formed, half of a pair's work: two steps of a
-// 1024^2 plane 1526 -> 1355 us, gradient of a 512^2 flow 10.9 -> 9.95 ms.
+// are then never formed, half of a pair's work.  Measured: one step of a
+// 1024^2 plane 0.763 -> 0.678 ms, 2048x1024 viscous 1.82 -> 1.66 ms, gradient
+// of a 512^2 flow 10.9 -> 9.95 ms.  The 1-D kernels, whose flux outweighs
+// their one selection per cell, lost 2 % to the branch and pass QUICK = false.
+template <bool QUICK = true>
 GKS_HD bool teno_select_x2(const f2 q[5], const TenoT<float>& P, TenoSel2& S)
 {
     TenoSel<f2> C;
@@ -139,7 +142,7 @@ GKS_HD bool teno_select_x2(const f2 q[5], const TenoT<float>& P, TenoSel2& S)
     f2 p[4];
     p[3] = pair_pow(m * f2(1.0f / t[3].x(), 1.0f / t[3].y()), P.q);
     const float sure = 4.001f * P.ct1;
-    if (p[3].x() >= sure && p[3].y() >= sure) {
+    if (QUICK && p[3].x() >= sure && p[3].y() >= sure) {
         S.l = f2(1.0f);
         S.w[0] = S.w[1] = S.w[2] = f2(0.0f);
         return true;
@@ -239,20 +242,20 @@ GKS_HD void recon_cell3(const T q[3][5], const TenoT<T>& P, T* vp, T* dp, T* vm,
         for (int s = 0; s < 5; ++s) qq[s] = f2(q[0][s], q[1][s]);
         TenoSel2 S2;
         f2 a, b, c, d;
-        if (teno_select_x2(qq, P, S2)) teno_faces_x2(S2, true, a, b, c, d);
-        else teno_faces_x2(S2, false, a, b, c, d);
+        teno_select_x2<false>(qq, P, S2);
+        teno_faces_x2(S2, false, a, b, c, d);
         vp[0] = a.x(); vp[1] = a.y();
         dp[0] = b.x(); dp[1] = b.y();
         vm[0] = c.x(); vm[1] = c.y();
         dm[0] = d.x(); dm[1] = d.y();
         TenoSel<T> S;
-        teno_select(q[2], P, S);
+        teno_select<false>(q[2], P, S);
         teno_faces(q[2], S, vp[2], dp[2], vm[2], dm[2]);
     } else {
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
             TenoSel<T> S;
-            rec_select<REC>(q[v], P, S);
+            rec_select<REC, false>(q[v], P, S);
             rec_faces<REC>(q[v], S, vp[v], dp[v], vm[v], dm[v]);
         }
     }
@@ -313,12 +316,12 @@ GKS_HD TenoT<f2> pair_teno(const TenoT<float>& P)
 // Gauss points (tangential).  REC 0: TENO-D with the folded selection above;
 // REC 1: WENO5-AO through its templated arithmetic, whose weights have no
 // branches.
-template <int REC>
+template <int REC, bool QUICK = true>
 GKS_HD void packed_faces(const f2 q[5], const TenoT<float>& P, f2& vp, f2& dp, f2& vm, f2& dm)
 {
     if constexpr (REC == 0) {
         TenoSel2 S;
-        if (teno_select_x2(q, P, S)) teno_faces_x2(S, true, vp, dp, vm, dm);
+        if (teno_select_x2<QUICK>(q, P, S)) teno_faces_x2(S, true, vp, dp, vm, dm);
         else teno_faces_x2(S, false, vp, dp, vm, dm);
     } else {
         TenoSel<f2> S;
