@@ -62,8 +62,7 @@ struct BatchDev {
 template <typename T, int NT>
 __device__ __forceinline__ T block_max(T v, T* red)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    v = warp_max(v);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -75,13 +74,13 @@ __device__ __forceinline__ T block_max(T v, T* red)
 
 __device__ __forceinline__ unsigned int block_or(unsigned int v, unsigned int* red)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
+    if (!__syncthreads_or(v != 0u)) return 0u;
+    v = __reduce_or_sync(0xffffffffu, v);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     unsigned int r = 0;
     for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r |= red[k];
+    __syncthreads();
     return r;
 }
 
@@ -122,13 +121,16 @@ __device__ void stage_chunk(ChunkSmem<T, NT>& sm, double* W, float* Wf, T* Ws, T
     float* Wfv[3] = {Wf, Wf + vstride, Wf + 2 * vstride};
     T* Wsv[3] = {Ws, Ws + vstride, Ws + 2 * vstride};
     T* Av[3] = {A, A + vstride, A + 2 * vstride};
-    for (int k = tid; k < 3 * (TN + 6); k += NT) {
-        const int v = k / (TN + 6), c = k % (TN + 6);
-        int i = c0 - 3 + c;
+    static_assert(TN + 6 == NT, "one cell per thread and variable");
+    {
+        int i = c0 - 3 + tid;
         i = i < 0 ? 0 : (i >= n ? n - 1 : i);
-        if (stage == 2) sm.q[v][c] = (v == 0 ? Ws : (v == 1 ? Wsv[1] : Wsv[2]))[i];
-        else if constexpr (sizeof(T) == 4) sm.q[v][c] = (v == 0 ? Wf : (v == 1 ? Wfv[1] : Wfv[2]))[i];
-        else sm.q[v][c] = (v == 0 ? W : (v == 1 ? Wv[1] : Wv[2]))[i];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            if (stage == 2) sm.q[v][tid] = Wsv[v][i];
+            else if constexpr (sizeof(T) == 4) sm.q[v][tid] = Wfv[v][i];
+            else sm.q[v][tid] = Wv[v][i];
+        }
     }
     __syncthreads();
     const T ih = sc.ih;
@@ -141,8 +143,11 @@ __device__ void stage_chunk(ChunkSmem<T, NT>& sm, double* W, float* Wf, T* Ws, T
         recon_cell3<0>(q, tn, vp, dp, vm, dm);  // the single-grid 1-D kernel's arithmetic
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
-            if (c <= TN) { sm.L[v][0][c] = vp[v]; sm.L[v][1][c] = dp[v] * ih; }
-            if (c >= 1) { sm.R[v][0][c - 1] = vm[v]; sm.R[v][1][c - 1] = dm[v] * ih; }
+            // R holds face c - 1's at c: every cell stores both its faces' values
+            sm.L[v][0][c] = vp[v];
+            sm.L[v][1][c] = dp[v] * ih;
+            sm.R[v][0][c] = vm[v];
+            sm.R[v][1][c] = dm[v] * ih;
         }
     }
     __syncthreads();
@@ -156,8 +161,8 @@ __device__ void stage_chunk(ChunkSmem<T, NT>& sm, double* W, float* Wf, T* Ws, T
         for (int v = 0; v < 3; ++v) {
             L.W[slot[v]] = sm.L[v][0][f];
             L.Wn[slot[v]] = sm.L[v][1][f];
-            R.W[slot[v]] = sm.R[v][0][f];
-            R.Wn[slot[v]] = sm.R[v][1][f];
+            R.W[slot[v]] = sm.R[v][0][f + 1];
+            R.Wn[slot[v]] = sm.R[v][1][f + 1];
         }
         auto state = [&](int side, Side<T>& S, Prim<T>& p) {
             if (prim_state<T, 1>(S.W, fp.gm1, p)) return;

@@ -194,6 +194,21 @@ __device__ __forceinline__ T cell_sigma(const WT* w, int dim, T gamma, T mu, T h
     return s;
 }
 
+// maximum of a warp's non-negative values, NaN only where every lane holds
+// NaN (as fmax has it); float32 by one integer reduction on the bits, which
+// order like the values
+__device__ __forceinline__ float warp_max(float s)
+{
+    const unsigned k = __reduce_max_sync(0xffffffffu, s != s ? 0u : __float_as_uint(s) + 1u);
+    return k == 0u ? __uint_as_float(0x7fffffffu) : __uint_as_float(k - 1u);
+}
+__device__ __forceinline__ double warp_max(double s)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
+    return s;
+}
+
 // Block reduction of the CFL rate (only when with_sigma), the error word and
 // the fallback count; one atomic of each per block.  commit: the last block
 // to get here commits the step (every block has read dt and done by then).
@@ -203,20 +218,27 @@ __device__ __forceinline__ void block_commit(T s, bool with_sigma, unsigned int 
 {
     __shared__ T red_s[NT / 32];
     __shared__ unsigned int red_e[NT / 32], red_f[NT / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (with_sigma) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
-        err |= __shfl_xor_sync(0xffffffffu, err, o);
-        nfb += __shfl_xor_sync(0xffffffffu, nfb, o);
-    }
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) { red_s[w] = s; red_e[w] = err; red_f[w] = nfb; }
-    __syncthreads();
+    if (with_sigma) {
+        const T m = warp_max(s);
+        if (l == 0) red_s[w] = m;
+    }
+    // errors and fallbacks are rare: one vote says whether there are any
+    const bool any = __syncthreads_or((err | nfb) != 0u);
+    if (any) {
+        err = __reduce_or_sync(0xffffffffu, err);
+        nfb = __reduce_add_sync(0xffffffffu, nfb);
+        if (l == 0) { red_e[w] = err; red_f[w] = nfb; }
+        __syncthreads();
+    }
     if (threadIdx.x == 0) {
+        if (with_sigma) s = red_s[0];
         for (int k = 1; k < NT / 32; ++k) {
             if (with_sigma) s = fmax(s, red_s[k]);
-            err |= red_e[k];
-            nfb += red_f[k];
+            if (any) {
+                err |= red_e[k];
+                nfb += red_f[k];
+            }
         }
         const double sd = (double)s;
         if (with_sigma && (sd > 0.0 || sd != sd))
@@ -305,7 +327,7 @@ __device__ __noinline__ void load_edge_1d(T* sq, const E* src, const GridDev& g,
 }
 
 template <typename T, bool NONEQ, bool PRFIX, int TN, int REC = 0>
-__global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ GridDev g, Stage1DArgs a,
+__global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(const __grid_constant__ GridDev g, Stage1DArgs a,
                                                     FluxParams<T> fp, TenoT<T> tn, DevState* ds)
 {
     if (ds->done) return;
@@ -325,7 +347,10 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
         s_scal[5] = (T)g.dx;
     }
     __shared__ T sq[3][TN + 6];
-    __shared__ T sL[3][2][TN + 1], sR[3][2][TN + 1];  // [var][value, slope][face]
+    // [var][value, slope][face], and one entry beyond each end that no face
+    // reads, so that every cell stores both its faces' values
+    __shared__ T sL[3][2][TN + 2], sR_[3][2][TN + 2];
+    T(*sR)[2][TN + 2] = reinterpret_cast<T(*)[2][TN + 2]>(&sR_[0][0][1]);
     __shared__ T sG[2][3][TN + 1];                     // face fluxes for the update
     const int i0 = blockIdx.x * TN;
     const int tid = threadIdx.x;
@@ -360,10 +385,10 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
             load_edge_1d<T, TN>(&sq[0][0], src, g, i0, ds, a.stage);
             return;
         }
-        for (int k = tid; k < 3 * (TN + 6); k += NT) {
-            const int v = k / (TN + 6), c = k % (TN + 6);
-            sq[v][c] = load_as<T>(src[v * pl + i0 + c]);
-        }
+        static_assert(TN + 6 - NT == 4, "four cells beyond one per thread");
+#pragma unroll
+        for (int v = 0; v < 3; ++v) sq[v][tid] = load_as<T>(src[v * pl + i0 + tid]);
+        if (tid < 12) sq[tid >> 2][NT + (tid & 3)] = load_as<T>(src[(tid >> 2) * pl + i0 + NT + (tid & 3)]);
     };
     if constexpr (sizeof(T) == 4) {
         if (a.srcf) load(a.srcf);
@@ -407,8 +432,10 @@ __global__ void __launch_bounds__(TN + 2) k1d_stage(const __grid_constant__ Grid
             recon_cell3<REC>(q, tn, vp, dp, vm, dm);
 #pragma unroll
             for (int v = 0; v < 3; ++v) {
-                if (c <= TN) { sL[v][0][c] = vp[v]; sL[v][1][c] = dp[v] * idx_; }
-                if (c >= 1) { sR[v][0][c - 1] = vm[v]; sR[v][1][c - 1] = dm[v] * idx_; }
+                sL[v][0][c] = vp[v];
+                sL[v][1][c] = dp[v] * idx_;
+                sR_[v][0][c] = vm[v];
+                sR_[v][1][c] = dm[v] * idx_;
             }
         }
     }
