@@ -78,9 +78,10 @@ __device__ __forceinline__ int gvar_(int v, bool swap) { return (swap && (v == 1
 
 // scratch indices: faces f in [0, nn], line rows r in [-2, nt+2), Gauss rows
 // in [0, nt), cells i in [-1, nn]
+template <int D>
 __device__ __forceinline__ long long lidx(const AdjDir& a, int f, int r)
 {
-    return a.dirn == 0 ? (long long)(r + 2) * (a.nn + 1) + f : (long long)f * (a.nt + 4) + (r + 2);
+    return D == 0 ? (long long)(r + 2) * (a.nn + 1) + f : (long long)f * (a.nt + 4) + (r + 2);
 }
 // A k_adj_gauss block holds 128 face segments (float64: 64, as a block's time
 // is its share of the float64 pipe): 16 along the unit stride.  Rows of its
@@ -89,17 +90,20 @@ template <typename T> constexpr int ADJ_PAIRS = sizeof(T) == 4 ? 128 : 64;
 __host__ __device__ constexpr int adj_tile(int dirn, bool f32) { return dirn == 0 ? (f32 ? 8 : 4) : 16; }
 // line cotangents: own rows of a tile, and its edge rows e = 0, 1 (the two
 // rows before it) and 2, 3 (after it)
+template <int D>
 __device__ __forceinline__ long long midx(const AdjDir& a, int f, int r)
 {
-    return a.dirn == 0 ? (long long)r * (a.nn + 1) + f : (long long)f * a.ntp + r;
+    return D == 0 ? (long long)r * (a.nn + 1) + f : (long long)f * a.ntp + r;
 }
+template <int D>
 __device__ __forceinline__ long long eidx(const AdjDir& a, int f, int tile, int e)
 {
-    return a.dirn == 0 ? (long long)(tile * 4 + e) * (a.nn + 1) + f : (long long)f * (a.tiles * 4) + tile * 4 + e;
+    return D == 0 ? (long long)(tile * 4 + e) * (a.nn + 1) + f : (long long)f * (a.tiles * 4) + tile * 4 + e;
 }
+template <int D>
 __device__ __forceinline__ long long didx(const AdjDir& a, int i, int r)
 {
-    return a.dirn == 0 ? (long long)(r + 2) * (a.nn + 2) + (i + 1) : (long long)(i + 1) * (a.nt + 4) + (r + 2);
+    return D == 0 ? (long long)(r + 2) * (a.nn + 2) + (i + 1) : (long long)(i + 1) * (a.nt + 4) + (r + 2);
 }
 
 // a direction scalar in the arithmetic type
@@ -119,10 +123,11 @@ __device__ __forceinline__ T load_src(const AdjDir& a, long long gi)
 
 // map the launch to (normal index, tangential index): the unit-stride grid
 // direction runs along threadIdx.x
-__device__ __forceinline__ void map2(const AdjDir& a, int& n, int& t, int n0, int t0)
+template <int D>
+__device__ __forceinline__ void map2(int& n, int& t, int n0, int t0)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (a.dirn == 0) { n = n0 + x; t = t0 + y; }
+    if (D == 0) { n = n0 + x; t = t0 + y; }
     else { n = n0 + y; t = t0 + x; }
 }
 
@@ -161,11 +166,12 @@ __device__ __forceinline__ unsigned fwd_faces2(const T qa[5], const T qb[5], con
         for (int s = 0; s < 5; ++s) qq[s] = f2(qa[s], qb[s]);
         TenoSel2 S2;
         f2 a, b, c, d;
-        if (teno_select_x2(qq, P, S2)) teno_faces_x2(S2, true, a, b, c, d);
+        const bool both = teno_select_x2(qq, P, S2);
+        if (both) teno_faces_x2(S2, true, a, b, c, d);
         else teno_faces_x2(S2, false, a, b, c, d);
         vp[0] = a.x(); dp[0] = b.x(); vm[0] = c.x(); dm[0] = d.x();
         vp[1] = a.y(); dp[1] = b.y(); vm[1] = c.y(); dm[1] = d.y();
-        return sel_code_x(S2) | (sel_code_y(S2) << 4);
+        return both ? 0x11u : sel_code_x(S2) | (sel_code_y(S2) << 4);
     } else {
         unsigned code = 0;
         const T* q[2] = {qa, qb};
@@ -189,11 +195,12 @@ __device__ __forceinline__ unsigned fwd_gauss2(const T qa[5], const T qb[5], con
         for (int s = 0; s < 5; ++s) qq[s] = f2(qa[s], qb[s]);
         TenoSel2 S2;
         f2 a, b, c, d;
-        if (teno_select_x2(qq, P, S2)) teno_gauss_pm_x2(S2, true, gB, a, b, c, d);  // gA = -gB
+        const bool both = teno_select_x2(qq, P, S2);
+        if (both) teno_gauss_pm_x2(S2, true, gB, a, b, c, d);  // gA = -gB
         else teno_gauss_pm_x2(S2, false, gB, a, b, c, d);
         va[0] = a.x(); da[0] = b.x(); vb[0] = c.x(); db[0] = d.x();
         va[1] = a.y(); da[1] = b.y(); vb[1] = c.y(); db[1] = d.y();
-        return sel_code_x(S2) | (sel_code_y(S2) << 4);
+        return both ? 0x11u : sel_code_x(S2) | (sel_code_y(S2) << 4);
     } else {
         unsigned code = 0;
         const T* q[2] = {qa, qb};
@@ -209,13 +216,13 @@ __device__ __forceinline__ unsigned fwd_gauss2(const T qa[5], const T qb[5], con
 }
 
 // ---- phase 1: normal TENO-D of the stage input (as the forward sweep)
-template <typename T>
+template <typename T, int D>
 __global__ void __launch_bounds__(256) k_adj_lines(GridDev g, AdjDir a, TenoT<T> tn)
 {
     int i, r;
-    map2(a, i, r, -1, -2);
+    map2<D>(i, r, -1, -2);
     if (i > a.nn || r >= a.nt + 2) return;
-    const bool swap = a.dirn != 0;
+    const bool swap = D != 0;
     const long long org = (long long)NG * g.pitch + NG;
     const long long LP = (long long)(a.nn + 1) * (a.nt + 4);
     T* L = static_cast<T*>(a.lines);
@@ -235,12 +242,12 @@ __global__ void __launch_bounds__(256) k_adj_lines(GridDev g, AdjDir a, TenoT<T>
         for (int l = 0; l < 2; ++l) {
             const int v = vv + l;
             if (i + 1 <= a.nn) {
-                L[(0 * 4 + v) * LP + lidx(a, i + 1, r)] = vp[l];
-                L[(1 * 4 + v) * LP + lidx(a, i + 1, r)] = dp[l] * ih;
+                L[(0 * 4 + v) * LP + lidx<D>(a, i + 1, r)] = vp[l];
+                L[(1 * 4 + v) * LP + lidx<D>(a, i + 1, r)] = dp[l] * ih;
             }
             if (i >= 0) {
-                L[(2 * 4 + v) * LP + lidx(a, i, r)] = vm[l];
-                L[(3 * 4 + v) * LP + lidx(a, i, r)] = dm[l] * ih;
+                L[(2 * 4 + v) * LP + lidx<D>(a, i, r)] = vm[l];
+                L[(3 * 4 + v) * LP + lidx<D>(a, i, r)] = dm[l] * ih;
             }
         }
     }
@@ -255,8 +262,15 @@ __global__ void __launch_bounds__(256) k_adj_lines(GridDev g, AdjDir a, TenoT<T>
 // by k_adj_normal) was most of both kernels' memory traffic; the block's 128
 // segments now add theirs up in shared memory, and 1.25 to 1.5 values per
 // segment and quantity go out.
-template <typename T>
-__global__ void __launch_bounds__(2 * ADJ_PAIRS<T>, (sizeof(T) == 4) ? 2 : 1)
+//
+// Bound by its chain of dependent arithmetic at few warps per SM, so float32
+// runs three blocks of 256 threads at 80 registers (some values spill) rather
+// than two at 128, and a segment that keeps its large stencils throughout (one
+// compare of its codes) skips the sub-stencils: with the direction a template
+// parameter, 12 steps and their reverse on a 512^2 float32 plane 9.86 -> 9.07
+// ms, 4 on a 96^2 float64 plane 5.45 -> 5.35 ms.
+template <typename T, int D>
+__global__ void __launch_bounds__(2 * ADJ_PAIRS<T>, (sizeof(T) == 4) ? 3 : 2)
 k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
 {
     constexpr int NP = ADJ_PAIRS<T>;
@@ -264,11 +278,11 @@ k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
     const int gp = threadIdx.x & 1;
     const int x = (blockIdx.x * blockDim.x + threadIdx.x) >> 1, y = blockIdx.y * blockDim.y + threadIdx.y;
     int f, r;
-    if (a.dirn == 0) { f = x; r = y; }
+    if (D == 0) { f = x; r = y; }
     else { f = y; r = x; }
     const bool valid = f <= a.nn && r < a.nt;
     const int fc = valid ? f : 0, rc = valid ? r : 0;  // in-range indices for the idle lanes' loads
-    const bool swap = a.dirn != 0;
+    const bool swap = D != 0;
     const long long org = (long long)NG * g.pitch + NG;
     const long long LP = (long long)(a.nn + 1) * (a.nt + 4);
     const T* Lq = static_cast<const T*>(a.lines);
@@ -281,8 +295,8 @@ k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
     unsigned codes = 0;  // selections of the own side: 4 bits per quantity kk * 4 + v
     const T gs = gp ? T(0.28867513459481288) : T(-0.28867513459481288);
     {
-        const int ls = a.dirn == 0 ? a.nn + 1 : 1;  // element stride of line rows
-        const T* Lp = Lq + (long long)(8 * gp) * LP + lidx(a, fc, rc - 2);
+        const int ls = D == 0 ? a.nn + 1 : 1;  // element stride of line rows
+        const T* Lp = Lq + (long long)(8 * gp) * LP + lidx<D>(a, fc, rc - 2);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             // the side's value and normal-slope streams as one pair, as the forward
@@ -383,17 +397,19 @@ k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
         oWt[v] = __shfl_xor_sync(0xffffffffu, gR.Wt[v], 1);
     }
     const int pair = threadIdx.y * 16 + (threadIdx.x >> 1), tid = threadIdx.y * 32 + threadIdx.x;
-    const int TT = adj_tile(a.dirn, sizeof(T) == 4), NF = NP / TT;  // the tile's rows and faces
-    const int tile = a.dirn == 0 ? blockIdx.y : blockIdx.x, f0 = (a.dirn == 0 ? blockIdx.x : blockIdx.y) * NF;
+    const int TT = adj_tile(D, sizeof(T) == 4), NF = NP / TT;  // the tile's rows and faces
+    const int tile = D == 0 ? blockIdx.y : blockIdx.x, f0 = (D == 0 ? blockIdx.x : blockIdx.y) * NF;
     const long long MP = (long long)(a.nn + 1) * a.ntp, EP = (long long)(a.nn + 1) * a.tiles * 4;
     T* M = static_cast<T*>(a.contrib);
     T* Eg = M + NQ * MP;
+    const bool all_large = codes == 0x11111111u;
 #pragma unroll 1
     for (int kk = 0; kk < 2; ++kk) {  // values, then normal slopes, of both sides
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             TenoSel<T> S;
-            sel_decode((codes >> (4 * (kk * 4 + v))) & 15u, S);
+            S.large = true;
+            if (!all_large) sel_decode((codes >> (4 * (kk * 4 + v))) & 15u, S);
             T gq[5];
             if (kk == 0) teno_gauss_pm_T(S, gs, oW[v], oWt[v] * iht, gL.W[v], gL.Wt[v] * iht, gq);
             else teno_gauss_pm_T(S, gs, oWn[v], T(0), gL.Wn[v], T(0), gq);
@@ -405,7 +421,7 @@ k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
         // segments of a row (dirn 0) or of a face (dirn 1) are adjacent
         for (int k = tid; k < 8 * (TT + 4) * NF; k += 2 * NP) {
             int l, fl, qq;
-            if (a.dirn == 0) { fl = k % 16; l = (k / 16) % (NP / 16 + 4); qq = k / (NP + 64); }
+            if (D == 0) { fl = k % 16; l = (k / 16) % (NP / 16 + 4); qq = k / (NP + 64); }
             else { l = k % 20; fl = (k / 20) % (NP / 16); qq = k / (20 * (NP / 16)); }
             const int f2_ = f0 + fl;
             if (f2_ > a.nn) continue;
@@ -413,33 +429,33 @@ k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
 #pragma unroll
             for (int s = 0; s < 5; ++s) {
                 const int rl = l - s;
-                if (rl >= 0 && rl < TT) acc += sc[qq][s][a.dirn == 0 ? rl * 16 + fl : fl * 16 + rl];
+                if (rl >= 0 && rl < TT) acc += sc[qq][s][D == 0 ? rl * 16 + fl : fl * 16 + rl];
             }
             const int qi = (2 * (qq >> 2) + kk) * 4 + (qq & 3);
-            if (l >= 2 && l < TT + 2) M[qi * MP + midx(a, f2_, tile * TT + l - 2)] = acc;
-            else Eg[qi * EP + eidx(a, f2_, tile, l < 2 ? l : l - TT)] = acc;
+            if (l >= 2 && l < TT + 2) M[qi * MP + midx<D>(a, f2_, tile * TT + l - 2)] = acc;
+            else Eg[qi * EP + eidx<D>(a, f2_, tile, l < 2 ? l : l - TT)] = acc;
         }
         __syncthreads();
     }
 }
 
 // ---- per cell: line cotangents of its faces -> transposed normal TENO-D
-template <typename T>
+template <typename T, int D>
 __global__ void __launch_bounds__(256) k_adj_normal(GridDev g, AdjDir a, TenoT<T> tn)
 {
     int i, r;
-    map2(a, i, r, -1, -2);
+    map2<D>(i, r, -1, -2);
     if (i > a.nn || r >= a.nt + 2) return;
-    const bool swap = a.dirn != 0;
+    const bool swap = D != 0;
     const long long org = (long long)NG * g.pitch + NG;
     const long long MP = (long long)(a.nn + 1) * a.ntp, EP = (long long)(a.nn + 1) * a.tiles * 4;
     const long long DP = (long long)(a.nn + 2) * (a.nt + 4);
     const T* M = static_cast<const T*>(a.contrib);
     const T* Eg = M + NQ * MP;
-    T* D = static_cast<T*>(a.dcell);
+    T* dc = static_cast<T*>(a.dcell);
     const T ih = scal<T>(a.ihn, a.fihn);
     // line row r: its tile's sum, and the edge rows of the tiles beside it
-    const int TT = adj_tile(a.dirn, sizeof(T) == 4);
+    const int TT = adj_tile(D, sizeof(T) == 4);
     int own = -1, e1 = -1, e2 = -1, t1 = 0, t2 = 0;  // own row; edge rows of tiles t1, t2
     if (r < 0) { t1 = 0; e1 = r + 2; }
     else if (r >= a.ntp) { t1 = a.tiles - 1; e1 = 2 + r - a.ntp; }
@@ -451,9 +467,9 @@ __global__ void __launch_bounds__(256) k_adj_normal(GridDev g, AdjDir a, TenoT<T
     }
     auto gline = [&](int q, int f) {
         T acc = T(0);
-        if (e1 >= 0) acc += Eg[q * EP + eidx(a, f, t1, e1)];
-        if (own >= 0) acc += M[q * MP + midx(a, f, own)];
-        if (e2 >= 0) acc += Eg[q * EP + eidx(a, f, t2, e2)];
+        if (e1 >= 0) acc += Eg[q * EP + eidx<D>(a, f, t1, e1)];
+        if (own >= 0) acc += M[q * MP + midx<D>(a, f, own)];
+        if (e2 >= 0) acc += Eg[q * EP + eidx<D>(a, f, t2, e2)];
         return acc;
     };
     {
@@ -484,29 +500,29 @@ __global__ void __launch_bounds__(256) k_adj_normal(GridDev g, AdjDir a, TenoT<T
             T gq[5] = {T(0), T(0), T(0), T(0), T(0)};
             teno_faces_T(S, gvp, gdp, gvm, gdm, gq);
 #pragma unroll
-            for (int s = 0; s < 5; ++s) D[(long long)(s * 4 + v) * DP + didx(a, i, r)] = gq[s];
+            for (int s = 0; s < 5; ++s) dc[(long long)(s * 4 + v) * DP + didx<D>(a, i, r)] = gq[s];
         }
     }
 }
 
 // ---- per cell: sum of the contributions of the cells whose stencil holds it
-template <typename T>
+template <typename T, int D>
 __global__ void __launch_bounds__(256) k_adj_gather(GridDev g, AdjDir a)
 {
     int j, r;
-    map2(a, j, r, -3, -2);
+    map2<D>(j, r, -3, -2);
     if (j > a.nn + 2 || r >= a.nt + 2) return;
-    const bool swap = a.dirn != 0;
+    const bool swap = D != 0;
     const long long org = (long long)NG * g.pitch + NG;
     const long long DP = (long long)(a.nn + 2) * (a.nt + 4);
-    const T* D = static_cast<const T*>(a.dcell);
+    const T* dc = static_cast<const T*>(a.dcell);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
         T acc = T(0);
 #pragma unroll
         for (int s = 0; s < 5; ++s) {
             const int i = j + 2 - s;  // cell i's stencil position s is cell i - 2 + s = j
-            if (i >= -1 && i <= a.nn) acc += D[(long long)(s * 4 + v) * DP + didx(a, i, r)];
+            if (i >= -1 && i <= a.nn) acc += dc[(long long)(s * 4 + v) * DP + didx<D>(a, i, r)];
         }
         a.gW[(long long)gvar_(v, swap) * g.plane + org + j * a.sn + r * a.st] += to_f64(acc);
     }
@@ -649,7 +665,7 @@ gks_status load_state(gks_adjoint* A, const double* Wg)
     return GKS_OK;
 }
 
-template <typename T>
+template <typename T, int D>
 gks_status sweep_vjp_t(gks_adjoint* A, AdjDir d)
 {
     gks_ctx* c = A->c;
@@ -660,17 +676,17 @@ gks_status sweep_vjp_t(gks_adjoint* A, AdjDir d)
     cudaStream_t st = c->stream;
     // launch shapes: x along the unit-stride direction
     auto grid_for = [&](int nnorm, int ntan, dim3 blk, int xmul) {
-        const int ex = d.dirn == 0 ? nnorm : ntan, ey = d.dirn == 0 ? ntan : nnorm;
+        const int ex = D == 0 ? nnorm : ntan, ey = D == 0 ? ntan : nnorm;
         return dim3((unsigned)((ex * xmul + blk.x - 1) / blk.x), (unsigned)((ey + blk.y - 1) / blk.y));
     };
     const dim3 b256(32, 8), bg(32, ADJ_PAIRS<T> / 16);
     // the per-cell kernels take the two variable pairs in blockIdx.z
     dim3 gcell = grid_for(d.nn + 2, d.nt + 4, b256, 1);
     gcell.z = 2;
-    k_adj_lines<T><<<gcell, b256, 0, st>>>(g, d, tn);
-    k_adj_gauss<T><<<grid_for(d.nn + 1, d.nt, bg, 2), bg, 0, st>>>(g, d, fp, tt);
-    k_adj_normal<T><<<gcell, b256, 0, st>>>(g, d, tn);
-    k_adj_gather<T><<<grid_for(d.nn + 6, d.nt + 4, b256, 1), b256, 0, st>>>(g, d);
+    k_adj_lines<T, D><<<gcell, b256, 0, st>>>(g, d, tn);
+    k_adj_gauss<T, D><<<grid_for(d.nn + 1, d.nt, bg, 2), bg, 0, st>>>(g, d, fp, tt);
+    k_adj_normal<T, D><<<gcell, b256, 0, st>>>(g, d, tn);
+    k_adj_gather<T, D><<<grid_for(d.nn + 6, d.nt + 4, b256, 1), b256, 0, st>>>(g, d);
     CK(cudaGetLastError());
     A->launches += 4;
     return GKS_OK;
@@ -715,7 +731,8 @@ gks_status stage_vjp(gks_adjoint* A, const void* input, const double* lam1, cons
         d.fcD2 = (float)d.cD2;
         d.fihn = (float)d.ihn;
         d.fiht = (float)d.iht;
-        gks_status s = f32 ? sweep_vjp_t<float>(A, d) : sweep_vjp_t<double>(A, d);
+        gks_status s = f32 ? (dirn == 0 ? sweep_vjp_t<float, 0>(A, d) : sweep_vjp_t<float, 1>(A, d))
+                           : (dirn == 0 ? sweep_vjp_t<double, 0>(A, d) : sweep_vjp_t<double, 1>(A, d));
         if (s) return s;
     }
     const GridDev& g = c->g;
