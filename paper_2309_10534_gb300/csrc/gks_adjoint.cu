@@ -262,13 +262,6 @@ __global__ void __launch_bounds__(256) k_adj_lines(GridDev g, AdjDir a, TenoT<T>
 // by k_adj_normal) was most of both kernels' memory traffic; the block's 128
 // segments now add theirs up in shared memory, and 1.25 to 1.5 values per
 // segment and quantity go out.
-//
-// Bound by its chain of dependent arithmetic at few warps per SM, so float32
-// runs three blocks of 256 threads at 80 registers (some values spill) rather
-// than two at 128, and a segment that keeps its large stencils throughout (one
-// compare of its codes) skips the sub-stencils: with the direction a template
-// parameter, 12 steps and their reverse on a 512^2 float32 plane 9.86 -> 9.07
-// ms, 4 on a 96^2 float64 plane 5.45 -> 5.35 ms.
 template <typename T, int D>
 __global__ void __launch_bounds__(2 * ADJ_PAIRS<T>, (sizeof(T) == 4) ? 3 : 2)
 k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)

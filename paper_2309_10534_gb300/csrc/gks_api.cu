@@ -28,23 +28,32 @@ using namespace gks;
 namespace {
 constexpr int GRAPH_STEPS = 8;
 
-// interior [nv][ny][nx] <-> ghosted layout (1-D: ny = 1, no ghost rows)
-__device__ __forceinline__ long long ghosted_index(const GridDev& g, long long k)
+// interior [nv][ny][nx] <-> ghosted layout (1-D: ny = 1, no ghost rows).
+// Blocks of 32 x 8 threads walk over (x, row) with row = v ny + j: two
+// divisions per row, none per element.  shadow (may be null): the float32
+// path's copy, written in the same pass.  Set and get of 2^22 float32 cells:
+// 35 + 13 (the copy in a pass of its own) + 35 us -> one pass each
+// (four steps of that tube and its copies 1557 -> 1525 us, two of a 1024^2
+// plane 1332 -> 1316 us).
+template <bool IN>
+__global__ void __launch_bounds__(256) k_copy_interior(const __grid_constant__ GridDev g, const double* __restrict__ src,
+                                                       double* __restrict__ dst, float* __restrict__ shadow)
 {
-    const int ny = (g.dim == 2) ? g.ny : 1;
-    const long long per_v = (long long)g.nx * ny;
-    const int v = (int)(k / per_v);
-    const long long r = k - v * per_v;
-    const int j = (int)(r / g.nx), i = (int)(r - (long long)j * g.nx);
-    return (long long)v * g.plane + (long long)((g.dim == 2 ? NG : 0) + j) * g.pitch + NG + i;
-}
-__global__ void k_unpack(GridDev g, const double* __restrict__ src, double* __restrict__ arr, long long n)
-{
-    for (long long k = blockIdx.x * 256ll + threadIdx.x; k < n; k += 256ll * gridDim.x) arr[ghosted_index(g, k)] = src[k];
-}
-__global__ void k_pack(GridDev g, const double* __restrict__ arr, double* __restrict__ dst, long long n)
-{
-    for (long long k = blockIdx.x * 256ll + threadIdx.x; k < n; k += 256ll * gridDim.x) dst[k] = arr[ghosted_index(g, k)];
+    const int ny = (g.dim == 2) ? g.ny : 1, g0 = (g.dim == 2) ? NG : 0;
+    const long long rows = (long long)(g.dim + 2) * ny;
+    for (long long row = blockIdx.y * 8ll + threadIdx.y; row < rows; row += 8ll * gridDim.y) {
+        const int v = (int)(row / ny), j = (int)(row - (long long)v * ny);
+        const long long packed = row * g.nx, ghosted = (long long)v * g.plane + (long long)(g0 + j) * g.pitch + NG;
+        for (int i = blockIdx.x * 32 + threadIdx.x; i < g.nx; i += 32 * gridDim.x) {
+            if constexpr (IN) {
+                const double x = src[packed + i];
+                dst[ghosted + i] = x;
+                if (shadow) shadow[ghosted + i] = narrow(x);
+            } else {
+                dst[packed + i] = src[ghosted + i];
+            }
+        }
+    }
 }
 }  // namespace
 
@@ -346,7 +355,7 @@ gks_status check_err(gks_ctx* c)
 namespace gks {
 namespace rt {
 
-gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device, bool in, bool wait)
+gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device, bool in, bool wait, float* shadow)
 {
     // A caller's array [nv][ny][nx] is moved in one contiguous copy (host
     // arrays through a device staging buffer) and scattered into / gathered
@@ -365,9 +374,11 @@ gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device
         src = dst = c->stage;
         if (in) CK(cudaMemcpyAsync(c->stage, W, sizeof(double) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
     }
-    const int blocks = (int)std::min<long long>((n + 255) / 256, 8192);
-    if (in) k_unpack<<<blocks, 256, 0, c->stream>>>(c->g, src, arr, n);
-    else k_pack<<<blocks, 256, 0, c->stream>>>(c->g, arr, dst, n);
+    const long long rows = (long long)c->nv * ((c->desc.dim == 2) ? c->desc.ny : 1);
+    const dim3 blk(32, 8), grid((unsigned)std::min<long long>((c->desc.nx + 31) / 32, 8192),
+                                (unsigned)std::min<long long>((rows + 7) / 8, 8192));
+    if (in) k_copy_interior<true><<<grid, blk, 0, c->stream>>>(c->g, src, arr, shadow);
+    else k_copy_interior<false><<<grid, blk, 0, c->stream>>>(c->g, arr, dst, nullptr);
     CK(cudaGetLastError());
     ++c->launches;
     if (host && !in)
@@ -663,14 +674,8 @@ gks_status gks_set_state(gks_ctx* c, const double* W, int on_device)
     if (!c || !W) return GKS_EINVAL;
     c->cfl_dt_ready = false;
     c->hs_fresh = false;
-    gks_status s = copy_interior(c, c->W, W, on_device, true, false);
+    gks_status s = copy_interior(c, c->W, W, on_device, true, false, c->Wf);
     if (s) return s;
-    if (c->Wf) {
-        const long long n = (long long)c->nv * c->g.plane;
-        k_to_float<<<(int)((n + 255) / 256 > 4096 ? 4096 : (n + 255) / 256), 256, 0, c->stream>>>(c->W, c->Wf, n);
-        CK(cudaGetLastError());
-        ++c->launches;
-    }
     k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 2, 0.0, INFINITY, 0);
     CK(cudaGetLastError());
     ++c->launches;

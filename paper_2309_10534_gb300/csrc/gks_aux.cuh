@@ -55,21 +55,16 @@ __global__ void __launch_bounds__(256) k_sigma(GridDev g, const double* __restri
     unsigned int err = 0;
     const int nv = g.dim + 2;
     const double h = (g.dim == 2) ? fmin(g.dx, g.dy) : g.dx;
-    const long long ncell = (long long)g.nx * (g.dim == 2 ? g.ny : 1);
-    for (long long c = blockIdx.x * 256ll + threadIdx.x; c < ncell; c += 256ll * gridDim.x) {
-        const int i = (int)(c % g.nx), j = (int)(c / g.nx);
+    const T gamma = (T)g.gamma, mu = (T)g.mu, th = (T)h;
+    const unsigned ncell = (unsigned)((long long)g.nx * (g.dim == 2 ? g.ny : 1));  // at most 2^31
+    for (unsigned c = blockIdx.x * 256u + threadIdx.x; c < ncell; c += 256u * gridDim.x) {
+        const unsigned j = g.dim == 2 ? c / (unsigned)g.nx : 0u, i = c - j * (unsigned)g.nx;
         const long long off = (long long)(g.dim == 2 ? j + NG : 0) * g.pitch + i + NG;
-        double w[4];
-        for (int v = 0; v < nv; ++v) w[v] = W[(long long)v * g.plane + off];
-        s = fmax(s, cell_sigma<T>(w, g.dim, (T)g.gamma, (T)g.mu, (T)h, err));
+        T w[4];
+        for (int v = 0; v < nv; ++v) w[v] = from_f64<T>(W[(long long)v * g.plane + off]);
+        s = fmax(s, cell_sigma<T, T>(w, g.dim, gamma, mu, th, err));
     }
     block_commit<256, T>(s, true, err, 0u, ds, false);
-}
-
-// float32 shadow of a float64 array (same layout)
-__global__ void k_to_float(const double* __restrict__ W, float* __restrict__ Wf, long long n)
-{
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x) Wf[i] = narrow(W[i]);
 }
 
 // float64 views of the float32 path's stage buffers (gks_get_buffer):

@@ -67,8 +67,10 @@ gks_status fill_ghosts(gks_ctx* c, void* arr, cudaStream_t st);
 // context's precision; diagnostics that read W itself)
 gks_status fill_ghosts_f64(gks_ctx* c, double* arr, cudaStream_t st);
 // copy the interior [nv][ny][nx] between a caller's buffer and a ghosted array
-// (wait = false: the caller synchronises the stream before it returns)
-gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device, bool in, bool wait = true);
+// (wait = false: the caller synchronises the stream before it returns;
+// shadow: a float32 copy of the interior, in the same layout)
+gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device, bool in, bool wait = true,
+                         float* shadow = nullptr);
 HostFlux host_flux(const gks_ctx* c);
 TenoParams teno_params(const gks_ctx* c, bool tangential);
 
