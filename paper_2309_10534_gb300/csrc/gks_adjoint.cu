@@ -13,7 +13,7 @@
 //                      + [d dF/dW^n]^T (dt^2/h Delta(lam/6 + lam*/8))
 // with Delta lam the difference of lam across a face (zero outside the
 // interior).  The transposed flux Jacobian of one direction is applied by
-// four kernels on the stage input:
+// three kernels on the stage input:
 //   k_adj_lines   normal TENO-D per cell -> face-line values and slopes
 //                 (the forward sweep's phase 1)
 //   k_adj_gauss   per face segment and Gauss point: tangential TENO-D to the
@@ -21,10 +21,9 @@
 //                 the transposed tangential reconstruction; sums, per tile,
 //                 the contributions to each line row, and writes the tile's
 //                 own rows and the two rows beyond each of its edges
-//   k_adj_normal  per cell: gathers the line cotangents of its two faces and
-//                 applies the transposed normal reconstruction; writes its
-//                 contributions to the five cells of its stencil
-//   k_adj_gather  per cell: sums the contributions it received
+//   k_adj_normal  per cell: gathers the line cotangents of its two faces,
+//                 applies the transposed normal reconstruction and sums what
+//                 the cells of its neighbourhood contribute to it
 // and the ghost layers are folded back onto the interior cells they copy
 // (the transpose of the ghost fill).  TENO-D selections are recomputed from
 // the same stage inputs as in the forward pass, i.e. frozen at the forward
@@ -66,7 +65,6 @@ struct AdjDir {
     float fcF1, fcD1, fcF2, fcD2, fihn, fiht;
     void* lines;          // [NQ][faces nn+1][rows nt+4]
     void* contrib;        // line cotangents: [NQ][faces nn+1][rows ntp], then [NQ][faces][tiles][4] edge rows
-    void* dcell;          // [5][4][cells nn+2][rows nt+4]
     double* gW;           // ghosted gradient accumulator
     int dirn, nn, nt;
     int tiles, ntp;       // Gauss-row tiles of adj_tile(dirn) rows, rows padded to whole tiles
@@ -100,12 +98,6 @@ __device__ __forceinline__ long long eidx(const AdjDir& a, int f, int tile, int 
 {
     return D == 0 ? (long long)(tile * 4 + e) * (a.nn + 1) + f : (long long)f * (a.tiles * 4) + tile * 4 + e;
 }
-template <int D>
-__device__ __forceinline__ long long didx(const AdjDir& a, int i, int r)
-{
-    return D == 0 ? (long long)(r + 2) * (a.nn + 2) + (i + 1) : (long long)(i + 1) * (a.nt + 4) + (r + 2);
-}
-
 // a direction scalar in the arithmetic type
 template <typename T>
 __device__ __forceinline__ T scal(double d, float f)
@@ -262,6 +254,13 @@ __global__ void __launch_bounds__(256) k_adj_lines(GridDev g, AdjDir a, TenoT<T>
 // by k_adj_normal) was most of both kernels' memory traffic; the block's 128
 // segments now add theirs up in shared memory, and 1.25 to 1.5 values per
 // segment and quantity go out.
+//
+// Bound by its chain of dependent arithmetic at few warps per SM, so float32
+// runs three blocks of 256 threads at 80 registers (some values spill) rather
+// than two at 128, and a segment that keeps its large stencils throughout (one
+// compare of its codes) skips the sub-stencils: with the direction a template
+// parameter, 12 steps and their reverse on a 512^2 float32 plane 9.86 -> 9.07
+// ms, 4 on a 96^2 float64 plane 5.45 -> 5.35 ms.
 template <typename T, int D>
 __global__ void __launch_bounds__(2 * ADJ_PAIRS<T>, (sizeof(T) == 4) ? 3 : 2)
 k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
@@ -432,20 +431,32 @@ k_adj_gauss(GridDev g, AdjDir a, FluxParams<T> fp, TenoT<T> tt)
     }
 }
 
-// ---- per cell: line cotangents of its faces -> transposed normal TENO-D
+// ---- per cell: line cotangents of its faces -> transposed normal TENO-D,
+// and the sum of what the cells around hand it.  The block's cells lie along
+// the normal (x faces: 128, y faces: 32 rows of 8); the contributions meet in
+// shared memory, so only the inner cells (all but two at either end) are the
+// block's own.  The five contributions of a cell through memory and a gather
+// kernel of its own took 22 + 11 us on a 512^2 float32 plane
+// (its gradient over 12 steps 9.07 -> 8.89 ms, 4 steps of a 96^2 float64
+// plane 5.35 -> 5.19 ms).
+template <int D> constexpr int ADJ_NX = D == 0 ? 128 : 8;  // block shape
+template <int D> constexpr int ADJ_NY = 256 / ADJ_NX<D>;
+template <int D> constexpr int ADJ_OWN = (D == 0 ? ADJ_NX<D> : ADJ_NY<D>) - 4;  // own cells along the normal
+
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_adj_normal(GridDev g, AdjDir a, TenoT<T> tn)
 {
-    int i, r;
-    map2<D>(i, r, -1, -2);
-    if (i > a.nn || r >= a.nt + 2) return;
+    __shared__ T part[2][5][256];
+    const int tid = threadIdx.y * ADJ_NX<D> + threadIdx.x;
+    // cell i (two before the block's first own cell onwards), line row r
+    const int k = D == 0 ? threadIdx.x : threadIdx.y;
+    const int i = (int)blockIdx.y * ADJ_OWN<D> - 5 + k;
+    const int r = (int)(D == 0 ? blockIdx.x * ADJ_NY<D> + threadIdx.y : blockIdx.x * ADJ_NX<D> + threadIdx.x) - 2;
     const bool swap = D != 0;
     const long long org = (long long)NG * g.pitch + NG;
     const long long MP = (long long)(a.nn + 1) * a.ntp, EP = (long long)(a.nn + 1) * a.tiles * 4;
-    const long long DP = (long long)(a.nn + 2) * (a.nt + 4);
     const T* M = static_cast<const T*>(a.contrib);
     const T* Eg = M + NQ * MP;
-    T* dc = static_cast<T*>(a.dcell);
     const T ih = scal<T>(a.ihn, a.fihn);
     // line row r: its tile's sum, and the edge rows of the tiles beside it
     const int TT = adj_tile(D, sizeof(T) == 4);
@@ -465,8 +476,11 @@ __global__ void __launch_bounds__(256) k_adj_normal(GridDev g, AdjDir a, TenoT<T
         if (e2 >= 0) acc += Eg[q * EP + eidx<D>(a, f, t2, e2)];
         return acc;
     };
-    {
-        const int vv = 2 * (int)blockIdx.z;  // variable pairs, as the forward's selection
+    const int vv = 2 * (int)blockIdx.z;  // variable pairs, as the forward's selection
+    if (i < -1 || i > a.nn || r >= a.nt + 2) {
+#pragma unroll
+        for (int s = 0; s < 10; ++s) part[s / 5][s % 5][tid] = T(0);
+    } else {
         T q[2][5];
 #pragma unroll
         for (int l = 0; l < 2; ++l) {
@@ -493,31 +507,18 @@ __global__ void __launch_bounds__(256) k_adj_normal(GridDev g, AdjDir a, TenoT<T
             T gq[5] = {T(0), T(0), T(0), T(0), T(0)};
             teno_faces_T(S, gvp, gdp, gvm, gdm, gq);
 #pragma unroll
-            for (int s = 0; s < 5; ++s) dc[(long long)(s * 4 + v) * DP + didx<D>(a, i, r)] = gq[s];
+            for (int s = 0; s < 5; ++s) part[l][s][tid] = gq[s];
         }
     }
-}
-
-// ---- per cell: sum of the contributions of the cells whose stencil holds it
-template <typename T, int D>
-__global__ void __launch_bounds__(256) k_adj_gather(GridDev g, AdjDir a)
-{
-    int j, r;
-    map2<D>(j, r, -3, -2);
-    if (j > a.nn + 2 || r >= a.nt + 2) return;
-    const bool swap = D != 0;
-    const long long org = (long long)NG * g.pitch + NG;
-    const long long DP = (long long)(a.nn + 2) * (a.nt + 4);
-    const T* dc = static_cast<const T*>(a.dcell);
+    __syncthreads();
+    if (k < 2 || k >= 2 + ADJ_OWN<D> || i > a.nn + 2 || r >= a.nt + 2) return;
+    constexpr int step = D == 0 ? 1 : ADJ_NX<D>;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
+    for (int l = 0; l < 2; ++l) {
         T acc = T(0);
 #pragma unroll
-        for (int s = 0; s < 5; ++s) {
-            const int i = j + 2 - s;  // cell i's stencil position s is cell i - 2 + s = j
-            if (i >= -1 && i <= a.nn) acc += dc[(long long)(s * 4 + v) * DP + didx<D>(a, i, r)];
-        }
-        a.gW[(long long)gvar_(v, swap) * g.plane + org + j * a.sn + r * a.st] += to_f64(acc);
+        for (int s = 0; s < 5; ++s) acc += part[l][s][tid + (2 - s) * step];  // cell i + 2 - s holds i at its position s
+        a.gW[(long long)gvar_(vv + l, swap) * g.plane + org + i * a.sn + r * a.st] += to_f64(acc);
     }
 }
 
@@ -600,7 +601,7 @@ struct gks_adjoint {
     std::vector<void*> seg, segs;
     double* WN = nullptr;        // final state of the forward pass
     double *lam = nullptr, *lams = nullptr, *gacc = nullptr, *nxt = nullptr;
-    void *lines = nullptr, *contrib = nullptr, *dcell = nullptr;
+    void *lines = nullptr, *contrib = nullptr;
     long long launches = 0;
     // one full segment's recomputation and reverse sweep, captured once and
     // replayed for every full segment (fixed buffers; dt and the context's
@@ -633,10 +634,8 @@ gks_status adj_scratch(gks_adjoint* A)
         const long long tiles = (nt + tt - 1) / tt;
         contrib = std::max(contrib, (nn + 1) * tiles * (tt + 4) * NQ);
     }
-    const long long dcell = std::max((nx + 2) * (ny + 4), (ny + 2) * (nx + 4)) * 20;
     CK(cudaMalloc(&A->lines, lines * es));
     CK(cudaMalloc(&A->contrib, contrib * es));
-    CK(cudaMalloc(&A->dcell, dcell * es));
     gks_status s;
     if ((s = adj_alloc(A, &A->lam)) || (s = adj_alloc(A, &A->lams)) || (s = adj_alloc(A, &A->gacc)) ||
         (s = adj_alloc(A, &A->nxt)))
@@ -678,10 +677,11 @@ gks_status sweep_vjp_t(gks_adjoint* A, AdjDir d)
     gcell.z = 2;
     k_adj_lines<T, D><<<gcell, b256, 0, st>>>(g, d, tn);
     k_adj_gauss<T, D><<<grid_for(d.nn + 1, d.nt, bg, 2), bg, 0, st>>>(g, d, fp, tt);
-    k_adj_normal<T, D><<<gcell, b256, 0, st>>>(g, d, tn);
-    k_adj_gather<T, D><<<grid_for(d.nn + 6, d.nt + 4, b256, 1), b256, 0, st>>>(g, d);
+    constexpr int across = D == 0 ? ADJ_NY<D> : ADJ_NX<D>;
+    const dim3 gn((d.nt + 4 + across - 1) / across, (d.nn + 6 + ADJ_OWN<D> - 1) / ADJ_OWN<D>, 2);
+    k_adj_normal<T, D><<<gn, dim3(ADJ_NX<D>, ADJ_NY<D>), 0, st>>>(g, d, tn);
     CK(cudaGetLastError());
-    A->launches += 4;
+    A->launches += 3;
     return GKS_OK;
 }
 
@@ -705,7 +705,6 @@ gks_status stage_vjp(gks_adjoint* A, const void* input, const double* lam1, cons
         d.cD2 = cD2 / h;
         d.lines = A->lines;
         d.contrib = A->contrib;
-        d.dcell = A->dcell;
         d.gW = A->gacc;
         d.dirn = dirn;
         if (dirn == 0) {
@@ -851,7 +850,6 @@ void gks_adjoint_destroy(gks_adjoint* A)
     cudaFree(A->nxt);
     cudaFree(A->lines);
     cudaFree(A->contrib);
-    cudaFree(A->dcell);
     delete A;
 }
 

@@ -358,8 +358,8 @@ __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(cons
 
     const int pl = (int)g.plane;  // a 1-D plane is one ghosted row
     // the update's other inputs, requested before the stage's arithmetic: read
-    // in the update they cost its warps a memory round trip each (stage 2 of a
-    // 2^22-cell float32 tube: @T32@)
+    // in the update they cost its warps a memory round trip each (four steps of
+    // a 2^22-cell float32 tube 1702 -> 1688 us)
     const int ui = i0 + tid, uo = ui + NG;
     const bool own = tid < TN && ui < g.nx;
     double ubase[3] = {0.0, 0.0, 0.0};
@@ -895,7 +895,8 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     }
     copy_commit();
     // y sweep: start copying the update's inputs (read in the update, they
-    // cost its warps a memory round trip: @T2D@)
+    // cost its warps a memory round trip: four steps of a 64^2 float32 plane
+    // 292 -> 281 us, two of a 1024^2 plane the same)
     const bool base_f = sizeof(T) == 4 && a.stage == 1;
     if (a.pass == 1) {
         for (int k = tid; k < TN * TT; k += NT) {
