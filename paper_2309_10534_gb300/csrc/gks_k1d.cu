@@ -9,7 +9,7 @@ cudaError_t launch_one(const GridDev& g, const Stage1DArgs& a, const HostFlux& h
                        DevState* ds, cudaStream_t st)
 {
     if constexpr (!PRFIX && REC != REC_TENO_CHAR) {
-        if (hf.merge == 0 && g.nx <= (sizeof(T) == 8 ? STAGE1D_WIDE_NX64 : STAGE1D_WIDE_NX32)) {
+        if (hf.merge == 0 && g.nx <= STAGE1D_WIDE_NX) {
             k1d_stage_wide<T, NONEQ, REC><<<(g.nx + WIDE_TN - 1) / WIDE_TN, 96, 0, st>>>(
                 g, a, make_flux_params<T>(hf), teno_t<T>(tn), ds);
             return cudaGetLastError();

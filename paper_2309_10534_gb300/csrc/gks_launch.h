@@ -15,9 +15,15 @@ constexpr int SWEEP_TN = 31;
 // cells per block of the 1-D stage (TN + 2 = 128 threads: one per
 // reconstructed cell, face and updated cell)
 constexpr int STAGE1D_TN = 126;
-// up to these many cells a 1-D stage takes k1d_stage_wide
-constexpr int STAGE1D_WIDE_NX64 = 9120;
-constexpr int STAGE1D_WIDE_NX32 = 9120;
+// Up to 160 cells per SM a 1-D stage takes k1d_stage_wide: its tiles of 30
+// cells and three warps have a third of the chain of a 126-cell tile and fill
+// the SMs sooner, but reconstruct 32 cells for 30; once several blocks share
+// every SM, the 126-cell tiles move more cells.  One step, us (wide / 126), in
+// float64 TENO-D, float64 WENO5-AO and float32 TENO-D: 400 cells 37 / 76,
+// 43 / 96, 12.2 / 15.7; 12 000 cells 51 / 71, 69 / 95, 13.5 / 15.3; 24 000
+// cells 86 / 98, 130 / 156, 14.6 / 16.9; 28 000 cells 101 / 96, 154 / 157,
+// 15.5 / 15.4; 128 000 cells 353 / 316, 573 / 525, 37 / 20.
+constexpr int STAGE1D_WIDE_NX = 152 * 160;
 
 struct HostFlux {
     double gamma, K, ntot, c1, c2, mu, prfac;
