@@ -326,6 +326,21 @@ __device__ __noinline__ void load_edge_1d(T* sq, const E* src, const GridDev& g,
     }
 }
 
+// 4- or 8-byte copies from global to shared memory that the thread waits for
+// only when it reads them
+template <int B>
+__device__ __forceinline__ void copy_async(void* dst, const void* src)
+{
+    static_assert(B == 4 || B == 8, "cp.async size");
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if constexpr (B == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the last N committed groups of this thread are done
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 template <typename T, bool NONEQ, bool PRFIX, int TN, int REC = 0>
 __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(const __grid_constant__ GridDev g, Stage1DArgs a,
                                                     FluxParams<T> fp, TenoT<T> tn, DevState* ds)
@@ -357,24 +372,8 @@ __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(cons
     const int slot[3] = {0, 1, 3};
 
     const int pl = (int)g.plane;  // a 1-D plane is one ghosted row
-    // the update's other inputs, requested before the stage's arithmetic: read
-    // in the update they cost its warps a memory round trip each (four steps of
-    // a 2^22-cell float32 tube 1702 -> 1688 us)
     const int ui = i0 + tid, uo = ui + NG;
     const bool own = tid < TN && ui < g.nx;
-    double ubase[3] = {0.0, 0.0, 0.0};
-    T uacc[3] = {T(0), T(0), T(0)};
-    if (own && (a.stage == 2 || sizeof(T) == 8)) {
-#pragma unroll
-        for (int v = 0; v < 3; ++v) {
-            if constexpr (sizeof(T) == 4) {
-                ubase[v] = a.base[v * pl + uo];
-                uacc[v] = a.accf[v * pl + uo];
-            } else {
-                ubase[v] = a.stage == 1 ? a.src[v * pl + uo] : a.acc[v * pl + uo];
-            }
-        }
-    }
     // one loop per source type: a per-element choice between the float32
     // and the converted float64 source was compiled as both, and every
     // element then paid a float64 -> float32 conversion on the slow float64
@@ -386,6 +385,12 @@ __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(cons
             return;
         }
         static_assert(TN + 6 - NT == 4, "four cells beyond one per thread");
+        if constexpr (std::is_same<decltype(src), const T*>::value) {
+#pragma unroll
+            for (int v = 0; v < 3; ++v) copy_async<sizeof(T)>(&sq[v][tid], src + (v * pl + i0 + tid));
+            if (tid < 12) copy_async<sizeof(T)>(&sq[tid >> 2][NT + (tid & 3)], src + ((tid >> 2) * pl + i0 + NT + (tid & 3)));
+            return;
+        }
 #pragma unroll
         for (int v = 0; v < 3; ++v) sq[v][tid] = load_as<T>(src[v * pl + i0 + tid]);
         if (tid < 12) sq[tid >> 2][NT + (tid & 3)] = load_as<T>(src[(tid >> 2) * pl + i0 + NT + (tid & 3)]);
@@ -396,6 +401,26 @@ __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(cons
     } else {
         load(a.src);
     }
+    copy_commit();
+    // the update's other inputs, on their way while the stage computes: read in
+    // the update they cost its warps a memory round trip each (four steps of a
+    // 2^22-cell float32 tube 1541 -> 1465 us against reads at the update's or the
+    // stage's start into registers, which also took 64 registers instead of 56)
+    __shared__ double s_base[3][TN];
+    __shared__ float s_acc[3][sizeof(T) == 4 ? TN : 1];
+    if (own && (a.stage == 2 || sizeof(T) == 8)) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            if constexpr (sizeof(T) == 4) {
+                copy_async<8>(&s_base[v][tid], a.base + (v * pl + uo));
+                copy_async<4>(&s_acc[v][tid], a.accf + (v * pl + uo));
+            } else {
+                copy_async<8>(&s_base[v][tid], (a.stage == 1 ? a.src : a.acc) + (v * pl + uo));
+            }
+        }
+    }
+    copy_commit();
+    copy_wait<1>();  // the tile
     __syncthreads();
     fp.dt = s_scal[0];
     const T idx_ = s_scal[2];
@@ -483,6 +508,7 @@ __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(cons
     T sig = T(0);
     const double cx = dt * a.idx;
     const T cxt = s_scal[1];
+    copy_wait<0>();
     if (own) {
         const int c = tid, o = uo;
         T w[4];
@@ -494,15 +520,15 @@ __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(cons
                     a.out0f[v * pl + o] = wstar32(sq[v][c + 3], cxt, d0);
                     a.out1f[v * pl + o] = cxt * (sG[1][v][c + 1] - sG[1][v][c]);
                 } else {
-                    const double r = wnew32(ubase[v], uacc[v], cxt, d0);
+                    const double r = wnew32(s_base[v][tid], s_acc[v][tid], cxt, d0);
                     a.out0[v * pl + o] = r;
                     w[v] = narrow(r);
                     if (a.out0f) a.out0f[v * pl + o] = w[v];
                 }
             } else {
-                const double r = upd64(ubase[v], cx, (double)d0);
+                const double r = upd64(s_base[v][tid], cx, (double)d0);
                 a.out0[v * pl + o] = r;
-                if (a.stage == 1) a.out1[v * pl + o] = upd64(ubase[v], cx, (double)(sG[1][v][c + 1] - sG[1][v][c]));
+                if (a.stage == 1) a.out1[v * pl + o] = upd64(s_base[v][tid], cx, (double)(sG[1][v][c + 1] - sG[1][v][c]));
                 w[v] = (T)r;
             }
         }
@@ -785,21 +811,6 @@ template <typename T, int TN, int TT, bool CONV = false> struct SweepSmem {
     // slope per face and row (Step 2)
     T w0[CONV ? 2 : 1][4][CONV ? TT + 4 : 1][CONV ? TN + 1 : 1];
 };
-
-// 4- or 8-byte copies from global to shared memory that the thread waits for
-// only when it reads them
-template <int B>
-__device__ __forceinline__ void copy_async(void* dst, const void* src)
-{
-    static_assert(B == 4 || B == 8, "cp.async size");
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    if constexpr (B == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// all but the last N committed groups of this thread are done
-template <int N>
-__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // the cells of a tile that reaches past the boundary, ghosts by the boundary
 // rules (out of line: the other tiles keep their registers)
