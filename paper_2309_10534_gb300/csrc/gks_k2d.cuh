@@ -10,12 +10,15 @@ namespace gks {
 template <typename T, int TT, int NT, int MB>
 struct SweepTile {
     template <bool NONEQ, bool PRFIX, int REC>
-    static cudaError_t one(const GridDev& g, const SweepArgs& a, const FluxParams<T>& fp, const TenoParams& tn,
+    static cudaError_t one(const GridDev& g, SweepArgs a, const FluxParams<T>& fp, const TenoParams& tn,
                            const TenoParams& tt, DevState* ds, cudaStream_t st)
     {
         constexpr int TN = SWEEP_TN;
         const size_t smem = sizeof(SweepSmem<T, TN, TT, rec_conventional(REC)>);
-        dim3 grid((a.nn + TN - 1) / TN, (a.nt + TT - 1) / TT);
+        const unsigned cols = (a.nn + TN - 1) / TN, rows = (a.nt + TT - 1) / TT;
+        const bool fits = sizeof(T) == 4 || rows <= 65535;  // float32: 16 rows a tile where 8 are too many
+        a.cols = fits ? 0 : (int)cols;
+        const dim3 grid(fits ? cols : cols * rows, fits ? rows : 1);
         k2d_sweep<T, NONEQ, PRFIX, TN, TT, NT, MB, REC><<<grid, NT, smem, st>>>(g, a, fp, teno_t<T>(tn), teno_t<T>(tt), ds);
         return cudaGetLastError();
     }

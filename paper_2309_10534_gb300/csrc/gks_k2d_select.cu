@@ -52,7 +52,7 @@ cudaError_t launch_sweep_f32(const GridDev& g, const SweepArgs& a, const HostFlu
     if (blocks(a, 4) <= sms) return sweep_f32_t4(g, a, hf, tn, tt, ds, st);
     // waves of two blocks per SM, weighted by a block's time
     const long long w16 = 10 * ((b16 + 2 * sms - 1) / (2 * sms)), w8 = 6 * ((b8 + 2 * sms - 1) / (2 * sms));
-    return w16 <= w8 ? sweep_f32_t16(g, a, hf, tn, tt, ds, st) : sweep_f32_t8(g, a, hf, tn, tt, ds, st);
+    return w16 <= w8 || a.nt > 65535 * 8 ? sweep_f32_t16(g, a, hf, tn, tt, ds, st) : sweep_f32_t8(g, a, hf, tn, tt, ds, st);
 }
 
 // float64: 4 rows (128 threads at 206 registers, two blocks per SM, which

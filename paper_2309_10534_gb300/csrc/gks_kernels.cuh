@@ -791,6 +791,8 @@ struct SweepArgs {
     int with_sigma;
     int commit;          // the last block commits the step
     int sms;             // multiprocessors of the device (tile choice)
+    int cols;            // float64, > 0: more rows of tiles than a grid's y extent takes;
+                         // tiles are numbered along x, cols to a row
 };
 
 // global variable index of local variable v (swap: faces normal to y)
@@ -844,7 +846,6 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
 {
     if (ds->done) return;
     constexpr int NF = TN + 1;           // faces per tile row
-    constexpr int NP = TT * NF;          // (face, row) pairs
     constexpr int NW = NT / 32;
     constexpr bool CONV = rec_conventional(REC);
     constexpr int RB = rec_base(REC);  // the tangential (per-quantity) reconstruction
@@ -873,7 +874,9 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
         s_scal[5] = (T)g.mu;
         s_scal[6] = (T)a.hmin;
     }
-    const int n0 = blockIdx.x * TN, t0 = blockIdx.y * TT;
+    const int cols = sizeof(T) == 8 ? a.cols : 0;
+    const int n0 = (cols ? blockIdx.x % cols : blockIdx.x) * TN;
+    const int t0 = (cols ? blockIdx.x / cols : blockIdx.y) * TT;
     static_assert(TN == 31, "lanes of a warp along the tile's faces");
     // local frame: normal momentum first; y faces swap the two momentum components
     const bool swap = a.dirn != 0;
@@ -932,6 +935,16 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     __syncthreads();
     fp.dt = s_scal[0];
 
+    // The last tiles of a line or column do only their own work.  float64,
+    // whose blocks' time is their work on the slow pipe, counts through the
+    // tile's nf faces and nr rows alone (4 steps and their reverse on 96^2,
+    // four tiles of 31 where the last holds 3 cells: 5.18 -> 4.60 ms).  float32
+    // skips the warps that lie outside (two steps of 2048 x 1024 viscous cells
+    // 3213 -> 3182 us); counting costs it registers (1024^2 1316 -> 1344 us).
+    constexpr bool COUNT = sizeof(T) == 8;
+    const int nf = COUNT ? min(NF, a.nn - n0 + 1) : NF, nr = COUNT ? min(TT, a.nt - t0) : TT;
+    const bool whole = !COUNT || nf == NF;
+
     // phase 1: normal TENO-D per (cell, row, var): cell c <-> normal n0-1+c
     if constexpr (REC == REC_TENO_CHAR) {
         // characteristic variables: per (face, row), the six cells around
@@ -964,6 +977,7 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
             const int e = line ? k : (k - NL) * 32 + lane, c = line ? lane : 32;
             if (e >= NL) continue;
             const int vv = 2 * (e & 1), r = e >> 1;
+            if (t0 - 2 + r > a.nt + 1) continue;  // no Gauss point reads this row
             f2 q[5];
 #pragma unroll
             for (int s = 0; s < 5; ++s) q[s] = f2(sm.w[vv][r][c + s], sm.w[vv + 1][r][c + s]);
@@ -981,12 +995,19 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
         }
     } else {
         const T ih = s_scal[2];
-        constexpr int NL = 4 * (TT + 4);  // (row, variable) lines, as above
-        for (int k = warp; k < NL + (NL + 31) / 32; k += NW) {
-            const bool line = k < NL;
-            const int e = line ? k : (k - NL) * 32 + lane, c = line ? lane : 32;
+        // (row, variable) lines as above; narrow tiles count through their cells
+        const int NL = 4 * (nr + 4), NK = whole ? 32 * (NL + (NL + 31) / 32) : NL * (nf + 1);
+        for (int k = tid; k < NK; k += NT) {
+            const int w = k >> 5;
+            const bool line = w < NL;
+            int e = line ? w : (w - NL) * 32 + lane, c = line ? lane : 32;
+            if (!whole) {
+                e = k / (nf + 1);
+                c = k - e * (nf + 1);
+            }
             if (e >= NL) continue;
             const int v = e & 3, r = e >> 2;
+            if (t0 - 2 + r > a.nt + 1) continue;
             T q[5];
 #pragma unroll
             for (int s = 0; s < 5; ++s) q[s] = sm.w[v][r][c + s];
@@ -1047,12 +1068,15 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     const T tdt = s_scal[0];
     const T iht = s_scal[3];
     const T gA = T(-0.28867513459481288), gB = T(0.28867513459481288);  // -+1/(2 sqrt 3)
+    const int np = nr * nf;
 #pragma unroll 1
-    for (int task = tid; task < 2 * NP; task += NT) {  // 2 NP is a multiple of NT: whole warps
-        const int pair = task >> 1, gpi = task & 1;
-        const int r = pair / NF, f = pair % NF;
+    for (int task = tid; (task & ~31) < 2 * np; task += NT) {  // whole warps
+        // lanes past the last pair repeat it
+        const int pair = COUNT ? min(task >> 1, np - 1) : task >> 1, gpi = task & 1;
+        const int r = whole ? pair / NF : pair / nf, f = pair - r * nf;
         // faces n0+f <= nn on rows t0+r < nt exist; the rest of the tile is padding
-        const bool valid = (n0 + f <= a.nn) && (t0 + r < a.nt);
+        const bool valid = COUNT || ((n0 + f <= a.nn) && (t0 + r < a.nt));
+        if (!COUNT && !__any_sync(0xffffffffu, valid)) continue;
         const T gs = gpi ? gB : gA;
         Side<T> L, R;  // own side, partner's side
 #pragma unroll
@@ -1101,7 +1125,7 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
                 const int side = k ^ gpi;  // 0: left, 1: right
 #pragma unroll
                 for (int v = 0; v < 4; ++v) { S.W[v] = sm.w[v][r + 2][f + 2 + side]; S.Wn[v] = S.Wt[v] = T(0); }
-                ++nfb;
+                nfb += task < 2 * np;
                 if (!prim_state<T, 2>(S.W, fp.gm1, p)) err |= 2u;
             };
             if constexpr (CONV) {
@@ -1124,7 +1148,7 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
                 if (physical<T, 2>(w0g, fp.gm1)) {
                     point_flux<T, 2, NONEQ, PRFIX>(L, R, gpi ? T(-1) : T(1), fp, F, dF, a.stage == 1, state, w0n, w0g, w0t);
                 } else {
-                    ++nfb;
+                    nfb += task < 2 * np;
                     point_flux<T, 2, NONEQ, PRFIX>(L, R, gpi ? T(-1) : T(1), fp, F, dF, a.stage == 1, state);
                 }
             } else {
@@ -1159,7 +1183,6 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     copy_wait<0>();
     T sig = T(0);
     const T cn = s_scal[1];
-    static_assert((2 * NP) % NT == 0, "whole warps of tasks");
 #pragma unroll 1
     for (int k = tid; k < TN * TT; k += NT) {
         // x faces: the normal (x) index fastest; y faces: the tangential (x) index

@@ -5,7 +5,7 @@
 // by another allocator (a framework's caching allocator, or a fixed memory
 // budget handed out by a scheduler), or a latency-critical loop that cannot
 // afford cudaMalloc's implicit device-wide synchronisation.  For them the
-// working buffers of the step (ghosted copies of W^n and W*, the stage
+// working buffers of the step (W^n and W* in the ghosted layout, the stage
 // accumulator, the new state and the small device-side step state) live in
 // one file-scope static __device__ array, sized for at most
 // GKS_NOALLOC_MAX_NX cells (about 1.6 MB, held by every GPU that loads the

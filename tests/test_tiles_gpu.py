@@ -133,3 +133,22 @@ def test_vjp_at_tile_remainders(gks, nx, ny, precision, tol):
     h = 1e-6
     fd = (O.step(P, W + h * d, dt) - O.step(P, W - h * d, dt)) / (2 * h)
     assert abs(float((gin * d).sum()) - float((g * fd).sum())) <= tol * float(np.abs(g * fd).sum())
+
+
+@pytest.mark.parametrize("nx,ny", [(3, 264000), (264000, 3)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_more_rows_of_tiles_than_a_grid_extent_takes(gks, nx, ny, precision):
+    """A long periodic strip made of copies of a short one stays that: every
+    copy takes the short strip's values (the same cells in other tiles)."""
+    k = 2000
+    sx, sy = (nx, ny // k) if ny > nx else (nx // k, ny)
+    W = WL.random_smooth_2d(sx, sy, seed=9, kmax=1)
+    kw = dict(bc=("periodic",) * 4, precision=precision)
+    a = gks.Solver(2, sx, sy, lx=float(sx), ly=float(sy), **kw)
+    b = gks.Solver(2, nx, ny, lx=float(nx), ly=float(ny), **kw)
+    a.set_state(W)
+    b.set_state(np.tile(W, (1, k, 1) if ny > nx else (1, 1, k)))
+    a.step(0.2)
+    b.step(0.2)
+    ref = a.get_state()
+    assert rel_l1(b.get_state(), np.tile(ref, (1, k, 1) if ny > nx else (1, 1, k))) < (1e-14 if precision == "fp64" else 1e-7)
