@@ -55,14 +55,18 @@ cudaError_t launch_sweep_f32(const GridDev& g, const SweepArgs& a, const HostFlu
     return w16 <= w8 || a.nt > 65535 * 8 ? sweep_f32_t16(g, a, hf, tn, tt, ds, st) : sweep_f32_t8(g, a, hf, tn, tt, ds, st);
 }
 
-// float64: 4 rows (128 threads at 206 registers, two blocks per SM, which
-// cover each other's barriers); 2 rows where even those leave SMs idle.  One
-// step, ms (8 rows in one 256-thread block / 4 / 2): 64^2 0.83 / 0.55 / 0.37,
-// 96^2 0.82 / 0.54 / 0.57, 400^2 3.11 / 2.89 / 3.09, 1024^2 16.8 / 16.5 / 18.0.
+// float64: 4 rows (128 threads at 210 registers, two blocks per SM, which
+// cover each other's barriers); 2 rows where even those leave SMs idle (a last
+// column of less than 8 cells is a small part of a block's work).  One step,
+// ms (8 rows in one 256-thread block / 4 / 2), when the last tiles of a line
+// were whole: 64^2 0.83 / 0.55 / 0.37, 400^2 3.11 / 2.89 / 3.09, 1024^2 16.8 /
+// 16.5 / 18.0; since they do only their own work (4 / 2): 96^2 0.350 / 0.337,
+// 100^2 0.348 / 0.336, and 64^2 0.209, 400^2 2.53 with the choice made here.
 cudaError_t launch_sweep_f64(const GridDev& g, const SweepArgs& a, const HostFlux& hf, const TenoParams& tn,
                              const TenoParams& tt, DevState* ds, cudaStream_t st)
 {
-    if (blocks(a, 2) <= std::max(1, a.sms)) return sweep_f64_t2(g, a, hf, tn, tt, ds, st);
+    const long long full = std::max(1ll, ((long long)a.nn + SWEEP_TN - 8) / SWEEP_TN) * ((a.nt + 1ll) / 2);
+    if (full <= std::max(1, a.sms)) return sweep_f64_t2(g, a, hf, tn, tt, ds, st);
     return sweep_f64_t4(g, a, hf, tn, tt, ds, st);
 }
 

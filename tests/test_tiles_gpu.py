@@ -76,7 +76,7 @@ def test_1d_weno_family_at_tile_edges(gks, nx, recon):
 
 # float32: 4 rows while its blocks fit the SMs, then 8, 16 where those fill
 # the chip's last wave better; float64: 2 rows, then 4
-SIZES_2D = [(3, 3), (31, 9), (32, 33), (64, 64), (5, 303), (5, 305), (617, 5), (95, 62), (4, 2441), (2441, 4)]
+SIZES_2D = [(3, 3), (31, 9), (32, 33), (64, 64), (5, 303), (5, 305), (617, 5), (95, 62), (96, 96), (4, 2441), (2441, 4)]
 
 
 @pytest.mark.parametrize("nx,ny", SIZES_2D)
