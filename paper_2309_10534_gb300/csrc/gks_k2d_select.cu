@@ -21,7 +21,15 @@ GKS_SWEEP(sweep_f64_t2)
 #undef GKS_SWEEP
 
 namespace {
-long long blocks(const SweepArgs& a, int tt) { return (long long)((a.nn + SWEEP_TN - 1) / SWEEP_TN) * ((a.nt + tt - 1) / tt); }
+// A sweep's time by its most loaded SM: the blocks it gets times a block's
+// time when the SM is shared, and what the launch and the first block's chain
+// add (relative units; the measurements stand at each use)
+int sweep_time(const SweepArgs& a, int rows, int per_block, int fixed)
+{
+    const long long blocks = (long long)((a.nn + SWEEP_TN - 1) / SWEEP_TN) * ((a.nt + rows - 1) / rows);
+    const long long sms = std::max(1, a.sms), load = (blocks + sms - 1) / sms;
+    return (int)std::min<long long>(load, 1 << 20) * per_block + fixed;
+}
 }  // namespace
 
 cudaError_t prepare_sweep_f32()
@@ -38,35 +46,28 @@ cudaError_t prepare_sweep_f64()
 }
 
 // float32: 16 rows (512 threads, two face points per thread, two blocks per
-// SM) move the most cells per second, 8 rows (512 threads, one point per
-// thread) take 0.6 of their time per block and half the cells, 4 rows half of
-// that again.  So 16 rows win where the chip is filled many times over and
-// the others where a last wave would be nearly empty or the grid does not
-// fill the chip at all.  One step, ms (16 / 8 / 4 rows): 64^2 0.083 / 0.053 /
-// 0.048, 256^2 0.089 / 0.080 / 0.087, 400^2 0.182 / 0.168 / 0.170, 512^2
-// 0.228 / 0.246 / 0.254, 1024^2 0.750 / 0.833 / 0.893.
+// SM) reconstruct the least halo, 8 rows (512 threads, one point per thread)
+// and 4 rows (256 threads) spread a grid over more SMs.  One step, us (16 / 8
+// / 4 rows), by which the times below are taken: 64^2 72 / 47 / 45, 128^2 73 /
+// 48 / 50, 192^2 72 / 64 / 58, 256^2 73 / 65 / 68, 320^2 103 / 91 / 102, 400^2
+// 145 / 127 / 134, 512^2 182 / 184 / 199, 1024^2 595 / 627 / 695.
 cudaError_t launch_sweep_f32(const GridDev& g, const SweepArgs& a, const HostFlux& hf, const TenoParams& tn,
                              const TenoParams& tt, DevState* ds, cudaStream_t st)
 {
-    const long long sms = std::max(1, a.sms), b16 = blocks(a, 16), b8 = blocks(a, 8);
-    if (blocks(a, 4) <= sms) return sweep_f32_t4(g, a, hf, tn, tt, ds, st);
-    // waves of two blocks per SM, weighted by a block's time
-    const long long w16 = 10 * ((b16 + 2 * sms - 1) / (2 * sms)), w8 = 6 * ((b8 + 2 * sms - 1) / (2 * sms));
-    return w16 <= w8 || a.nt > 65535 * 8 ? sweep_f32_t16(g, a, hf, tn, tt, ds, st) : sweep_f32_t8(g, a, hf, tn, tt, ds, st);
+    const int t16 = sweep_time(a, 16, 385, 320), t8 = sweep_time(a, 8, 208, 240), t4 = sweep_time(a, 4, 117, 260);
+    if (t4 < t8 && t4 < t16) return sweep_f32_t4(g, a, hf, tn, tt, ds, st);
+    return t8 < t16 ? sweep_f32_t8(g, a, hf, tn, tt, ds, st) : sweep_f32_t16(g, a, hf, tn, tt, ds, st);
 }
 
-// float64: 4 rows (128 threads at 210 registers, two blocks per SM, which
-// cover each other's barriers); 2 rows where even those leave SMs idle (a last
-// column of less than 8 cells is a small part of a block's work).  One step,
-// ms (8 rows in one 256-thread block / 4 / 2), when the last tiles of a line
-// were whole: 64^2 0.83 / 0.55 / 0.37, 400^2 3.11 / 2.89 / 3.09, 1024^2 16.8 /
-// 16.5 / 18.0; since they do only their own work (4 / 2): 96^2 0.350 / 0.337,
-// 100^2 0.348 / 0.336, and 64^2 0.209, 400^2 2.53 with the choice made here.
+// float64: 4 rows (128 threads at 210 registers, two face points per thread,
+// two blocks per SM, which cover each other's barriers) or 2 rows (one point
+// per thread) where those even out the SMs' loads.  One step, us (4 / 2 rows),
+// by which the times below are taken: 64^2 353 / 208, 96^2 350 / 338, 128^2
+// 592 / 416, 200^2 997 / 870, 400^2 2532 / 2718, 1024^2 15 670 / 16 918.
 cudaError_t launch_sweep_f64(const GridDev& g, const SweepArgs& a, const HostFlux& hf, const TenoParams& tn,
                              const TenoParams& tt, DevState* ds, cudaStream_t st)
 {
-    const long long full = std::max(1ll, ((long long)a.nn + SWEEP_TN - 8) / SWEEP_TN) * ((a.nt + 1ll) / 2);
-    if (full <= std::max(1, a.sms)) return sweep_f64_t2(g, a, hf, tn, tt, ds, st);
+    if (sweep_time(a, 2, 151, 40) < sweep_time(a, 4, 280, 70)) return sweep_f64_t2(g, a, hf, tn, tt, ds, st);
     return sweep_f64_t4(g, a, hf, tn, tt, ds, st);
 }
 
