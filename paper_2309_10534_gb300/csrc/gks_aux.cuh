@@ -9,12 +9,12 @@ namespace gks {
 
 // ------------------------------------------------------------------ ghosts
 // The ghost layers in memory, for callers that read them there (the adjoint,
-// the selection count); the stage kernels form their own.  One thread per
-// ghost cell (cell_source).
+// the selection count); the stage kernels form their own, and no step writes
+// these, so they are filled whether or not a run is marked as finished.  One
+// thread per ghost cell (cell_source).
 template <typename E>
 __global__ void k_fill_ghosts(const __grid_constant__ GridDev g, E* __restrict__ W, const DevState* ds, double toff)
 {
-    if (ds && ds->done) return;
     const int gx = g.nx + 2 * NG;
     const int nv = g.dim + 2;
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
