@@ -951,7 +951,6 @@ gks_status gks_adjoint_backward(gks_adjoint* A, const double* gWN, double* gW0, 
     const NvtxRange range("gks_adjoint_backward");
     if (!A || !gWN || !gW0) return GKS_EINVAL;
     gks_ctx* c = A->c;
-    c->hs_fresh = false;
     if (!A->have_forward) return rt::fail(c, GKS_EINVAL, "gks_adjoint_backward needs a completed forward pass");
     gks_status s;
     if ((s = reserve(A, A->nsteps))) return s;

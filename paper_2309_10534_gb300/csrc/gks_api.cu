@@ -279,8 +279,8 @@ gks_status enqueue_stage(gks_ctx* c, int stage, int with_commit, cudaStream_t st
 
 __global__ void k_prepare(DevState* ds, int mode, double dt, double t_end, long long max_steps)
 {
-    // mode 0: fixed dt, no t_end; 1: CFL dt towards t_end; 2: reset t, counters
-    // and error word; 3: CFL dt, no t_end
+    // mode 0: fixed dt, no t_end; 1: CFL dt towards t_end, max_steps from here;
+    // 2: reset t, counters and error word; 3: CFL dt, no t_end
     if (threadIdx.x || blockIdx.x) return;
     if (mode == 2) {
         ds->t = 0.0;
@@ -288,9 +288,11 @@ __global__ void k_prepare(DevState* ds, int mode, double dt, double t_end, long 
         ds->fallbacks = 0;
         ds->err = 0;
     }
-    ds->done = 0;
+    ds->steps0 = ds->steps;
+    ds->idle = mode == 1 && !(ds->t < t_end);
+    ds->done = ds->idle;
     ds->sigma = 0;
-    ds->max_steps = max_steps;
+    ds->max_steps = max_steps > 0 ? ds->steps + max_steps : 0;
     if (mode == 0) {
         ds->dt = dt;
         ds->fixed_dt = 1;
@@ -301,14 +303,14 @@ __global__ void k_prepare(DevState* ds, int mode, double dt, double t_end, long 
     }
 }
 
-gks_status enqueue_sigma(gks_ctx* c, cudaStream_t st)
+gks_status enqueue_sigma(gks_ctx* c, cudaStream_t st, bool honour_done)
 {
     const long long ncell = (long long)c->desc.nx * (c->desc.dim == 2 ? c->desc.ny : 1);
     int blocks = (int)((ncell + 255) / 256);
     if (blocks > 4096) blocks = 4096;
     const int pi = prof_begin(c, st, 2);
-    if (c->desc.precision == GKS_FP32_FLUX) k_sigma<float><<<blocks, 256, 0, st>>>(c->g, c->W, c->ds);
-    else k_sigma<double><<<blocks, 256, 0, st>>>(c->g, c->W, c->ds);
+    if (c->desc.precision == GKS_FP32_FLUX) k_sigma<float><<<blocks, 256, 0, st>>>(c->g, c->W, c->ds, honour_done);
+    else k_sigma<double><<<blocks, 256, 0, st>>>(c->g, c->W, c->ds, honour_done);
     CK(cudaGetLastError());
     prof_end(c, st, pi);
     ++c->launches;
@@ -336,7 +338,6 @@ gks_status sync_state(gks_ctx* c)
 {
     CK(cudaMemcpyAsync(c->hs, c->ds, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    c->hs_fresh = true;
     return GKS_OK;
 }
 
@@ -673,20 +674,12 @@ gks_status gks_set_state(gks_ctx* c, const double* W, int on_device)
 {
     if (!c || !W) return GKS_EINVAL;
     c->cfl_dt_ready = false;
-    c->hs_fresh = false;
     gks_status s = copy_interior(c, c->W, W, on_device, true, false, c->Wf);
     if (s) return s;
     k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 2, 0.0, INFINITY, 0);
     CK(cudaGetLastError());
     ++c->launches;
-    if (on_device == GKS_HOST_PINNED_ASYNC) {
-        // the host mirror of t and the counters is refreshed by the next
-        // synchronising call
-        c->hs->t = 0.0;
-        c->hs->steps = 0;
-        return GKS_OK;
-    }
-    return sync_state(c);
+    return on_device == GKS_HOST_PINNED_ASYNC ? GKS_OK : sync_state(c);
 }
 
 gks_status gks_get_state(gks_ctx* c, double* W, int on_device)
@@ -716,7 +709,7 @@ gks_status gks_compute_dt(gks_ctx* c, double* dt)
 {
     if (!c || !dt) return GKS_EINVAL;
     CK(cudaMemsetAsync(&c->ds->sigma, 0, sizeof(unsigned long long), c->stream));
-    gks_status s = enqueue_sigma(c, c->stream);
+    gks_status s = enqueue_sigma(c, c->stream, false);
     if (s) return s;
     if ((s = sync_state(c))) return s;
     if ((s = check_err(c))) return s;
@@ -731,7 +724,7 @@ gks_status gks_stage(gks_ctx* c, int stage, double dt)
 {
     const NvtxRange range("gks_stage");
     if (!c || (stage != 1 && stage != 2) || !(dt > 0.0) || !std::isfinite(dt)) return GKS_EINVAL;
-    c->cfl_dt_ready = c->hs_fresh = false;
+    c->cfl_dt_ready = false;
     k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 0, dt, 0.0, 0);
     CK(cudaGetLastError());
     ++c->launches;
@@ -743,7 +736,6 @@ gks_status gks_step(gks_ctx* c, double dt)
     const NvtxRange range("gks_step");
     if (!c || !std::isfinite(dt)) return GKS_EINVAL;
     gks_status s;
-    c->hs_fresh = false;
     if (dt > 0.0) {
         c->cfl_dt_ready = false;
         k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 0, dt, 0.0, 0);
@@ -753,7 +745,7 @@ gks_status gks_step(gks_ctx* c, double dt)
         k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 3, 0.0, 0.0, 0);
         CK(cudaGetLastError());
         ++c->launches;
-        if ((s = enqueue_sigma(c, c->stream))) return s;
+        if ((s = enqueue_sigma(c, c->stream, true))) return s;
         if ((s = enqueue_first_dt(c, c->stream))) return s;
     }
     // else: the previous CFL step's commit already chose dt from this state
@@ -768,21 +760,17 @@ gks_status gks_advance_to(gks_ctx* c, double t_end, long long max_steps, long lo
     if (!c || !std::isfinite(t_end)) return GKS_EINVAL;
     c->cfl_dt_ready = false;
     gks_status s;
-    if (!c->hs_fresh && (s = sync_state(c))) return s;
-    const long long steps0 = c->hs->steps;
-    if (!(c->hs->t < t_end)) {
-        if (steps_done) *steps_done = 0;
-        if (t_out) *t_out = c->hs->t;
-        return GKS_OK;
-    }
-    c->hs_fresh = false;
-    const long long limit = max_steps > 0 ? steps0 + max_steps : 0;
-    k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 1, 0.0, t_end, limit);
+    // The device decides where the call starts and ends (k_prepare): t and the
+    // step count are only there, since a caller may replay captured steps that
+    // the library does not see.  The host reads them back with the first
+    // replay's completion flag, so the call needs no synchronisation of its own.
+    k_prepare<<<1, 32, 0, c->stream>>>(c->ds, 1, 0.0, t_end, max_steps);
     CK(cudaGetLastError());
     ++c->launches;
-    if ((s = enqueue_sigma(c, c->stream))) return s;
+    if ((s = enqueue_sigma(c, c->stream, true))) return s;
     if ((s = enqueue_first_dt(c, c->stream))) return s;
-    long long left = limit ? limit - steps0 : GRAPH_STEPS;
+    const bool limit = max_steps > 0;
+    long long left = limit ? max_steps : GRAPH_STEPS;
     for (;;) {
         // the last few steps of a limited call one by one: a full replay
         // would launch the steps beyond the limit too, each to return at once
@@ -796,10 +784,11 @@ gks_status gks_advance_to(gks_ctx* c, double t_end, long long max_steps, long lo
         }
         if (limit) left -= GRAPH_STEPS;
         if ((s = sync_state(c))) return s;
+        if (c->hs->idle) break;  // t_end had passed: no step, no check
         if ((s = check_err(c))) return s;
         if (c->hs->done) break;
     }
-    if (steps_done) *steps_done = c->hs->steps - steps0;
+    if (steps_done) *steps_done = c->hs->steps - c->hs->steps0;
     if (t_out) *t_out = c->hs->t;
     return GKS_OK;
 }

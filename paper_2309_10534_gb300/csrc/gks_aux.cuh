@@ -48,9 +48,12 @@ __global__ void k_fill_ghosts(const __grid_constant__ GridDev g, E* __restrict__
     }
 }
 
+// honour_done: nothing where the run is finished (a call that finds its end
+// time passed)
 template <typename T>
-__global__ void __launch_bounds__(256) k_sigma(GridDev g, const double* __restrict__ W, DevState* ds)
+__global__ void __launch_bounds__(256) k_sigma(GridDev g, const double* __restrict__ W, DevState* ds, bool honour_done)
 {
+    if (honour_done && ds->done) return;
     T s = T(0);
     unsigned int err = 0;
     const int nv = g.dim + 2;

@@ -37,7 +37,6 @@ struct gks_ctx {
         unsigned long long version = 0;
     } graph, graph1;
     unsigned long long param_version = 1;
-    bool hs_fresh = false;  // hs holds the device state's time and step count
     long long launches = 0;
     // the device already holds the CFL time step of the current state (set by
     // a CFL step's commit, cleared by anything else that changes W or dt)

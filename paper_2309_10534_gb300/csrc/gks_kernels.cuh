@@ -32,6 +32,8 @@ struct DevState {
     unsigned int done;             // 1: t_end or max_steps reached; kernels return early
     unsigned int fixed_dt;         // 1: keep dt (caller-given), 0: CFL time step
     unsigned int ticket;           // blocks of a committing kernel that have finished
+    long long steps0;              // steps before the present gks_advance_to
+    unsigned int idle;             // 1: that call found t_end already reached
 };
 
 // state-setting boundary rules: conserved states (energy in slot 3) and the

@@ -38,3 +38,39 @@ def test_selection_counts_after_a_finished_run(gks, dim, bc, precision):
     fresh = gks.Solver(dim, n, n if dim == 2 else 1, **kw)
     fresh.set_state(S.get_state())
     assert S.selection_flips() == fresh.selection_flips()
+
+
+# ------------------------------------------------------------ steps the library did not launch itself
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_advance_after_steps_replayed_from_a_callers_graph(gks, precision):
+    """gks_step only launches, so a caller can capture it and replay it.  Time
+    and step count are the device's: advance_to goes on from there, whatever
+    the library last read back."""
+    import torch
+    s = WL.riemann2d(24, split=0.8)
+    S, ref = gks.solver_for(s, precision), gks.solver_for(s, precision)
+    dt = 0.5 * S.compute_dt()
+    S.step(dt)       # every kernel is loaded before the capture
+    S.diagnostics()  # and that step is done before the stream changes
+    st = torch.cuda.Stream()
+    S.set_stream(st.cuda_stream)
+    S.set_state(s.W)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        S.step(dt)
+    assert S.diagnostics().steps == 0
+    with torch.cuda.stream(st):
+        for _ in range(3):
+            g.replay()
+    n, t = S.advance_to(1e9, max_steps=2)
+    for _ in range(3):
+        ref.step(dt)
+    nr, tr = ref.advance_to(1e9, max_steps=2)
+    assert (n, t) == (nr, tr) == (2, t) and S.diagnostics().steps == ref.diagnostics().steps == 5
+    assert np.array_equal(S.get_state(), ref.get_state())
+    with torch.cuda.stream(st):
+        g.replay()
+    st.synchronize()
+    # a time already passed: nothing runs
+    W = S.get_state()
+    assert S.advance_to(0.5 * t) == (0, S.diagnostics().t) and np.array_equal(S.get_state(), W)
