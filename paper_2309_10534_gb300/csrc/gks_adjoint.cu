@@ -952,6 +952,9 @@ gks_status gks_adjoint_backward(gks_adjoint* A, const double* gWN, double* gW0, 
     if (!A || !gWN || !gW0) return GKS_EINVAL;
     gks_ctx* c = A->c;
     if (!A->have_forward) return rt::fail(c, GKS_EINVAL, "gks_adjoint_backward needs a completed forward pass");
+    // W and the device's dt change below, also where a replayed segment runs no
+    // host code that would say so
+    c->cfl_dt_ready = false;
     gks_status s;
     if ((s = reserve(A, A->nsteps))) return s;
     CK(cudaMemsetAsync(A->lam, 0, c->arr_bytes, c->stream));

@@ -74,3 +74,26 @@ def test_advance_after_steps_replayed_from_a_callers_graph(gks, precision):
     # a time already passed: nothing runs
     W = S.get_state()
     assert S.advance_to(0.5 * t) == (0, S.diagnostics().t) and np.array_equal(S.get_state(), W)
+
+
+# ------------------------------------------------------------ the time step after a gradient
+def test_cfl_step_after_a_replayed_gradient(gks):
+    """backward leaves the context at the forward pass's final state; the CFL
+    step after it takes its time step from that state, also when every
+    segment of the pass was a replayed graph."""
+    s = WL.isentropic_vortex(24, seed=None)
+    S = gks.solver_for(s, "fp64", tau="zero")
+    dt = 0.25 * S.compute_dt()
+    A = gks.Adjoint(S, 2)
+    A.forward(4, dt)
+    WN = S.get_state()
+    g = np.ones_like(s.W)
+    A.backward(g)  # captures the segment
+    S.step(0.0)    # leaves the next CFL time step on the device
+    A.backward(g)
+    assert np.array_equal(S.get_state(), WN)
+    S.step(0.0)
+    fresh = gks.solver_for(s, "fp64", tau="zero")
+    fresh.set_state(WN)
+    fresh.step(0.0)
+    assert np.array_equal(S.get_state(), fresh.get_state())
