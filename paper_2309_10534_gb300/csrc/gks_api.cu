@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(256) k_copy_interior(const __grid_constant__ G
     for (long long row = blockIdx.y * 8ll + threadIdx.y; row < rows; row += 8ll * gridDim.y) {
         const int v = (int)(row / ny), j = (int)(row - (long long)v * ny);
         const long long packed = row * g.nx, ghosted = (long long)v * g.plane + (long long)(g0 + j) * g.pitch + NG;
-        for (int i = blockIdx.x * 32 + threadIdx.x; i < g.nx; i += 32 * gridDim.x) {
+        for (unsigned i = blockIdx.x * 32u + threadIdx.x; i < (unsigned)g.nx; i += 32u * gridDim.x) {
             if constexpr (IN) {
                 const double x = src[packed + i];
                 dst[ghosted + i] = x;
@@ -376,7 +376,7 @@ gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device
         if (in) CK(cudaMemcpyAsync(c->stage, W, sizeof(double) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
     }
     const long long rows = (long long)c->nv * ((c->desc.dim == 2) ? c->desc.ny : 1);
-    const dim3 blk(32, 8), grid((unsigned)std::min<long long>((c->desc.nx + 31) / 32, 8192),
+    const dim3 blk(32, 8), grid((unsigned)std::min<long long>((c->desc.nx - 1) / 32 + 1, 8192),
                                 (unsigned)std::min<long long>((rows + 7) / 8, 8192));
     if (in) k_copy_interior<true><<<grid, blk, 0, c->stream>>>(c->g, src, arr, shadow);
     else k_copy_interior<false><<<grid, blk, 0, c->stream>>>(c->g, arr, dst, nullptr);

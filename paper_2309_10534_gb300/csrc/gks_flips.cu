@@ -86,10 +86,10 @@ __device__ void tally(unsigned (&c)[NCOUNT], int k, unsigned code64, unsigned co
 __global__ void k_flips1d(GridDev g, const double* __restrict__ W, TenoT<double> pd, TenoT<float> pf,
                           unsigned long long* out)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // interior cell
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // interior cell
     unsigned cnt[NCOUNT] = {0, 0, 0, 0, 0};
     if (i < g.nx) {
-        const int pl = (int)g.plane;
+        const long long pl = g.plane;
         double q[3][5];
 #pragma unroll
         for (int v = 0; v < 3; ++v)
@@ -232,7 +232,7 @@ extern "C" gks_status gks_selection_flips(gks_ctx* c, gks_flip_count* out)
         if (cudaMemsetAsync(d, 0, sizeof h, c->stream) != cudaSuccess) { st = GKS_ECUDA; break; }
         if ((st = rt::fill_ghosts_f64(c, c->W, c->stream)) != GKS_OK) break;
         if (c->desc.dim == 1) {
-            k_flips1d<<<(c->desc.nx + 255) / 256, 256, 0, c->stream>>>(c->g, c->W, teno_t<double>(tn),
+            k_flips1d<<<(c->desc.nx - 1) / 256 + 1, 256, 0, c->stream>>>(c->g, c->W, teno_t<double>(tn),
                                                                      teno_t<float>(tn), d);
             ++c->launches;
         } else {

@@ -315,11 +315,12 @@ struct Stage1DArgs {
 template <typename T, int TN, typename E>
 __device__ __noinline__ void load_edge_1d(T* sq, const E* src, const GridDev& g, int i0, const DevState* ds, int stage)
 {
-    const int pl = (int)g.plane;
+    const long long pl = g.plane;
     for (int k = threadIdx.x; k < 3 * (TN + 6); k += blockDim.x) {
-        const int v = k / (TN + 6), i = i0 - NG + k % (TN + 6);
+        const int v = k / (TN + 6), c = k % (TN + 6) - NG;
         T val = T(0);
-        if (i < g.nx + NG) {  // beyond: padding
+        if (c < g.nx - i0 + NG) {  // beyond: padding
+            const int i = i0 + c;
             const CellSrc cs = cell_source<false>(g, i, 0, ds, stage == 1 ? 0.0 : 0.5);
             val = cs.state ? (T)state_value(g, cs.state, v) : load_as<T>(src[v * pl + NG + cs.i]);
             if (v == 1 && cs.n1) val = -val;
@@ -373,14 +374,17 @@ __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(cons
     const int tid = threadIdx.x;
     const int slot[3] = {0, 1, 3};
 
-    const int pl = (int)g.plane;  // a 1-D plane is one ghosted row
-    const int ui = i0 + tid, uo = ui + NG;
-    const bool own = tid < TN && ui < g.nx;
+    // a 1-D plane is one ghosted row; three of them pass 2^31 elements from
+    // 7.2e8 cells on, so a variable's offset is a 64-bit one (every comparison
+    // with nx is of differences, which stay in range up to the largest grid)
+    const long long pl = g.plane;
+    const int uo = i0 + tid + NG;
+    const bool own = tid < TN && tid < g.nx - i0;
     // one loop per source type: a per-element choice between the float32
     // and the converted float64 source was compiled as both, and every
     // element then paid a float64 -> float32 conversion on the slow float64
     // pipe whichever source it took
-    const bool edge = i0 < NG || i0 + TN + NG > g.nx;
+    const bool edge = i0 < NG || TN + NG > g.nx - i0;
     auto load = [&](auto src) {
         if (edge) {
             load_edge_1d<T, TN>(&sq[0][0], src, g, i0, ds, a.stage);
@@ -470,7 +474,7 @@ __global__ void __launch_bounds__(TN + 2, sizeof(T) == 4 ? 8 : 4) k1d_stage(cons
     // phase 2: flux at face f (between interior i0+f-1 and i0+f)
     unsigned int nfb = 0, err = 0;
     for (int f = tid; f <= TN; f += NT) {
-        if (i0 + f > g.nx) continue;  // padding past the last face
+        if (f > g.nx - i0) continue;  // padding past the last face
         Side<T> L, R;
 #pragma unroll
         for (int k = 0; k < 4; ++k) { L.W[k] = L.Wn[k] = L.Wt[k] = R.W[k] = R.Wn[k] = R.Wt[k] = T(0); }
@@ -565,7 +569,7 @@ __global__ void __launch_bounds__(96) k1d_stage_wide(const __grid_constant__ Gri
     __shared__ double s_cx;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i0 = blockIdx.x * TN;
-    const int pl = (int)g.plane;
+    const int pl = (int)g.plane;  // a short grid: three rows fit in 32 bits
     constexpr int slot[3] = {0, 1, 3};
     const double dt = ds->dt;
     fp.dt = (T)dt;
