@@ -16,9 +16,9 @@ struct SweepTile {
         constexpr int TN = SWEEP_TN;
         const size_t smem = sizeof(SweepSmem<T, TN, TT, rec_conventional(REC)>);
         const unsigned cols = (a.nn + TN - 1) / TN, rows = (a.nt + TT - 1) / TT;
-        const bool fits = sizeof(T) == 4 || rows <= 65535;  // float32 grids that tall take 16 rows
-        a.cols = fits ? 0 : (int)cols;
-        const dim3 grid(fits ? cols : cols * rows, fits ? rows : 1);
+        // a grid's y extent ends at 65535 (a plane that tall has few columns)
+        a.tall = sweep_tall<T>(TT) && rows > 65535;
+        const dim3 grid(a.tall ? rows : cols, a.tall ? cols : rows);
         k2d_sweep<T, NONEQ, PRFIX, TN, TT, NT, MB, REC><<<grid, NT, smem, st>>>(g, a, fp, teno_t<T>(tn), teno_t<T>(tt), ds);
         return cudaGetLastError();
     }

@@ -54,6 +54,9 @@ cudaError_t prepare_sweep_f64()
 cudaError_t launch_sweep_f32(const GridDev& g, const SweepArgs& a, const HostFlux& hf, const TenoParams& tn,
                              const TenoParams& tt, DevState* ds, cudaStream_t st)
 {
+    // more 16-row tiles than a grid's y extent takes (1 048 560 rows): the
+    // tiles whose rows can lie along x
+    if ((a.nt + 15) / 16 > 65535) return sweep_f32_t4(g, a, hf, tn, tt, ds, st);
     const int t16 = sweep_time(a, 16, 385, 320), t8 = sweep_time(a, 8, 208, 240), t4 = sweep_time(a, 4, 117, 260);
     if (t4 < t8 && t4 < t16) return sweep_f32_t4(g, a, hf, tn, tt, ds, st);
     return t8 < t16 ? sweep_f32_t8(g, a, hf, tn, tt, ds, st) : sweep_f32_t16(g, a, hf, tn, tt, ds, st);

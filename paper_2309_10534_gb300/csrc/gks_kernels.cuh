@@ -797,12 +797,18 @@ struct SweepArgs {
     int with_sigma;
     int commit;          // the last block commits the step
     int sms;             // multiprocessors of the device (tile choice)
-    int cols;            // float64, > 0: more rows of tiles than a grid's y extent takes;
-                         // tiles are numbered along x, cols to a row
+    int tall;            // more rows of tiles than a grid's y extent takes: rows along x (sweep_tall)
 };
 
 // global variable index of local variable v (swap: faces normal to y)
 __device__ __forceinline__ int gvar(int v, bool swap) { return (swap && (v == 1 || v == 2)) ? 3 - v : v; }
+
+// Tiles that can lie with their rows along the grid's x extent: the float64
+// ones and the lowest float32 ones, which the tallest grids take.  The choice
+// costs the taller float32 tiles, which spill, 1.5 % (2048 x 1024 viscous
+// 3209 -> 3257 us for two steps); 64^2 float32 254 us either way.
+template <typename T>
+__host__ __device__ constexpr bool sweep_tall(int rows) { return sizeof(T) == 8 || rows == 4; }
 
 template <typename T> struct alignas(2 * sizeof(T)) Pair2 {
     T v, s;
@@ -880,9 +886,8 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
         s_scal[5] = (T)g.mu;
         s_scal[6] = (T)a.hmin;
     }
-    const int cols = sizeof(T) == 8 ? a.cols : 0;
-    const int n0 = (cols ? blockIdx.x % cols : blockIdx.x) * TN;
-    const int t0 = (cols ? blockIdx.x / cols : blockIdx.y) * TT;
+    const bool tall = sweep_tall<T>(TT) && a.tall;
+    const int n0 = (tall ? blockIdx.y : blockIdx.x) * TN, t0 = (tall ? blockIdx.x : blockIdx.y) * TT;
     static_assert(TN == 31, "lanes of a warp along the tile's faces");
     // local frame: normal momentum first; y faces swap the two momentum components
     const bool swap = a.dirn != 0;
