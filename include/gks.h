@@ -369,6 +369,13 @@ gks_status gks_count_flops_recon(int dim, int precision, int tau_mode, double Pr
  * small output buffer; synchronises the device. */
 gks_status gks_alu_peak(int precision, double target_ms, double *tflops);
 
+/* Start of the half-space moments of Eqs. (2.6), (3.25) as the kernels form it
+ * (their device arithmetic, which the host replica does not share): for n
+ * host values z (float32 path: rounded to float32) half = erfc(-z) / 2 and
+ * gauss = exp(-z^2).  For accuracy checks; allocates and frees 24 n bytes on
+ * the current device and synchronises. */
+gks_status gks_eval_half_space(int precision, const double *z, int n, double *half, double *gauss);
+
 /* ---- allocation-free 1-D step (the paper has no counterpart) ---- */
 
 /* Largest grid gks_step1d_noalloc accepts. */

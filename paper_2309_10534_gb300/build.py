@@ -44,7 +44,7 @@ FAST_F32 = ["-ftz=true", "-prec-div=false", "-prec-sqrt=false"]
 # (the adjoint recomputes the forward pass's float32 selections and
 # reconstructions, so it takes the same flags as the forward kernels)
 EXTRA = {"gks_k2d_f32_t16": FAST_F32, "gks_k2d_f32_t8": FAST_F32, "gks_k2d_f32_t4": FAST_F32, "gks_k1d": FAST_F32, "gks_ensemble": FAST_F32, "gks_adjoint": FAST_F32,
-         "gks_flips": FAST_F32}
+         "gks_flips": FAST_F32, "gks_probe": FAST_F32}
 
 
 def _compile(unit):

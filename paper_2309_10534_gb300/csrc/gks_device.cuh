@@ -973,7 +973,12 @@ GKS_HD void mom(T* o, T r, T uk, T uk1, T uk2, T V, T e)
 // Start of the half-space moments: h0 = 1/2 erfc(-sg z) (the mass fraction
 // on the side sg of u = 0, z = sqrt(lambda) U) and g = exp(-z^2).
 // float64: erfc(|z|) = erfcx(|z|) g, so one exponential serves both (erfc
-// itself holds a second one).  float32: erfc by Abramowitz & Stegun 7.1.26
+// itself holds a second one).  The rounding of z^2 alone would put a relative
+// error of z^2 2^-53 into g and the vanishing half (514 units of 2^-53 at |z| =
+// 20 .. 26, 66 at 4 .. 10, where erfc itself is within 4.1); g (1 - lo), lo
+// what z^2 lost, takes it out (2.0 and 4.1 at any |z|; z^2 is at most ~1e17
+// in a state whose p is resolved) for two operations of the point's ~520.
+// float32: erfc by Abramowitz & Stegun 7.1.26
 // (Hastings' rational approximation, |error| <= 1.5e-7 on x >= 0), which
 // reuses g the same way.
 template <typename T>
@@ -985,11 +990,14 @@ GKS_HD void half_space_start(T z, T sg, T& h0, T& g)
 template <>
 GKS_HD void half_space_start<double>(double z, double sg, double& h0, double& g)
 {
-    g = exp(-z * z);
 #ifdef __CUDA_ARCH__
+    const double zz = z * z;
+    g = exp(-zz);
+    g = fma(-fma(z, z, -zz), g, g);
     const double h = 0.5 * (g * erfcx(fabs(z)));
     h0 = ((hi_word(z) < 0) == (sg < 0.0)) ? 1.0 - h : h;
 #else
+    g = exp(-z * z);
     h0 = 0.5 * erfc(-sg * z);
 #endif
 }

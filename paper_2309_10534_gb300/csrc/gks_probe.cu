@@ -1,8 +1,10 @@
-// gks_probe.cu -- FMA-chain throughput probe: the measured float32 / float64
-// arithmetic peak that the sweep kernels are compared against.
+// gks_probe.cu -- probes of the device: the FMA-chain throughput that the sweep
+// kernels are compared against, and device arithmetic that differs from its
+// host replica.  Compiled with the float32 kernels' arithmetic flags.
 #include <cuda_runtime.h>
 
 #include "../../include/gks.h"
+#include "gks_device.cuh"
 
 namespace {
 
@@ -60,7 +62,40 @@ gks_status probe(double target_ms, double* tflops)
     return st;
 }
 
+template <typename T>
+__global__ void k_half_space(const double* z, int n, double* half, double* gauss)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    T h, g;
+    gks::half_space_start<T>((T)z[i], T(1), h, g);
+    half[i] = (double)h;
+    gauss[i] = (double)g;
+}
+
 }  // namespace
+
+extern "C" gks_status gks_eval_half_space(int precision, const double* z, int n, double* half, double* gauss)
+{
+    if (!z || !half || !gauss || n < 1) return GKS_EINVAL;
+    const size_t bytes = sizeof(double) * (size_t)n;
+    double* d = nullptr;  // z, then both results
+    if (cudaMalloc(&d, 3 * bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return GKS_ENOMEM;
+    }
+    cudaError_t e = cudaMemcpy(d, z, bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        const int blocks = (n - 1) / 256 + 1;
+        if (precision == GKS_FP32_FLUX) k_half_space<float><<<blocks, 256>>>(d, n, d + n, d + 2 * (size_t)n);
+        else k_half_space<double><<<blocks, 256>>>(d, n, d + n, d + 2 * (size_t)n);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(half, d + n, bytes, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(gauss, d + 2 * (size_t)n, bytes, cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return e == cudaSuccess ? GKS_OK : GKS_ECUDA;
+}
 
 extern "C" gks_status gks_alu_peak(int precision, double target_ms, double* tflops)
 {

@@ -331,6 +331,19 @@ def alu_peak(precision="fp32", target_ms=200.0):
     return v.value
 
 
+def eval_half_space(z, precision="fp64"):
+    """(erfc(-z)/2, exp(-z^2)) of a float64 array by the kernels' device
+    arithmetic (gks_eval_half_space)."""
+    z = np.ascontiguousarray(z, dtype=np.float64)
+    h, g = np.empty(z.shape), np.empty(z.shape)
+    f = lib().gks_eval_half_space
+    f.argtypes, f.restype = [C.c_int, _vp, C.c_int, _vp, _vp], C.c_int
+    st = f(PRECISION[precision], z.ctypes.data_as(_vp), z.size, h.ctypes.data_as(_vp), g.ctypes.data_as(_vp))
+    if st != GKS_OK:
+        raise GKSError(st, "gks_eval_half_space")
+    return h, g
+
+
 GKS_COUNT_TENO_CHARVARS = 4
 
 
