@@ -29,22 +29,25 @@ namespace {
 constexpr int GRAPH_STEPS = 8;
 
 // interior [nv][ny][nx] <-> ghosted layout (1-D: ny = 1, no ghost rows).
-// Blocks of 32 x 8 threads walk over (x, row) with row = v ny + j: two
-// divisions per row, none per element.  shadow (may be null): the float32
-// path's copy, written in the same pass.  Set and get of 2^22 float32 cells:
-// 35 + 13 (the copy in a pass of its own) + 35 us -> one pass each
-// (four steps of that tube and its copies 1557 -> 1525 us, two of a 1024^2
-// plane 1332 -> 1316 us).
+// Blocks of 256 threads walk over (x, row) with row = v ny + j: 32 along x,
+// fewer (a power of two from 4 on) where a row is shorter, all 256 in 1-D,
+// which has three rows.  A whole warp for every row left 29 of 32 lanes idle on
+// a 3 x 200000 float64 plane: get 80.6 -> 28.5 us, set 79.5 -> 34.6; eight rows
+// a block left five of them empty in 1-D: get of 2^22 cells 56 -> 51 us, float32
+// set 75 -> 64.  shadow (may be null): the float32 path's copy, written in the
+// same pass rather than in one of its own (set of a 1024^2 float32 plane 53 ->
+// 38 us).
 template <bool IN>
 __global__ void __launch_bounds__(256) k_copy_interior(const __grid_constant__ GridDev g, const double* __restrict__ src,
                                                        double* __restrict__ dst, float* __restrict__ shadow)
 {
     const int ny = (g.dim == 2) ? g.ny : 1, g0 = (g.dim == 2) ? NG : 0;
     const long long rows = (long long)(g.dim + 2) * ny;
-    for (long long row = blockIdx.y * 8ll + threadIdx.y; row < rows; row += 8ll * gridDim.y) {
+    for (long long row = (long long)blockIdx.y * blockDim.y + threadIdx.y; row < rows;
+         row += (long long)blockDim.y * gridDim.y) {
         const int v = (int)(row / ny), j = (int)(row - (long long)v * ny);
         const long long packed = row * g.nx, ghosted = (long long)v * g.plane + (long long)(g0 + j) * g.pitch + NG;
-        for (unsigned i = blockIdx.x * 32u + threadIdx.x; i < (unsigned)g.nx; i += 32u * gridDim.x) {
+        for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (unsigned)g.nx; i += blockDim.x * gridDim.x) {
             if constexpr (IN) {
                 const double x = src[packed + i];
                 dst[ghosted + i] = x;
@@ -376,8 +379,10 @@ gks_status copy_interior(gks_ctx* c, double* arr, const double* W, int on_device
         if (in) CK(cudaMemcpyAsync(c->stage, W, sizeof(double) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
     }
     const long long rows = (long long)c->nv * ((c->desc.dim == 2) ? c->desc.ny : 1);
-    const dim3 blk(32, 8), grid((unsigned)std::min<long long>((c->desc.nx - 1) / 32 + 1, 8192),
-                                (unsigned)std::min<long long>((rows + 7) / 8, 8192));
+    unsigned bx = c->desc.dim == 1 ? 256 : 4;
+    while (bx < 32 && bx < (unsigned)c->desc.nx) bx *= 2;
+    const dim3 blk(bx, 256 / bx), grid((unsigned)std::min<long long>((c->desc.nx - 1) / (int)bx + 1, 8192),
+                                       (unsigned)std::min<long long>((rows - 1) / (int)blk.y + 1, 8192));
     if (in) k_copy_interior<true><<<grid, blk, 0, c->stream>>>(c->g, src, arr, shadow);
     else k_copy_interior<false><<<grid, blk, 0, c->stream>>>(c->g, arr, dst, nullptr);
     CK(cudaGetLastError());
