@@ -14,7 +14,7 @@ struct SweepTile {
                            const TenoParams& tt, DevState* ds, cudaStream_t st)
     {
         constexpr int TN = SWEEP_TN;
-        const size_t smem = sizeof(SweepSmem<T, TN, TT, rec_conventional(REC)>);
+        const size_t smem = sizeof(SweepShared<T, TN, TT, MB, rec_conventional(REC)>);
         const unsigned cols = (a.nn + TN - 1) / TN, rows = (a.nt + TT - 1) / TT;
         // a grid's y extent ends at 65535 (a plane that tall has few columns)
         a.tall = sweep_tall<T>(TT) && rows > 65535;
@@ -48,7 +48,7 @@ struct SweepTile {
     {
         return cudaFuncSetAttribute(k2d_sweep<T, NONEQ, PRFIX, SWEEP_TN, TT, NT, MB, REC>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sizeof(SweepSmem<T, SWEEP_TN, TT, rec_conventional(REC)>));
+                                    (int)sizeof(SweepShared<T, SWEEP_TN, TT, MB, rec_conventional(REC)>));
     }
     template <int REC>
     static cudaError_t smem_rec()

@@ -814,17 +814,32 @@ template <typename T> struct alignas(2 * sizeof(T)) Pair2 {
     T v, s;
 };
 
-template <typename T, int TN, int TT, bool CONV = false> struct SweepSmem {
+template <typename T, int TN, int TT, bool CONV, bool STAGED> struct SweepSmem {
     T w[4][TT + 4][TN + 6];           // cells: tangential rows t0-2.., normal n0-3..
     Pair2<T> rec[2][4][TT + 4][TN + 1];  // [side][var][row][face]: value and normal slope
     T flux[8 * (TN + 1) * (TT + 1)];  // face fluxes for the update (layout: sfi)
     // y sweep: the update's inputs, copied while the sweep computes
-    double base[4][TN * TT];             // W or A (float32 stage 1: its float32 shadow, in the first half)
-    T inc[2][4][TN * TT];                // the x sweep's increments
+    double base[STAGED ? 4 : 1][STAGED ? TN * TT : 1];  // W or A (float32 stage 1: its float32 shadow, in the first half)
+    T inc[2][STAGED ? 4 : 1][STAGED ? TN * TT : 1];     // the x sweep's increments
     // conventional path: line-averaged equilibrium state and its normal
     // slope per face and row (Step 2)
     T w0[CONV ? 2 : 1][4][CONV ? TT + 4 : 1][CONV ? TN + 1 : 1];
 };
+
+// MB blocks of a kernel with this struct fit an SM's 228 KB (1 KB of a block is
+// the system's, half a KB its static arrays)
+template <typename Smem>
+__host__ __device__ constexpr bool sweep_resident(int MB) { return MB * (sizeof(Smem) + 1536) <= 228 * 1024; }
+
+// The update's inputs go through shared memory where the tile keeps the MB
+// resident blocks its register budget is for: 16 rows of the conventional path
+// do not (122 KB a block, 91 without; one step of a float32 plane with one
+// resident block and with two: 768^2 TENO5 546 -> 459 us, WENO5-Z 467 -> 397,
+// 1024^2 965 -> 816 and 818 -> 697).
+template <typename T, int TN, int TT, int MB, bool CONV>
+__host__ __device__ constexpr bool sweep_staged() { return sweep_resident<SweepSmem<T, TN, TT, CONV, true>>(MB); }
+template <typename T, int TN, int TT, int MB, bool CONV>
+using SweepShared = SweepSmem<T, TN, TT, CONV, sweep_staged<T, TN, TT, MB, CONV>()>;
 
 // the cells of a tile that reaches past the boundary, ghosts by the boundary
 // rules (out of line: the other tiles keep their registers)
@@ -862,7 +877,10 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     constexpr bool CONV = rec_conventional(REC);
     constexpr int RB = rec_base(REC);  // the tangential (per-quantity) reconstruction
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    SweepSmem<T, TN, TT, CONV>& sm = *reinterpret_cast<SweepSmem<T, TN, TT, CONV>*>(smem_raw);
+    constexpr bool STAGED = sweep_staged<T, TN, TT, MB, CONV>();
+    using Shared = SweepShared<T, TN, TT, MB, CONV>;
+    static_assert(sweep_resident<Shared>(MB), "the MB blocks of the launch bounds fit an SM's shared memory");
+    Shared& sm = *reinterpret_cast<Shared*>(smem_raw);
     // face fluxes for the update: [k][row][face] for x faces; [k][face][row]
     // (rows padded) for y faces, so that phase 3 runs along the unit-stride x
     // direction in both sweeps
@@ -923,7 +941,7 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     // cost its warps a memory round trip: four steps of a 64^2 float32 plane
     // 292 -> 281 us, two of a 1024^2 plane the same)
     const bool base_f = sizeof(T) == 4 && a.stage == 1;
-    if (a.pass == 1) {
+    if (STAGED && a.pass == 1) {
         for (int k = tid; k < TN * TT; k += NT) {
             const int r = fy ? k % TT : k / TN, c = fy ? k / TT : k % TN;
             const int in = n0 + c, it = t0 + r;
@@ -1194,6 +1212,18 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
     copy_wait<0>();
     T sig = T(0);
     const T cn = s_scal[1];
+    auto base64 = [&](int v, int k, long long go) {
+        if constexpr (STAGED) return sm.base[v][k];
+        else return a.base[go];
+    };
+    auto basef = [&](int v, int k, long long go) {
+        if constexpr (STAGED) return reinterpret_cast<const float*>(sm.base[v])[k];
+        else return a.basef[go];
+    };
+    auto inc = [&](int q, int v, int k, long long go) {
+        if constexpr (STAGED) return sm.inc[q][v][k];
+        else return static_cast<const T*>(q ? a.inc1 : a.inc0)[go];
+    };
 #pragma unroll 1
     for (int k = tid; k < TN * TT; k += NT) {
         // x faces: the normal (x) index fastest; y faces: the tangential (x) index
@@ -1217,20 +1247,20 @@ k2d_sweep(const __grid_constant__ GridDev g, const __grid_constant__ SweepArgs a
                     if (a.stage == 1) inc1[go] = d1;
                 } else if constexpr (sizeof(T) == 4) {
                     if (a.stage == 1) {
-                        a.out0f[go] = reinterpret_cast<const float*>(sm.base[v])[k] - (sm.inc[0][v][k] + d0);
-                        inc1[go] = sm.inc[1][v][k] + d1;
+                        a.out0f[go] = basef(v, k, go) - (inc(0, v, k, go) + d0);
+                        inc1[go] = inc(1, v, k, go) + d1;
                     } else {
-                        const double res = sm.base[v][k] - widen(sm.inc[1][v][k] + sm.inc[0][v][k] + d0);
+                        const double res = base64(v, k, go) - widen(inc(1, v, k, go) + inc(0, v, k, go) + d0);
                         a.out0[go] = res;
                         wf[v] = narrow(res);  // local order; the CFL rate only needs |U|
                         a.out0f[go] = wf[v];
                     }
                 } else if (a.stage == 1) {
-                    const double w = sm.base[v][k];
-                    a.out0[go] = w - (double)(sm.inc[0][v][k] + d0);
-                    a.out1[go] = w - (double)(sm.inc[1][v][k] + d1);
+                    const double w = base64(v, k, go);
+                    a.out0[go] = w - (double)(inc(0, v, k, go) + d0);
+                    a.out1[go] = w - (double)(inc(1, v, k, go) + d1);
                 } else {
-                    const double res = sm.base[v][k] - (double)(sm.inc[0][v][k] + d0);
+                    const double res = base64(v, k, go) - (double)(inc(0, v, k, go) + d0);
                     a.out0[go] = res;
                     wn[v] = res;  // local order; the CFL rate only needs |U|
                 }
