@@ -114,10 +114,6 @@ HostFlux host_flux(const gks_ctx* c)
 }  // namespace gks
 using gks::rt::host_flux;
 
-namespace {
-
-}  // namespace
-
 namespace gks {
 namespace rt {
 
@@ -194,9 +190,9 @@ gks_status fill_ghosts(gks_ctx* c, void* arr, cudaStream_t st)
     const int n = (c->desc.dim == 1) ? 2 * NG : 2 * NG * gx + 2 * NG * c->desc.ny;
     const int pi = prof_begin(c, st, 1);
     if (c->desc.precision == GKS_FP32_FLUX)
-        k_fill_ghosts<float><<<(n + 127) / 128, 128, 0, st>>>(c->g, static_cast<float*>(arr), nullptr, 0.0);
+        k_fill_ghosts<float><<<(n + 127) / 128, 128, 0, st>>>(c->g, static_cast<float*>(arr), nullptr);
     else
-        k_fill_ghosts<double><<<(n + 127) / 128, 128, 0, st>>>(c->g, static_cast<double*>(arr), nullptr, 0.0);
+        k_fill_ghosts<double><<<(n + 127) / 128, 128, 0, st>>>(c->g, static_cast<double*>(arr), nullptr);
     CK(cudaGetLastError());
     prof_end(c, st, pi);
     ++c->launches;
@@ -207,7 +203,7 @@ gks_status fill_ghosts_f64(gks_ctx* c, double* arr, cudaStream_t st)
 {
     const int gx = c->desc.nx + 2 * NG;
     const int n = (c->desc.dim == 1) ? 2 * NG : 2 * NG * gx + 2 * NG * c->desc.ny;
-    k_fill_ghosts<double><<<(n + 127) / 128, 128, 0, st>>>(c->g, arr, c->ds, 0.0);
+    k_fill_ghosts<double><<<(n + 127) / 128, 128, 0, st>>>(c->g, arr, c->ds);
     CK(cudaGetLastError());
     ++c->launches;
     return GKS_OK;

@@ -13,7 +13,7 @@ namespace gks {
 // these, so they are filled whether or not a run is marked as finished.  One
 // thread per ghost cell (cell_source).
 template <typename E>
-__global__ void k_fill_ghosts(const __grid_constant__ GridDev g, E* __restrict__ W, const DevState* ds, double toff)
+__global__ void k_fill_ghosts(const __grid_constant__ GridDev g, E* __restrict__ W, const DevState* ds)
 {
     const int gx = g.nx + 2 * NG;
     const int nv = g.dim + 2;
@@ -38,8 +38,8 @@ __global__ void k_fill_ghosts(const __grid_constant__ GridDev g, E* __restrict__
         }
     }
     const int r0 = g.dim == 2 ? NG : 0;  // ghost rows below the interior
-    const CellSrc s = g.dim == 2 ? cell_source<true>(g, i - NG, j - NG, ds, toff)
-                                 : cell_source<false>(g, i - NG, 0, ds, toff);
+    const CellSrc s = g.dim == 2 ? cell_source<true>(g, i - NG, j - NG, ds, 0.0)
+                                 : cell_source<false>(g, i - NG, 0, ds, 0.0);
     for (int v = 0; v < nv; ++v) {
         E val = s.state ? (E)state_value(g, s.state, v)
                         : W[(long long)v * g.plane + (long long)(s.j + r0) * g.pitch + s.i + NG];

@@ -28,7 +28,6 @@ template <> struct M<float> {
     static GKS_HD float erfc_(float x) { return erfcf(x); }
     static GKS_HD float exp_(float x) { return expf(x); }
     static GKS_HD float sqrt_(float x) { return sqrtf(x); }
-    static GKS_HD float rcp(float x) { return 1.0f / x; }
 #ifdef __CUDA_ARCH__
     static GKS_HD float rsqrt_(float x) { return rsqrtf(x); }
 #else
@@ -43,7 +42,6 @@ template <> struct M<double> {
     static GKS_HD double erfc_(double x) { return erfc(x); }
     static GKS_HD double exp_(double x) { return exp(x); }
     static GKS_HD double sqrt_(double x) { return sqrt(x); }
-    static GKS_HD double rcp(double x) { return 1.0 / x; }
 #ifdef __CUDA_ARCH__
     static GKS_HD double rsqrt_(double x) { return rsqrt(x); }
 #else
@@ -1151,13 +1149,11 @@ GKS_HD void time_coeffs(T s, T is, T* cF, T* cD)  // is = 1 / s
 template <typename T> struct FluxParams {
     T gm1;        // gamma - 1
     T K;          // internal degrees of freedom of this dimension
-    T ntot;       // K + DIM
-    T inv_ntot;   // 1 / ntot
     T dt;
     T c1, c2, mu; // collision time (Sec. 5)
     T prfac;      // 1/Pr - 1
     T hkv;        // (K + DIM - 1) / 2
-    T cp;         // gamma / (gamma - 1) = (ntot + 2) / 2
+    T cp;         // gamma / (gamma - 1) = (K + DIM + 2) / 2
     int tau_mode; // 0 zero, 1 Euler, 2 NS
     int merge = 0; // 0 kinetic weighting (Eqs. 3.25, 3.26), 1 arithmetic average of the sides
 };

@@ -75,8 +75,6 @@ int flux_t(int tau_mode, double gamma, double mu, double Pr, double c1, double c
     gks::FluxParams<T> p;
     p.gm1 = (T)(gamma - 1.0);
     p.K = (T)K;
-    p.ntot = (T)(K + DIM);
-    p.inv_ntot = (T)(1.0 / (K + DIM));
     p.dt = (T)dt;
     p.c1 = (T)c1;
     p.c2 = (T)c2;
@@ -133,8 +131,6 @@ int flux_vjp_t(double gamma, const double* Wl, const double* Wln, const double* 
     gks::FluxParams<T> p{};
     p.gm1 = (T)(gamma - 1.0);
     p.K = (T)K;
-    p.ntot = (T)(K + 2.0);
-    p.inv_ntot = (T)(1.0 / (K + 2.0));
     p.hkv = (T)(0.5 * (K + 1.0));
     p.cp = (T)(0.5 * (K + 4.0));
     p.tau_mode = 0;

@@ -59,7 +59,6 @@ template <typename B> struct M<opc::Cnt<B>> {
     static C exp_(C x) { opc::g_cnt.exp += 1; return C(std::exp((double)x.v)); }
     static C sqrt_(C x) { opc::g_cnt.sqrt += 1; return C(std::sqrt((double)x.v)); }
     static C rsqrt_(C x) { opc::g_cnt.sqrt += 1; opc::g_cnt.div += 1; return C(1.0 / std::sqrt((double)x.v)); }
-    static C rcp(C x) { opc::g_cnt.div += 1; return C(1.0 / (double)x.v); }
     static constexpr double tiny = M<B>::tiny;
     static constexpr int nseries = M<B>::nseries;
     static constexpr double s_series = M<B>::s_series;
@@ -100,8 +99,6 @@ void count(int tau_mode, double Pr, gks_flop_model* out)
     FluxParams<T> fp;
     fp.gm1 = T(gamma - 1.0);
     fp.K = T(K);
-    fp.ntot = T(K + DIM);
-    fp.inv_ntot = T(1.0 / (K + DIM));
     fp.dt = T(1e-3);
     fp.c1 = T(0.01);
     fp.c2 = T(1.0);
