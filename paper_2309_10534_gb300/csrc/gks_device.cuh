@@ -1005,10 +1005,7 @@ GKS_HD void half_space_start<float>(float z, float sg, float& h0, float& g)
     const float x = fabsf(z);
 #ifdef __CUDA_ARCH__
     g = __expf(-x * x);
-    // the approximate reciprocal and one Newton step: rounded to nearest (the
-    // half's absolute error 4.0 units of 2^-24; 5.2 without the step)
-    const float d = fmaf(0.3275911f, x, 1.0f), t0 = __fdividef(1.0f, d);
-    const float t = fmaf(t0, fmaf(-t0, d, 1.0f), t0);
+    const float t = __fdividef(1.0f, fmaf(0.3275911f, x, 1.0f));
 #else
     g = expf(-x * x);
     const float t = 1.0f / (1.0f + 0.3275911f * x);
