@@ -308,8 +308,8 @@ long long  gks_batch_launches(const gks_batch *b);
  * checkpoint_every = k >= 1: the forward pass keeps W every k steps; the
  * backward pass recomputes one k-step segment at a time, keeping W and W* of
  * each of its steps (device memory: ceil(nsteps/k) + 2k + 6 state-sized
- * arrays plus scratch of about 40 x nx x ny values of the working
- * precision). */
+ * arrays plus scratch of about 40 (float32) or 48 (float64) x nx x ny values
+ * of the working precision). */
 typedef struct gks_adjoint gks_adjoint;
 gks_status gks_adjoint_create(gks_ctx *ctx, int checkpoint_every, gks_adjoint **out);
 void       gks_adjoint_destroy(gks_adjoint *adj);
